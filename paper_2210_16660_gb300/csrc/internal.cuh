@@ -195,6 +195,7 @@ struct Level {
 // that an iteration needs no host round trip.
 struct Ctl {
     double bnorm;        // ||b||
+    double stop2;        // (rtol ||b||)^2: the recursive residual's stop test, on ||r||^2
     double rho, rho_old; // r.z
     double pq, pq_old;   // p.Ap
     double zq;           // z . q_old (FCG)
@@ -207,11 +208,12 @@ struct Ctl {
     int mode;
     int flex;            // FCG(1) beta in either mode (iterative coarsest solve)
     int restart;         // next direction is p = z
-    int check;           // recursive residual met rtol: form the true one
+    int halt;            // whether the iteration's kernels run: 0 they do, 1 the recursive residual met
+                         // rtol and the true one is formed next, 2 the solve has ended
     int done;            // 1 converged, 2 error
     int status;          // AMG_* code once done
-    int bodies;          // executions of the graph's loop body (2 iterations each)
-    unsigned int counter[8];  // last-block-done counters of the reducing kernels
+    int bodies;          // executions of the graph's loop body
+    unsigned int counter;     // last-block-done counter of the true residual
 };
 
 // Iterative coarsest solve (flexible CG + block-Jacobi with ILU(1) blocks of
@@ -313,7 +315,8 @@ struct amg_hier {
     pcgamg::Ctl *ctl = nullptr;
     pcgamg::Ctl *ctl_host = nullptr;  // pinned mirror
     int nblk = 0;                // largest level-0 grid (sizes the partial sums)
-    int grid32 = 0, grid64 = 0, gridv = 0;  // one wave of the float32 sweeps, float64 sweeps, vector kernels
+    int grid32 = 0, grid64 = 0, gridp = 0;  // one wave of the float32 sweeps, float64 sweeps, prolongation
+    int gridv = 0, blockv = 0;              // vector kernels
     int wave[2][2][2] = {};      // blocks in one wave: [float, double][down, post][4- or 16-entry chunks]
     double last_true_rel = 0.0;
     double setup_ms[4] = {0, 0, 0, 0};

@@ -23,10 +23,13 @@
 // Krylov (float64): p = z + beta p; q = A p, p.q; x += alpha p,
 // r -= alpha q, ||r||^2 (+ r32 or xpre_0); true residual when rtol is met.
 //
-// Reductions are two-stage and deterministic: each block writes a partial,
-// the last block to finish (atomic ticket) sums the partials in index order
-// and updates the iteration's scalars in device memory (struct Ctl), so an
-// iteration needs no host round trip.
+// Reductions are two-stage and deterministic: each block of the producing
+// kernel writes a partial, and every block of the kernel that needs the sum
+// adds all partials before its own work (one block also records the scalars
+// in struct Ctl). So a reduction costs its consumer one L2 round trip and a
+// block sum, and the producer no fence, ticket or serial last block. Sums over
+// threads run on the integer pipe (reduce.cuh), and one thread per block forms
+// the scalars: a float64 quotient or root costs a warp 560 to 600 clocks.
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -35,45 +38,26 @@
 #include <type_traits>
 
 #include "internal.cuh"
+#include "reduce.cuh"
 #include "sell_row.cuh"
 
 namespace pcgamg {
 
 namespace {
 
+constexpr int kVecBlock = 1024;  // largest block of the vector kernels (k_axpy_p, k_update)
+
 template <typename T>
 __device__ __forceinline__ T ldg(const T *p) { return __ldg(p); }
 
-// Block-wide sum of two doubles (blockDim.x == kBlock); result in warp 0.
-__device__ __forceinline__ void block_sum2(double &a, double &b) {
-    __shared__ double sa[kBlock / 32], sb[kBlock / 32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_down_sync(0xffffffffu, a, o);
-        b += __shfl_down_sync(0xffffffffu, b, o);
-    }
-    int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) { sa[w] = a; sb[w] = b; }
-    __syncthreads();
-    if (w == 0) {
-        a = lane < kBlock / 32 ? sa[lane] : 0.0;
-        b = lane < kBlock / 32 ? sb[lane] : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            a += __shfl_down_sync(0xffffffffu, a, o);
-            b += __shfl_down_sync(0xffffffffu, b, o);
-        }
-    }
-}
-
-// Writes this block's partials; returns true in every thread of the last
-// block to finish, after which partials[0..gridDim) are complete.
-__device__ __forceinline__ bool publish_partials(double a, double b, double *partials, unsigned *counter) {
+// As write_partials, and true in every thread of the last block to finish,
+// after which all partials are complete: for the true residual, whose outcome
+// decides whether the loop goes on.
+template <int NV>
+__device__ __forceinline__ bool publish_partials(double (&a)[NV], double *partials, unsigned *counter) {
     __shared__ bool last;
-    block_sum2(a, b);
+    write_partials<NV>(a, partials);
     if (threadIdx.x == 0) {
-        partials[blockIdx.x] = a;
-        partials[gridDim.x + blockIdx.x] = b;
         __threadfence();
         unsigned t = atomicAdd(counter, 1u);
         last = (t == gridDim.x - 1);
@@ -82,37 +66,49 @@ __device__ __forceinline__ bool publish_partials(double a, double b, double *par
     return last;
 }
 
-// Sum of the partials in a fixed order (run by the whole last block).
-__device__ __forceinline__ void final_sum2(const double *partials, double &a, double &b) {
-    __threadfence();
-    a = 0.0;
-    b = 0.0;
-    int nb = gridDim.x;
-    for (int k = threadIdx.x; k < nb; k += blockDim.x) {
-        a += __ldcg(partials + k);
-        b += __ldcg(partials + nb + k);
-    }
-    block_sum2(a, b);
+// Ctl::halt: whether the iteration's kernels run
+constexpr int kRun = 0, kCheck = 1, kEnded = 2;
+
+__device__ __forceinline__ void finish(Ctl *c) {
+    c->done = 1;
+    c->halt = kEnded;
+    c->status = AMG_OK;
 }
 
 __device__ __forceinline__ void fail(Ctl *c, int status) {
     c->done = 2;
+    c->halt = kEnded;
     c->status = status;
 }
 
-// rho = r.z and beta of the next direction (last block of the kernel that
-// produced z): PCG beta = rho / rho_old, FCG(1) beta = -(z.q_old) / (p.q)_old
-// (the float32 V-cycle, and either precision when the iterative coarsest
-// solve makes the V-cycle vary from one application to the next).
-__device__ __forceinline__ void finish_rho(Ctl *ctl, double rz, double zq) {
-    ctl->counter[0] = 0;
-    if (!isfinite(rz) || !isfinite(zq)) { fail(ctl, AMG_ERR_NAN); return; }
-    if (!(rz > 0.0)) { fail(ctl, AMG_ERR_BREAKDOWN); return; }
-    ctl->rho = rz;
-    ctl->zq = zq;
-    double beta = 0.0;
-    if (!ctl->restart) beta = ctl->mode == AMG_MODE_FCG32 || ctl->flex ? -zq / ctl->pq_old : rz / ctl->rho_old;
-    ctl->beta = beta;
+// Outcome of the iteration whose update left g partial sums of ||r||^2:
+// kRun, or why the kernels that follow must not run (kCheck: rtol met, the
+// true residual is formed next; kEnded). Called by every thread of every block
+// of one kernel; one thread records the outcome in ctl->halt (one word, so a
+// block that reads it already takes the same way as on its own).
+__device__ __forceinline__ int step_outcome(const double *pc, int g, Ctl *ctl, double *hist) {
+    __shared__ int out;
+    __shared__ double srr;
+    const double stop2 = ctl->stop2;
+    const int it = ctl->iter, maxit = ctl->maxit;
+    double rr[1];
+    sum_partials<1>(pc, g, rr);
+    if (threadIdx.x == 0) {
+        const int o = !isfinite(rr[0]) ? kEnded : rr[0] <= stop2 ? kCheck : it >= maxit ? kEnded : kRun;
+        out = o;
+        if (blockIdx.x == 0) {
+            if (o == kCheck) ctl->halt = kCheck;
+            else if (o == kEnded) fail(ctl, isfinite(rr[0]) ? AMG_ERR_NOCONV : AMG_ERR_NAN);
+            srr = rr[0];
+        }
+    }
+    __syncthreads();
+    if (blockIdx.x == 0 && threadIdx.x == 32) {  // off the block's way: nothing waits for it
+        const double rel = sqrt(srr) / ctl->bnorm;
+        ctl->rel = rel;
+        hist[it] = rel;
+    }
+    return out;
 }
 
 #define SELL_ROW_BEGIN                                               \
@@ -142,11 +138,13 @@ struct SweepOcc {
 
 // Pre-smooth from zero, residual, weighted restriction input:
 // t_i = p_i (b_i - sum_j a_ij xpre_j), xpre = D^-1 b.
-template <typename T, typename IDX, int U, bool STREAM>
+// STEP: the first kernel of an iteration that follows another one in the same
+// loop body; it reads that iteration's outcome (step_outcome).
+template <typename T, typename IDX, int U, bool STREAM, bool STEP>
 __global__ void __launch_bounds__(kBlock, SweepOcc<T, U>::kMinBlocks) k_down(
     int n, const int32_t *__restrict__ sptr, const IDX *__restrict__ col, const T *__restrict__ val,
     const IDX *__restrict__ upat, const T *__restrict__ xpre, const T *__restrict__ b,
-    const T *__restrict__ p, T *__restrict__ t, const Ctl *__restrict__ ctl) {
+    const T *__restrict__ p, T *__restrict__ t, const double *pc, int gc, Ctl *ctl, double *hist) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int stride = gridDim.x * blockDim.x;
     RowOf<U, STREAM, IDX, T> R;
@@ -159,7 +157,8 @@ __global__ void __launch_bounds__(kBlock, SweepOcc<T, U>::kMinBlocks) k_down(
     xpre = after_wait(xpre);
     b = after_wait(b);
     ctl = after_wait(ctl);
-    if (ctl->done) return;
+    if (ctl->halt) return;
+    if (STEP && step_outcome(after_wait(pc), gc, ctl, hist) != kRun) return;
     for (; i < n; i += stride) {
         T acc = R.dot(i, [&](int j) { return ldg(xpre + j); });
         t[i] = pi * (ldg(b + i) - acc);
@@ -193,7 +192,7 @@ __global__ void __launch_bounds__(kBlock) k_down_ml(int n, const int32_t *__rest
     xpre = after_wait(xpre);
     b = after_wait(b);
     ctl = after_wait(ctl);
-    if (ctl->done) return;
+    if (ctl->halt) return;
     T acc = R.dot(row, [&](int j) { return ldg(xpre + j); });
     if (live && q == 0) t[row] = pi * (ldg(b + row) - acc);
 }
@@ -216,7 +215,7 @@ __global__ void __launch_bounds__(kBlock) k_post_ml(int n, const int32_t *__rest
     xp = after_wait(xp);
     b = after_wait(b);
     ctl = after_wait(ctl);
-    if (ctl->done) return;
+    if (ctl->halt) return;
     T acc = R.dot(row, [&](int j) { return ldg(xp + j); });
     if (live && q == 0) z[row] = ldg(xp + row) + di * (ldg(b + row) - acc);
 }
@@ -238,7 +237,7 @@ __global__ void __launch_bounds__(kBlock) k_prolong(int n, const T *__restrict__
     xpre = after_wait(xpre);
     xc = after_wait(xc);
     ctl = after_wait(ctl);
-    if (ctl->done) return;
+    if (ctl->halt) return;
     for (; i < n; i += stride) {
         T x = ldg(xpre + i);
         if (a >= 0) x += pw * ldg(xc + a);
@@ -251,8 +250,8 @@ __global__ void __launch_bounds__(kBlock) k_prolong(int n, const T *__restrict__
 }
 
 // Post-smooth z_i = xp_i + dinv_i (b_i - sum_j a_ij xp_j). On level 0 (DOT)
-// z is written in float64 and the kernel also forms r.z (float64 r) and, for
-// FCG(1), z.q_old; its last block turns them into rho and beta.
+// z is written in float64 and the kernel also leaves partial sums of r.z
+// (float64 r) and, for FCG(1), z.q_old for k_axpy_p.
 template <typename T, typename TZ, bool DOT, bool FCG, typename IDX, int U, bool STREAM>
 __global__ void __launch_bounds__(kBlock, SweepOcc<T, U>::kMinBlocks) k_post(
     int n, const int32_t *__restrict__ sptr, const IDX *__restrict__ col, const T *__restrict__ val,
@@ -273,7 +272,7 @@ __global__ void __launch_bounds__(kBlock, SweepOcc<T, U>::kMinBlocks) k_post(
     r64 = after_wait(r64);
     qold = after_wait(qold);
     ctl = after_wait(ctl);
-    if (ctl->done) return;
+    if (ctl->halt) return;
     double rz = 0.0, zq = 0.0;
     for (; i < n; i += stride) {
         T acc = R.dot(i, [&](int j) { return ldg(xp + j); });
@@ -289,11 +288,10 @@ __global__ void __launch_bounds__(kBlock, SweepOcc<T, U>::kMinBlocks) k_post(
         }
     }
     if (DOT) {
-        if (publish_partials(rz, zq, partials, &ctl->counter[0])) {
-            double a, bb;
-            final_sum2(partials, a, bb);
-            if (threadIdx.x == 0) finish_rho(ctl, a, bb);
-        }
+        double sums[FCG ? 2 : 1];
+        sums[0] = rz;
+        if (FCG) sums[FCG ? 1 : 0] = zq;
+        write_partials<FCG ? 2 : 1>(sums, partials);
     }
 }
 
@@ -320,7 +318,7 @@ __global__ void __launch_bounds__(kBlock) k_restrict(int nc, const int32_t *__re
     pdl_enter();
     t = after_wait(t);
     ctl = after_wait(ctl);
-    if (ctl->done || I >= nc) return;
+    if (ctl->halt || I >= nc) return;
     T tv[M];
 #pragma unroll
     for (int u = 0; u < M; u++) tv[u] = k0 + u < k1 ? ldg(t + m[u]) : T(0);
@@ -343,7 +341,7 @@ __global__ void __launch_bounds__(kBlock) k_restrict_sa(int nc, const int32_t *_
                                                         const T *__restrict__ dinvc, T *__restrict__ xprec,
                                                         const Ctl *__restrict__ ctl) {
     pdl_enter();
-    if (ctl->done) return;
+    if (ctl->halt) return;
     int I = blockIdx.x * blockDim.x + threadIdx.x;
     if (I >= nc) return;
     T s = 0;
@@ -359,7 +357,7 @@ __global__ void __launch_bounds__(kBlock) k_prolong_sa(int n, const int32_t *__r
                                                        const T *__restrict__ xpre, const T *__restrict__ xc,
                                                        T *__restrict__ xp, const Ctl *__restrict__ ctl) {
     pdl_enter();
-    if (ctl->done) return;
+    if (ctl->halt) return;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         T s = 0;
         for (int32_t q = ldg(prp + i); q < ldg(prp + i + 1); q++) s += ldg(pv + q) * ldg(xc + ldg(pci + q));
@@ -402,7 +400,7 @@ __global__ void __launch_bounds__(kBlock) k_down_restrict(int nc, const int32_t 
     xpre = after_wait(xpre);
     b = after_wait(b);
     ctl = after_wait(ctl);
-    if (ctl->done || I >= nc) return;
+    if (ctl->halt || I >= nc) return;
     T sum = 0;
     for (int32_t q = q0; q < q1; q++) {
         T acc = R.dot(i, [&](int j) { return ldg(xpre + j); });
@@ -443,7 +441,7 @@ __global__ void __launch_bounds__(kBlock) k_prolong_post(int n, const int32_t *_
     xc = after_wait(xc);
     b = after_wait(b);
     ctl = after_wait(ctl);
-    if (ctl->done) return;
+    if (ctl->halt) return;
     auto xp = [&](int j) {
         T x = ldg(xpre + j);
         int a = ldg(agg + j);
@@ -476,7 +474,7 @@ __global__ void __launch_bounds__(kBlock) k_gs_sweep(int n, int nb, const int32_
                                                      const T *__restrict__ dinv, const T *__restrict__ b,
                                                      const T *__restrict__ xo, T *xn, const Ctl *__restrict__ ctl) {
     pdl_enter();
-    if (ctl->done) return;
+    if (ctl->halt) return;
     int64_t lo64 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * nb;
     if (lo64 >= n) return;
     const int lo = (int)lo64, hi = (int)min((int64_t)n, lo64 + nb);
@@ -509,7 +507,7 @@ __global__ void __launch_bounds__(kBlock, Occ<T>::kMinBlocks) k_gs_offsum(
     int n, int nb, const int32_t *__restrict__ sptr, const IDX *__restrict__ col, const T *__restrict__ val,
     const T *__restrict__ xo, T *__restrict__ acc, const Ctl *__restrict__ ctl) {
     pdl_enter();
-    if (ctl->done) return;
+    if (ctl->halt) return;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         SELL_ROW_BEGIN
         const int lo = (i / nb) * nb, hi = min(n, lo + nb);
@@ -537,7 +535,7 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_block(int n, int nb, int w, c
                                                          const Ctl *__restrict__ ctl) {
     __shared__ T win[kGsThreads * 33];
     pdl_enter();
-    if (ctl->done) return;
+    if (ctl->halt) return;
     int64_t lo64 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * nb;
     if (lo64 >= n) return;
     const int lo = (int)lo64, hi = (int)min((int64_t)n, lo64 + nb);
@@ -577,7 +575,7 @@ __global__ void __launch_bounds__(kBlock, Occ<T>::kMinBlocks) k_gs_warp(
     const int32_t *__restrict__ pci, const T *__restrict__ pv, const T *__restrict__ dinv, const T *__restrict__ b,
     const T *__restrict__ xo, T *__restrict__ xn, const Ctl *__restrict__ ctl) {
     pdl_enter();
-    if (ctl->done) return;
+    if (ctl->halt) return;
     const int lane = threadIdx.x & 31;
     const int nsl = (n + 31) >> 5;
     const int wstride = (int)(((int64_t)gridDim.x * blockDim.x) >> 5);
@@ -644,8 +642,8 @@ __global__ void __launch_bounds__(kBlock, Occ<T>::kMinBlocks) k_gs_warp(
     }
 }
 
-// Level 0 after the Gauss-Seidel post-smoothing: z = x (widened), r.z and,
-// for FCG(1), z.q_old; the last block forms rho and beta. Same grid and row
+// Level 0 after the Gauss-Seidel post-smoothing: z = x (widened) and the
+// partial sums of r.z and, for FCG(1), z.q_old. Same grid and row
 // order as the level-0 k_post, so the sums are formed in the same order.
 template <typename T, bool FCG>
 __global__ void __launch_bounds__(kBlock, Occ<T>::kMinBlocks) k_gs_finish0(int n, const T *__restrict__ x,
@@ -654,7 +652,7 @@ __global__ void __launch_bounds__(kBlock, Occ<T>::kMinBlocks) k_gs_finish0(int n
                                                                            double *__restrict__ z, double *partials,
                                                                            Ctl *ctl) {
     pdl_enter();
-    if (ctl->done) return;
+    if (ctl->halt) return;
     double rz = 0.0, zq = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         double zo = (double)ldg(x + i);
@@ -662,11 +660,10 @@ __global__ void __launch_bounds__(kBlock, Occ<T>::kMinBlocks) k_gs_finish0(int n
         rz += ldg(r64 + i) * zo;
         if (FCG) zq += zo * ldg(qold + i);
     }
-    if (publish_partials(rz, zq, partials, &ctl->counter[0])) {
-        double a, bb;
-        final_sum2(partials, a, bb);
-        if (threadIdx.x == 0) finish_rho(ctl, a, bb);
-    }
+    double sums[FCG ? 2 : 1];
+    sums[0] = rz;
+    if (FCG) sums[FCG ? 1 : 0] = zq;
+    write_partials<FCG ? 2 : 1>(sums, partials);
 }
 
 // x_L = A_L^{-1} b_L, one warp per row; TO = float rounds the float64 result.
@@ -675,7 +672,7 @@ __global__ void __launch_bounds__(kBlock) k_coarse(int nL, const double *__restr
                                                    const double *__restrict__ bL, TO *__restrict__ xL,
                                                    const Ctl *__restrict__ ctl) {
     pdl_enter();
-    if (ctl->done) return;
+    if (ctl->halt) return;
     int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (row >= nL) return;
     const double *a = ainv + (int64_t)row * nL;
@@ -694,7 +691,7 @@ __global__ void __launch_bounds__(kBlock) k_coarse_only(int n, const double *__r
                                                         const double *__restrict__ qold, double *partials,
                                                         Ctl *ctl) {
     pdl_enter();
-    if (ctl->done) return;
+    if (ctl->halt) return;
     double rz = 0.0, zq = 0.0;
     int lane = threadIdx.x & 31;
     int wpb = blockDim.x >> 5;
@@ -715,30 +712,70 @@ __global__ void __launch_bounds__(kBlock) k_coarse_only(int n, const double *__r
             if (FCG) zq += zo * qold[row];
         }
     }
-    if (publish_partials(rz, zq, partials, &ctl->counter[0])) {
-        double a, bb;
-        final_sum2(partials, a, bb);
-        if (threadIdx.x == 0) finish_rho(ctl, a, bb);
-    }
+    double sums[FCG ? 2 : 1];
+    sums[0] = rz;
+    if (FCG) sums[FCG ? 1 : 0] = zq;
+    write_partials<FCG ? 2 : 1>(sums, partials);
 }
 
 // ------------------------------------------------------------ Krylov kernels
-// p = z + beta p (beta = 0 on a restart gives p = z).
-__global__ void __launch_bounds__(kBlock) k_axpy_p(int n, const double *__restrict__ z, double *__restrict__ p,
-                                                   const Ctl *__restrict__ ctl) {
+// rho = r.z and beta from the partial sums of the kernel that produced z:
+// PCG beta = rho / rho_old, FCG(1) beta = -(z.q_old) / (p.q)_old (the float32
+// V-cycle, and either precision when the iterative coarsest solve makes the
+// V-cycle vary from one application to the next); then p = z + beta p
+// (beta = 0 on a restart gives p = z). The first row's z and p and the scalars
+// are requested before the partials are summed.
+template <bool FCG>
+__global__ void __launch_bounds__(kVecBlock) k_axpy_p(int n, const double *__restrict__ z, double *__restrict__ p,
+                                                      const double *pa, int ga, Ctl *ctl) {
     pdl_enter();
-    if (ctl->done) return;
-    double beta = ctl->beta;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        p[i] = z[i] + beta * p[i];
+    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int stride = gridDim.x * blockDim.x;
+    const int halt = ctl->halt, restart = ctl->restart;
+    const double pq_old = ctl->pq_old, rho_old = ctl->rho_old;
+    double zi = 0.0, pi = 0.0;
+    if (i < n) {
+        zi = z[i];
+        pi = p[i];
+    }
+    if (halt) return;
+    __shared__ double sbeta;
+    __shared__ bool ok;
+    double sums[FCG ? 2 : 1];
+    sum_partials<FCG ? 2 : 1>(pa, ga, sums);
+    if (threadIdx.x == 0) {
+        const double rz = sums[0], zq = FCG ? sums[FCG ? 1 : 0] : 0.0;
+        const bool finite = isfinite(rz) && isfinite(zq);
+        ok = finite && rz > 0.0;
+        sbeta = restart ? 0.0 : FCG ? -zq / pq_old : rz / rho_old;
+        if (blockIdx.x == 0) {
+            if (ok) {
+                ctl->rho = rz;
+                ctl->zq = zq;
+                ctl->beta = sbeta;
+            } else {
+                fail(ctl, finite ? AMG_ERR_BREAKDOWN : AMG_ERR_NAN);
+            }
+        }
+    }
+    __syncthreads();
+    if (!ok) return;
+    const double beta = sbeta;
+    for (; i < n; i += stride) {
+        p[i] = zi + beta * pi;
+        if (i + stride < n) {
+            zi = z[i + stride];
+            pi = p[i + stride];
+        }
+    }
 }
 
-// q = A p and p.q; the last block forms alpha = rho / p.q.
+// q = A p and the partial sums of p.q.
 template <typename IDX>
 __global__ void __launch_bounds__(kBlock, 4) k_spmv(int n, const int32_t *__restrict__ sptr,
                                                     const IDX *__restrict__ col, const double *__restrict__ val,
                                                     const IDX *__restrict__ upat, const double *__restrict__ p,
-                                                    double *__restrict__ q, double *partials, Ctl *ctl) {
+                                                    double *__restrict__ q, double *partials, const Ctl *ctl) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int stride = gridDim.x * blockDim.x;
     SellRow<kUnroll, true, IDX, double> R;
@@ -746,7 +783,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_spmv(int n, const int32_t *__rest
     pdl_enter();
     p = after_wait(p);
     ctl = after_wait(ctl);
-    if (ctl->done) return;
+    if (ctl->halt) return;
     double pq = 0.0;
     for (; i < n; i += stride) {
         double acc = R.dot(i, [&](int j) { return ldg(p + j); });
@@ -754,17 +791,8 @@ __global__ void __launch_bounds__(kBlock, 4) k_spmv(int n, const int32_t *__rest
         pq += ldg(p + i) * acc;
         if (i + stride < n) R.load(sptr, col, val, i + stride, upat);
     }
-    if (publish_partials(pq, 0.0, partials, &ctl->counter[1])) {
-        double a, unused;
-        final_sum2(partials, a, unused);
-        if (threadIdx.x == 0) {
-            ctl->counter[1] = 0;
-            if (!isfinite(a)) { fail(ctl, AMG_ERR_NAN); return; }
-            if (!(a > 0.0)) { fail(ctl, AMG_ERR_BREAKDOWN); return; }
-            ctl->pq = a;
-            ctl->alpha = ctl->rho / a;
-        }
-    }
+    double sums[1] = {pq};
+    write_partials<1>(sums, partials);
 }
 
 // What the V-cycle of the mode reads besides r: FCG32 a float32 copy of r
@@ -789,55 +817,112 @@ __device__ __forceinline__ void emit_r(int i, double ri, const REmit &e) {
     }
 }
 
-// x += alpha p, r -= alpha q, ||r||^2; the last block records the relative
-// residual, advances the iteration and decides whether to check the true one.
+// alpha = rho / p.q from the partial sums of k_spmv, then x += alpha p,
+// r -= alpha q and the partial sums of ||r||^2; one thread advances the
+// iteration. The first row's vectors and the scalars are requested before the
+// partials are summed.
 template <int MODE>
-__global__ void __launch_bounds__(kBlock) k_update(int n, const double *__restrict__ p,
-                                                   const double *__restrict__ q, double *__restrict__ x,
-                                                   double *__restrict__ r, REmit em, double *partials, Ctl *ctl,
-                                                   double *hist) {
+__global__ void __launch_bounds__(kVecBlock) k_update(int n, const double *__restrict__ p,
+                                                      const double *__restrict__ q, double *__restrict__ x,
+                                                      double *__restrict__ r, REmit em, const double *pb, int gb,
+                                                      double *partials, Ctl *ctl) {
     pdl_enter();
-    if (ctl->done) return;
-    double alpha = ctl->alpha;
+    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int stride = gridDim.x * blockDim.x;
+    const int halt = ctl->halt;
+    const double rho = ctl->rho;
+    const int iter = ctl->iter;
+    double pi = 0.0, qi = 0.0, xi = 0.0, ro = 0.0;
+    if (i < n) {
+        pi = p[i];
+        qi = q[i];
+        xi = x[i];
+        ro = r[i];
+    }
+    if (halt) return;
+    __shared__ double salpha;
+    __shared__ bool ok;
+    double sums[1];
+    sum_partials<1>(pb, gb, sums);
+    if (threadIdx.x == 0) {
+        const double pq = sums[0];
+        const bool finite = isfinite(pq);
+        ok = finite && pq > 0.0;
+        salpha = rho / pq;
+        if (blockIdx.x == 0) {
+            if (ok) {
+                ctl->pq = pq;
+                ctl->alpha = salpha;
+                ctl->rho_old = rho;
+                ctl->pq_old = pq;
+                ctl->restart = 0;
+                ctl->iter = iter + 1;
+            } else {
+                fail(ctl, finite ? AMG_ERR_BREAKDOWN : AMG_ERR_NAN);
+            }
+        }
+    }
+    __syncthreads();
+    if (!ok) return;
+    const double alpha = salpha;
     double rr = 0.0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        x[i] = x[i] + alpha * p[i];
-        double ri = r[i] - alpha * q[i];
+    for (; i < n; i += stride) {
+        x[i] = xi + alpha * pi;
+        double ri = ro - alpha * qi;
         r[i] = ri;
         emit_r<MODE>(i, ri, em);
         rr += ri * ri;
-    }
-    if (publish_partials(rr, 0.0, partials, &ctl->counter[2])) {
-        double a, unused;
-        final_sum2(partials, a, unused);
-        if (threadIdx.x == 0) {
-            ctl->counter[2] = 0;
-            int it = ctl->iter + 1;
-            ctl->iter = it;
-            double rel = sqrt(a) / ctl->bnorm;
-            ctl->rel = rel;
-            hist[it] = rel;
-            ctl->rho_old = ctl->rho;
-            ctl->pq_old = ctl->pq;
-            ctl->restart = 0;
-            if (!isfinite(rel)) { fail(ctl, AMG_ERR_NAN); return; }
-            if (rel <= ctl->rtol) ctl->check = 1;
-            else if (it >= ctl->maxit) fail(ctl, AMG_ERR_NOCONV);
+        if (i + stride < n) {
+            pi = p[i + stride];
+            qi = q[i + stride];
+            xi = x[i + stride];
+            ro = r[i + stride];
         }
     }
+    sums[0] = rr;
+    write_partials<1>(sums, partials);
+}
+
+// Loop condition of the solve graph: run another body while not ended. The
+// body count is bounded independently of the kernels' own bookkeeping: a body
+// runs at least one iteration, so past maxit + 1 bodies the solve is ended as
+// not converged.
+struct Cond {
+    cudaGraphConditionalHandle hc;
+    int set;  // 0: not the last kernel of a graph's prefix or loop body
+};
+
+__device__ __forceinline__ void set_cond(const Cond &c, Ctl *ctl, bool body) {
+    if (!c.set) return;
+    if (body) {
+        const int b = ctl->bodies + 1;
+        ctl->bodies = b;
+        if (!ctl->done && b > ctl->maxit + 1) fail(ctl, AMG_ERR_NOCONV);
+    }
+    cudaGraphSetConditional(c.hc, ctl->done ? 0u : 1u);
 }
 
 // r = b - A x, ||r||^2 (and ||b||^2 on INIT); also the mode's copy of r.
-// Otherwise (not INIT) it runs only when the recursive residual met rtol.
+// INIT starts a solve. Otherwise it ends a loop body: it takes the outcome of
+// the iteration before it (unless a kernel of the body has taken it), forms
+// the true residual only when the recursive one met rtol, and sets the loop
+// condition.
 template <bool INIT, int MODE, typename IDX>
 __global__ void __launch_bounds__(kBlock, 4) k_residual(int n, const int32_t *__restrict__ sptr,
                                                         const IDX *__restrict__ col,
                                                         const double *__restrict__ val, const double *__restrict__ b,
                                                         const double *__restrict__ x, double *__restrict__ r,
-                                                        REmit em, double *partials, Ctl *ctl, double *hist) {
+                                                        REmit em, const double *pc, int gc, double *partials,
+                                                        Ctl *ctl, double *hist, Cond cond) {
     pdl_enter();
-    if (ctl->done) return;
-    if (!INIT && !ctl->check) return;
+    if (!INIT) {
+        int h = ctl->halt;
+        if (h == kRun) h = step_outcome(pc, gc, ctl, hist);
+        if (h != kCheck) {
+            if (blockIdx.x == 0 && threadIdx.x == 0) set_cond(cond, ctl, true);
+            return;
+        }
+    }
     double rr = 0.0, bb = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         SELL_ROW_BEGIN
@@ -849,55 +934,47 @@ __global__ void __launch_bounds__(kBlock, 4) k_residual(int n, const int32_t *__
         rr += ri * ri;
         if (INIT) bb += bi * bi;
     }
-    if (publish_partials(rr, bb, partials, &ctl->counter[3])) {
-        double a, bsq;
-        final_sum2(partials, a, bsq);
-        if (threadIdx.x == 0) {
-            ctl->counter[3] = 0;
-            if (INIT) {
-                double bn = sqrt(bsq);
-                ctl->bnorm = bn;
-                if (!isfinite(bn) || !isfinite(a)) { fail(ctl, AMG_ERR_NAN); return; }
-                if (bn == 0.0) { ctl->done = 1; ctl->status = AMG_OK; ctl->true_rel = 0.0; hist[0] = 0.0; return; }
-                double rel = sqrt(a) / bn;
-                ctl->rel = rel;
-                ctl->true_rel = rel;
-                hist[0] = rel;
-                if (rel <= ctl->rtol) { ctl->done = 1; ctl->status = AMG_OK; }
-                else if (ctl->maxit <= 0) fail(ctl, AMG_ERR_NOCONV);
+    double sums[2] = {rr, bb};
+    if (publish_partials<2>(sums, partials, &ctl->counter)) {
+        __threadfence();
+        sum_partials<2>(partials, gridDim.x, sums);
+        if (threadIdx.x != 0) return;
+        const double a = sums[0], bsq = sums[1];
+        ctl->counter = 0;
+        if (INIT) {
+            const double bn0 = sqrt(bsq), stop = ctl->rtol * bn0;
+            ctl->bnorm = bn0;
+            ctl->stop2 = stop * stop;
+        }
+        const double bn = ctl->bnorm, rel = sqrt(a) / bn;
+        if (INIT && (!isfinite(bn) || !isfinite(a))) {
+            fail(ctl, AMG_ERR_NAN);
+        } else if (INIT && bn == 0.0) {
+            ctl->true_rel = 0.0;
+            hist[0] = 0.0;
+            finish(ctl);
+        } else {
+            ctl->true_rel = rel;
+            if (INIT) ctl->rel = rel;
+            if (!isfinite(rel)) {
+                fail(ctl, AMG_ERR_NAN);
+            } else if (rel <= ctl->rtol) {
+                if (INIT) hist[0] = rel;
+                finish(ctl);
             } else {
-                double rel = sqrt(a) / ctl->bnorm;
-                ctl->true_rel = rel;
-                ctl->check = 0;
-                if (!isfinite(rel)) { fail(ctl, AMG_ERR_NAN); return; }
-                if (rel <= ctl->rtol) { ctl->done = 1; ctl->status = AMG_OK; return; }
                 ctl->restart = 1;
+                ctl->halt = kRun;
                 hist[ctl->iter] = rel;
                 if (ctl->iter >= ctl->maxit) fail(ctl, AMG_ERR_NOCONV);
             }
         }
+        set_cond(cond, ctl, !INIT);
     }
 }
 
 __global__ void k_zero(double *a, int n) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) a[i] = 0.0;
-}
-
-// Loop condition of the solve graph: run another body while not done. The
-// body count is bounded independently of the kernels' own bookkeeping: past
-// (maxit + 1) / 2 + 1 bodies the solve is ended as not converged.
-__global__ void k_set_cond(cudaGraphConditionalHandle hc, Ctl *ctl, int count_body) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    if (count_body) {
-        int b = ctl->bodies + 1;
-        ctl->bodies = b;
-        if (!ctl->done && b > (ctl->maxit + 1) / 2 + 1) {
-            ctl->done = 2;
-            ctl->status = AMG_ERR_NOCONV;
-        }
-    }
-    cudaGraphSetConditional(hc, ctl->done ? 0u : 1u);
 }
 
 inline int grid_rows(int64_t n) { return (int)((n + kBlock - 1) / kBlock); }
@@ -1060,11 +1137,13 @@ void launch_down(amg_hier *h, int l, unsigned char shape, cudaStream_t s) {
     }
     int g = shape_grid(h, n, prec_index<T>(), 0, shape);
     if (shape & 1)
-        WITH_COLS(lv.S, (launch_k(h->pdl, k_down<T, IDX, kUnrollSmall, false>, g, kBlock, s, n, lv.S.sptr, cols,
-                                  P::val(lv), pats, P::xpre(lv), P::b(lv), pdown<T>(h, lv), P::t(lv), (const Ctl *)h->ctl)));
+        WITH_COLS(lv.S, (launch_k(h->pdl, k_down<T, IDX, kUnrollSmall, false, false>, g, kBlock, s, n, lv.S.sptr,
+                                  cols, P::val(lv), pats, P::xpre(lv), P::b(lv), pdown<T>(h, lv), P::t(lv),
+                                  (const double *)nullptr, 0, h->ctl, (double *)nullptr)));
     else
-        WITH_COLS(lv.S, (launch_k(h->pdl, k_down<T, IDX, kUnroll, false>, g, kBlock, s, n, lv.S.sptr, cols,
-                                  P::val(lv), pats, P::xpre(lv), P::b(lv), pdown<T>(h, lv), P::t(lv), (const Ctl *)h->ctl)));
+        WITH_COLS(lv.S, (launch_k(h->pdl, k_down<T, IDX, kUnroll, false, false>, g, kBlock, s, n, lv.S.sptr, cols,
+                                  P::val(lv), pats, P::xpre(lv), P::b(lv), pdown<T>(h, lv), P::t(lv),
+                                  (const double *)nullptr, 0, h->ctl, (double *)nullptr)));
 }
 
 // Restriction from level l to l+1 (the coarsest gets float64 b_L).
@@ -1180,7 +1259,7 @@ int launch_coarsest(amg_hier *h, cudaStream_t s, int *kernels) {
     using P = LP<T>;
     Level &lc = h->lev.back();
     if (h->coarse_iter) {
-        PCG_TRY(launch_coarse_iter<T>(h, h->cws, h->bL, P::x(lc), &h->ctl->done, nullptr, s));
+        PCG_TRY(launch_coarse_iter<T>(h, h->cws, h->bL, P::x(lc), &h->ctl->halt, nullptr, s));
         *kernels += coarse_iter_launches(h);
         return AMG_OK;
     }
@@ -1198,23 +1277,37 @@ int grid0(const amg_hier *h) { return sizeof(T) == 4 ? h->grid32 : h->grid64; }
 // offset patterns (PatRow), else 4-entry chunks.
 inline bool pat_rows(const amg_hier *h) { return h->lev[0].S.upat != nullptr; }
 
+// Sections of the partial sums, 2 h->nblk values each: what k_post left for
+// k_axpy_p, k_spmv for k_update, k_update for the next iteration's first
+// kernel or k_residual, and k_residual's own.
+inline double *parts(const amg_hier *h, int section) { return h->partials + 2 * (size_t)h->nblk * section; }
+constexpr int kPartsRz = 0, kPartsPq = 1, kPartsRr = 2, kPartsTrue = 3, kPartSections = 4;
+
 // Level-0 down sweep t = p (b - A xpre) (evict-first matrix stream, shared
-// offset patterns where level 0 has them).
-template <typename T>
-void launch_down0(amg_hier *h, const T *b0, cudaStream_t s) {
+// offset patterns where level 0 has them). step: it takes the outcome of the
+// iteration before it.
+template <typename T, bool STEP>
+void launch_down0_t(amg_hier *h, const T *b0, cudaStream_t s) {
     using P = LP<T>;
     Level &l0 = h->lev[0];
+    const double *pc = parts(h, kPartsRr);
     if constexpr (sizeof(T) == 4) {
         if (pat_rows(h)) {
-            WITH_COLS(l0.S, (launch_k(h->pdl, k_down<T, IDX, kPatRow, true>, grid0<T>(h), kBlock, s, l0.A.n,
+            WITH_COLS(l0.S, (launch_k(h->pdl, k_down<T, IDX, kPatRow, true, STEP>, grid0<T>(h), kBlock, s, l0.A.n,
                                       l0.S.sptr, cols, P::val(l0), pats, (const T *)P::xpre(l0), b0,
-                                      pdown<T>(h, l0), P::t(l0), (const Ctl *)h->ctl)));
+                                      pdown<T>(h, l0), P::t(l0), pc, h->gridv, h->ctl, h->hist)));
             return;
         }
     }
-    WITH_COLS(l0.S, (launch_k(h->pdl, k_down<T, IDX, kUnroll, true>, grid0<T>(h), kBlock, s, l0.A.n,
-                                  l0.S.sptr, cols, P::val(l0), pats, (const T *)P::xpre(l0), b0, pdown<T>(h, l0),
-                                  P::t(l0), (const Ctl *)h->ctl)));
+    WITH_COLS(l0.S, (launch_k(h->pdl, k_down<T, IDX, kUnroll, true, STEP>, grid0<T>(h), kBlock, s, l0.A.n, l0.S.sptr,
+                              cols, P::val(l0), pats, (const T *)P::xpre(l0), b0, pdown<T>(h, l0), P::t(l0), pc,
+                              h->gridv, h->ctl, h->hist)));
+}
+
+template <typename T>
+void launch_down0(amg_hier *h, const T *b0, bool step, cudaStream_t s) {
+    if (step) launch_down0_t<T, true>(h, b0, s);
+    else launch_down0_t<T, false>(h, b0, s);
 }
 
 // Level-0 post sweep z = xp + dinv (b - A xp) with r.z (and z.q_old).
@@ -1226,25 +1319,25 @@ void launch_post0(amg_hier *h, const T *b0, cudaStream_t s) {
         if (pat_rows(h)) {
             WITH_COLS(l0.S, (launch_k(h->pdl, k_post<T, double, true, FCG, IDX, kPatRow, true>, grid0<T>(h), kBlock,
                                       s, l0.A.n, l0.S.sptr, cols, P::val(l0), pats, P::xp(l0), b0, P::dinv(l0), h->z,
-                                      h->r, h->q, h->partials, h->ctl)));
+                                      h->r, h->q, parts(h, kPartsRz), h->ctl)));
             return;
         }
     }
     WITH_COLS(l0.S, (launch_k(h->pdl, k_post<T, double, true, FCG, IDX, kUnroll, true>, grid0<T>(h), kBlock, s,
                                   l0.A.n, l0.S.sptr, cols, P::val(l0), pats, P::xp(l0), b0, P::dinv(l0), h->z, h->r,
-                                  h->q, h->partials, h->ctl)));
+                                  h->q, parts(h, kPartsRz), h->ctl)));
 }
 
 // z = B r (one V-cycle in precision T), including rho / beta. Kernels are
 // launched with programmatic dependent launch when h->pdl (see pdl_enter).
 template <typename T, bool FCG>
-int launch_vcycle(amg_hier *h, cudaStream_t s) {
+int launch_vcycle(amg_hier *h, bool step, cudaStream_t s) {
     using P = LP<T>;
     auto &lev = h->lev;
     int L = (int)lev.size() - 1;
     const T *b0 = P::r0(h);
     int sp1 = prof_begin(h, 0, s);
-    launch_down0<T>(h, b0, s);
+    launch_down0<T>(h, b0, step, s);
     prof_end(h, sp1, s);
     int sp2 = prof_begin(h, 5, s);
     // levels handled by separate launches: 0..F-1; the tail runs F..L
@@ -1285,7 +1378,7 @@ int launch_vcycle(amg_hier *h, cudaStream_t s) {
     kernels += 2;  // prolongation and post sweep of level 0
     prof_end(h, sp2, s);
     int sp7 = prof_begin(h, 7, s);
-    launch_prolong<T>(h, 0, h->gridv, s);
+    launch_prolong<T>(h, 0, h->gridp, s);
     prof_end(h, sp7, s);
     int sp3 = prof_begin(h, 1, s);
     launch_post0<T, FCG>(h, b0, s);
@@ -1422,7 +1515,7 @@ int launch_vcycle_gs(amg_hier *h, cudaStream_t s) {
     int kernels = 0;
     int sp1 = prof_begin(h, 0, s);
     kernels += launch_gs<T>(h, 0, true, b0, P::xpre(l0), s);
-    launch_down0<T>(h, b0, s);
+    launch_down0<T>(h, b0, false, s);
     kernels += 1;
     prof_end(h, sp1, s);
     int sp2 = prof_begin(h, 5, s);
@@ -1451,11 +1544,11 @@ int launch_vcycle_gs(amg_hier *h, cudaStream_t s) {
     }
     prof_end(h, sp2, s);
     int sp3 = prof_begin(h, 1, s);
-    launch_prolong<T>(h, 0, h->gridv, s);
+    launch_prolong<T>(h, 0, h->gridp, s);
     kernels += 1 + launch_gs<T>(h, 0, false, b0, P::x(l0), s);
     // the post sweep's grid, so rho is summed in the same order as there
     launch_k(pdl, k_gs_finish0<T, FCG>, grid0<T>(h), kBlock, s, l0.A.n, (const T *)P::x(l0), (const double *)h->r,
-             (const double *)h->q, h->z, h->partials, ctl);
+             (const double *)h->q, h->z, parts(h, kPartsRz), ctl);
     kernels += 1;
     prof_end(h, sp3, s);
     h->launches += kernels;
@@ -1463,64 +1556,81 @@ int launch_vcycle_gs(amg_hier *h, cudaStream_t s) {
     return AMG_OK;
 }
 
+// One iteration. first / last: its place in a loop body (or in a chunk of
+// stream launches); cond is set by the body's last kernel. An l1-Jacobi
+// V-cycle's first kernel takes the outcome of the iteration before it in the
+// body, so only the body's last iteration launches k_residual (one launch per
+// iteration less: 2.5 us); the other V-cycles launch it after every iteration.
 template <int MODE>
-int launch_iteration_t(amg_hier *h, cudaStream_t s) {
+int launch_iteration_t(amg_hier *h, bool first, bool last, const Cond &cond, cudaStream_t s) {
     int L = (int)h->lev.size() - 1;
     Level &l0 = h->lev[0];
     int n = l0.A.n;
     const bool pdl = h->pdl;
+    const bool takes = L > 0 && !h->gs_nu;  // the V-cycle can take an outcome
+    const bool step = takes && !first;
+    int ga = MODE == AMG_MODE_FCG32 ? h->grid32 : h->grid64;  // blocks of the kernel that left r.z
     if (L == 0) {
+        ga = h->gridv;
         launch_k(pdl, k_coarse_only<MODE == AMG_MODE_FCG32, MODE == AMG_MODE_FCG32>, h->gridv, kBlock, s, h->nL,
-                 h->Ainv, h->r, h->z, h->q, h->partials, h->ctl);
+                 h->Ainv, h->r, h->z, h->q, parts(h, kPartsRz), h->ctl);
         h->launches += 1;
     } else if (MODE == AMG_MODE_FCG32) {
         if (h->gs_nu) PCG_TRY((launch_vcycle_gs<float, true>(h, s)));
-        else PCG_TRY((launch_vcycle<float, true>(h, s)));
+        else PCG_TRY((launch_vcycle<float, true>(h, step, s)));
     } else if (h->coarse_iter) {
         // the float64 V-cycle is not a fixed operator either: FCG(1) beta
         if (h->gs_nu) PCG_TRY((launch_vcycle_gs<double, true>(h, s)));
-        else PCG_TRY((launch_vcycle<double, true>(h, s)));
+        else PCG_TRY((launch_vcycle<double, true>(h, step, s)));
     } else {
         if (h->gs_nu) PCG_TRY((launch_vcycle_gs<double, false>(h, s)));
-        else PCG_TRY((launch_vcycle<double, false>(h, s)));
+        else PCG_TRY((launch_vcycle<double, false>(h, step, s)));
     }
     int sp4 = prof_begin(h, 6, s);
-    launch_k(pdl, k_axpy_p, h->gridv, kBlock, s, n, h->z, h->p, h->ctl);
+    if (MODE == AMG_MODE_FCG32 || h->coarse_iter)
+        launch_k(pdl, k_axpy_p<true>, h->gridv, h->blockv, s, n, h->z, h->p, parts(h, kPartsRz), ga, h->ctl);
+    else
+        launch_k(pdl, k_axpy_p<false>, h->gridv, h->blockv, s, n, h->z, h->p, parts(h, kPartsRz), ga, h->ctl);
     prof_end(h, sp4, s);
     int sp5 = prof_begin(h, 2, s);
-    WITH_COLS(l0.S, (launch_k(pdl, k_spmv<IDX>, h->grid64, kBlock, s, n, l0.S.sptr, cols, l0.S.v64,
-                              pats, h->p, h->q,
-                              h->partials, h->ctl)));
+    WITH_COLS(l0.S, (launch_k(pdl, k_spmv<IDX>, h->grid64, kBlock, s, n, l0.S.sptr, cols, l0.S.v64, pats, h->p, h->q,
+                              parts(h, kPartsPq), h->ctl)));
     prof_end(h, sp5, s);
     int sp6 = prof_begin(h, 3, s);
-    launch_k(pdl, k_update<MODE>, h->gridv, kBlock, s, n, h->p, h->q, h->x, h->r, remit(h), h->partials, h->ctl,
-             h->hist);
+    launch_k(pdl, k_update<MODE>, h->gridv, h->blockv, s, n, h->p, h->q, h->x, h->r, remit(h), parts(h, kPartsPq),
+             h->grid64, parts(h, kPartsRr), h->ctl);
     prof_end(h, sp6, s);
-    int sp7 = prof_begin(h, 4, s);
-    WITH_COLS(l0.S, (launch_k(pdl, k_residual<false, MODE, IDX>, h->grid64, kBlock, s, n, l0.S.sptr, cols, l0.S.v64,
-                              h->b, h->x, h->r, remit(h), h->partials, h->ctl, h->hist)));
-    prof_end(h, sp7, s);
-    h->launches += 4;
+    h->launches += 3;
+    if (last || !takes) {
+        int sp7 = prof_begin(h, 4, s);
+        WITH_COLS(l0.S, (launch_k(pdl, k_residual<false, MODE, IDX>, h->grid64, kBlock, s, n, l0.S.sptr, cols,
+                                  l0.S.v64, h->b, h->x, h->r, remit(h), parts(h, kPartsRr), h->gridv,
+                                  parts(h, kPartsTrue), h->ctl, h->hist, last ? cond : Cond{})));
+        prof_end(h, sp7, s);
+        h->launches += 1;
+    }
     PCG_LAUNCH_CK();
     return AMG_OK;
 }
 
-int launch_iteration(amg_hier *h, cudaStream_t s) {
-    if (h->mode == AMG_MODE_FCG32) return launch_iteration_t<AMG_MODE_FCG32>(h, s);
-    return launch_iteration_t<AMG_MODE_PCG64>(h, s);
+int launch_iteration(amg_hier *h, bool first, bool last, const Cond &cond, cudaStream_t s) {
+    if (h->mode == AMG_MODE_FCG32) return launch_iteration_t<AMG_MODE_FCG32>(h, first, last, cond, s);
+    return launch_iteration_t<AMG_MODE_PCG64>(h, first, last, cond, s);
 }
 
-int launch_prefix(amg_hier *h, cudaStream_t s) {
+int launch_prefix(amg_hier *h, const Cond &cond, cudaStream_t s) {
     Level &l0 = h->lev[0];
     int n = l0.A.n;
     k_zero<<<grid_rows(n), kBlock, 0, s>>>(h->p, n);
     k_zero<<<grid_rows(n), kBlock, 0, s>>>(h->q, n);
     if (h->mode == AMG_MODE_FCG32)
         WITH_COLS(l0.S, (launch_k(h->pdl, k_residual<true, AMG_MODE_FCG32, IDX>, h->grid64, kBlock, s, n, l0.S.sptr,
-                                  cols, l0.S.v64, h->b, h->x, h->r, remit(h), h->partials, h->ctl, h->hist)));
+                                  cols, l0.S.v64, h->b, h->x, h->r, remit(h), (const double *)nullptr, 0,
+                                  parts(h, kPartsTrue), h->ctl, h->hist, cond)));
     else
         WITH_COLS(l0.S, (launch_k(h->pdl, k_residual<true, AMG_MODE_PCG64, IDX>, h->grid64, kBlock, s, n, l0.S.sptr,
-                                  cols, l0.S.v64, h->b, h->x, h->r, remit(h), h->partials, h->ctl, h->hist)));
+                                  cols, l0.S.v64, h->b, h->x, h->r, remit(h), (const double *)nullptr, 0,
+                                  parts(h, kPartsTrue), h->ctl, h->hist, cond)));
     h->launches += 3;
     PCG_LAUNCH_CK();
     return AMG_OK;
@@ -1530,13 +1640,13 @@ int launch_prefix(amg_hier *h, cudaStream_t s) {
 
 // Captures the prefix of one whole solve of h in `mode` onto cs, which must
 // be capturing (possibly as a forked branch of a larger capture): zero p/q,
-// first residual, the loop-condition kernel, and a while node whose body is
+// first residual (which sets the loop condition), and a while node whose body is
 // filled later by capture_solve_body. Kernel counts go to *prefix_k.
 int capture_solve_prefix(amg_hier *h, int mode, cudaStream_t cs, PendingBody *pb, int *prefix_k) {
     int saved_mode = h->mode;
     h->mode = mode;
     int64_t l0 = h->launches;
-    int st = launch_prefix(h, cs);
+    int st = AMG_OK;
     cudaGraph_t g = nullptr;
     cudaGraphConditionalHandle hc = 0;
     cudaStreamCaptureStatus cst;
@@ -1544,13 +1654,9 @@ int capture_solve_prefix(amg_hier *h, int mode, cudaStream_t cs, PendingBody *pb
     size_t nd = 0;
     cudaGraphNodeParams cp = {};
     cudaGraphNode_t cnode = nullptr;
-    cudaError_t e = cudaSuccess;
-    if (!st) e = cudaStreamGetCaptureInfo(cs, &cst, nullptr, &g, nullptr, nullptr, nullptr);
-    if (!st && e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&hc, g, 1, cudaGraphCondAssignDefault);
-    if (!st && e == cudaSuccess) {
-        k_set_cond<<<1, 32, 0, cs>>>(hc, h->ctl, 0);
-        e = cudaGetLastError();
-    }
+    cudaError_t e = cudaStreamGetCaptureInfo(cs, &cst, nullptr, &g, nullptr, nullptr, nullptr);
+    if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&hc, g, 1, cudaGraphCondAssignDefault);
+    if (e == cudaSuccess) st = launch_prefix(h, Cond{hc, 1}, cs);
     if (!st && e == cudaSuccess) e = cudaStreamGetCaptureInfo(cs, &cst, nullptr, &g, &deps, nullptr, &nd);
     if (!st && e == cudaSuccess) {
         cp.type = cudaGraphNodeTypeConditional;
@@ -1561,7 +1667,7 @@ int capture_solve_prefix(amg_hier *h, int mode, cudaStream_t cs, PendingBody *pb
     }
     if (!st && e == cudaSuccess)
         e = cudaStreamUpdateCaptureDependencies(cs, &cnode, nullptr, 1, cudaStreamSetCaptureDependencies);
-    *prefix_k = (int)(h->launches - l0) + 1;
+    *prefix_k = (int)(h->launches - l0);
     h->launches = l0;
     h->mode = saved_mode;
     if (st) return st;
@@ -1573,8 +1679,10 @@ int capture_solve_prefix(amg_hier *h, int mode, cudaStream_t cs, PendingBody *pb
     return AMG_OK;
 }
 
-// Fills the while node's body: two iterations and the condition kernel,
-// captured on s (not capturing). Kernel count of one body to *body_k.
+// Fills the while node's body: kBodyIters iterations, the last kernel of which
+// sets the loop condition, captured on s (not capturing). Kernel count of one
+// body to *body_k.
+constexpr int kBodyIters = 2;
 int capture_solve_body(const PendingBody &pb, cudaStream_t s, int *body_k) {
     amg_hier *h = pb.h;
     int saved_mode = h->mode;
@@ -1583,15 +1691,14 @@ int capture_solve_body(const PendingBody &pb, cudaStream_t s, int *body_k) {
     int st = AMG_OK;
     cudaError_t e = cudaStreamBeginCaptureToGraph(s, pb.body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        st = launch_iteration(h, s);
-        if (!st) st = launch_iteration(h, s);
-        if (!st) k_set_cond<<<1, 32, 0, s>>>(pb.hc, h->ctl, 1);
+        for (int k = 0; k < kBodyIters && !st; k++)
+            st = launch_iteration(h, k == 0, k + 1 == kBodyIters, Cond{pb.hc, 1}, s);
         cudaGraph_t bout = pb.body;
         cudaError_t e2 = cudaStreamEndCapture(s, &bout);
         if (e2 != cudaSuccess) e = e2;
         if (e == cudaSuccess) e = cudaGetLastError();
     }
-    *body_k = (int)(h->launches - l1) + 1;
+    *body_k = (int)(h->launches - l1);
     h->launches = l1;
     h->mode = saved_mode;
     if (st) return st;
@@ -1601,8 +1708,8 @@ int capture_solve_body(const PendingBody &pb, cudaStream_t s, int *body_k) {
 
 namespace {
 
-// Whole solve as one graph: prefix (zero p/q, first residual, condition),
-// then a while node whose body is two iterations plus the condition kernel.
+// Whole solve as one graph: prefix (zero p/q, first residual), then a while
+// node whose body is kBodyIters iterations.
 // tail = false builds the variant without the shared-memory tail.
 int build_graph(amg_hier *h, int mode, bool tail = true) {
     if (!h->cap_stream) PCG_CK(cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking));
@@ -1692,28 +1799,34 @@ int alloc_solve_workspace(amg_hier *h) {
         if (*grid < 1) *grid = 1;
         return AMG_OK;
     };
-    PCG_TRY(wave((const void *)k_down<float, int32_t, kUnroll, true>, &h->grid32));
+    PCG_TRY(wave((const void *)k_down<float, int32_t, kUnroll, true, true>, &h->grid32));
     if (pat_rows(h)) {
         // the whole-row sweeps: one wave of the fewer of their resident blocks
         int gd = 0, gp = 0;
         if (h->lev[0].S.col16) {
-            PCG_TRY(wave((const void *)k_down<float, int16_t, kPatRow, true>, &gd));
+            PCG_TRY(wave((const void *)k_down<float, int16_t, kPatRow, true, true>, &gd));
             PCG_TRY(wave((const void *)k_post<float, double, true, true, int16_t, kPatRow, true>, &gp));
         } else {
-            PCG_TRY(wave((const void *)k_down<float, int32_t, kPatRow, true>, &gd));
+            PCG_TRY(wave((const void *)k_down<float, int32_t, kPatRow, true, true>, &gd));
             PCG_TRY(wave((const void *)k_post<float, double, true, true, int32_t, kPatRow, true>, &gp));
         }
         h->grid32 = std::min(gd, gp);
     }
     PCG_TRY(wave((const void *)k_spmv<int32_t>, &h->grid64));
-    PCG_TRY(wave((const void *)k_update<AMG_MODE_FCG32>, &h->gridv));
+    PCG_TRY(wave((const void *)k_prolong<float>, &h->gridp));
+    // the vector kernels: at most two blocks per SM (their consumers read one
+    // partial per block), the block as large as the rows fill
+    const int vec_blocks = 2 * sms;
+    h->blockv = (int)std::min<int64_t>(kVecBlock, std::max<int64_t>(128, ((int64_t)n + vec_blocks - 1) / vec_blocks));
+    h->blockv = (h->blockv + 31) / 32 * 32;
+    h->gridv = std::min(vec_blocks, (n + h->blockv - 1) / h->blockv);
     h->nblk = std::max(h->grid32, std::max(h->grid64, h->gridv));
     // One wave of each coarse-level sweep variant, and the fixed shape rule.
     const void *fns[2][2][2] = {
-        {{(const void *)k_down<float, int16_t, kUnroll, false>, (const void *)k_down<float, int16_t, kUnrollSmall, false>},
+        {{(const void *)k_down<float, int16_t, kUnroll, false, false>, (const void *)k_down<float, int16_t, kUnrollSmall, false, false>},
          {(const void *)k_post<float, float, false, false, int16_t, kUnroll, false>,
           (const void *)k_post<float, float, false, false, int16_t, kUnrollSmall, false>}},
-        {{(const void *)k_down<double, int16_t, kUnroll, false>, (const void *)k_down<double, int16_t, kUnrollSmall, false>},
+        {{(const void *)k_down<double, int16_t, kUnroll, false, false>, (const void *)k_down<double, int16_t, kUnrollSmall, false, false>},
          {(const void *)k_post<double, double, false, false, int16_t, kUnroll, false>,
           (const void *)k_post<double, double, false, false, int16_t, kUnrollSmall, false>}}};
     for (int a = 0; a < 2; a++)
@@ -1734,7 +1847,7 @@ int alloc_solve_workspace(amg_hier *h) {
     PCG_TRY(alloc(M, &h->z, n));
     PCG_TRY(alloc(M, &h->q, n));
     PCG_TRY(alloc(M, &h->p, n));
-    PCG_TRY(alloc(M, &h->partials, 2 * (size_t)h->nblk));
+    PCG_TRY(alloc(M, &h->partials, 2 * (size_t)h->nblk * kPartSections));
     PCG_TRY(alloc(M, &h->ctl, 1));
     PCG_CK(cudaMemsetAsync(h->ctl, 0, sizeof(Ctl), M.stream));
     PCG_CK(cudaMallocHost(&h->ctl_host, sizeof(Ctl)));
@@ -1927,7 +2040,7 @@ int solve_impl(amg_hier *h, const double *b, double *x, double rtol, int maxit, 
         PCG_CK(cudaStreamSynchronize(s));
         h->launches += h->graph_prefix_kernels + (int64_t)h->ctl_host->bodies * h->graph_body_kernels[h->mode];
     } else {
-        PCG_TRY(launch_prefix(h, s));
+        PCG_TRY(launch_prefix(h, Cond{}, s));
         // Iterate in chunks; once done, every later kernel returns at once.
         const int chunk = 4;
         int launched = 0;
@@ -1936,7 +2049,9 @@ int solve_impl(amg_hier *h, const double *b, double *x, double rtol, int maxit, 
             PCG_CK(cudaStreamSynchronize(s));
             if (h->profile) prof_collect(h);
             if (h->ctl_host->done || launched >= maxit) break;
-            for (int k = 0; k < chunk && launched < maxit; k++, launched++) PCG_TRY(launch_iteration(h, s));
+            const int todo = std::min(chunk, maxit - launched);
+            for (int k = 0; k < todo; k++, launched++)
+                PCG_TRY(launch_iteration(h, k == 0, k + 1 == todo, Cond{}, s));
         }
     }
     Ctl &c = *h->ctl_host;
