@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(kCT) k_cinit(int n, int nb, int K, const doubl
                                                double *partials, CCtl *ctl, const int *outer_done,
                                                const int *outer_live) {
     pdl_enter();
-    if (*outer_done) {
+    if (__ldcg(outer_done)) {
         if (blockIdx.x == 0 && threadIdx.x == 0) ctl->any = 0;
         return;
     }
@@ -301,7 +301,7 @@ __global__ void __launch_bounds__(kCT) k_cinit(int n, int nb, int K, const doubl
             int any = 0;
             for (int c = 0; c < K; c++) {
                 double bn = sqrt(res[c]), rz = res[K + c];
-                int live = outer_live ? outer_live[c] : 1;
+                int live = outer_live ? __ldcg(outer_live + c) : 1;
                 int a = live && bn > 0.0 && isfinite(bn) && rz > 0.0 && isfinite(rz);
                 ctl->bn[c] = bn;
                 ctl->rho[c] = rz;
@@ -367,14 +367,14 @@ __global__ void __launch_bounds__(kCT) k_cq(int n, int nb, int K, const int32_t 
     pold = after_wait(pold);
     pnew = after_wait(pnew);
     q = after_wait(q);
-    if (!ctl->any) return;
+    if (!__ldcg(&ctl->any)) return;
     int c0 = it.g * KC;
     double beta[KC];
     bool live = false, first = true;
 #pragma unroll
     for (int v = 0; v < KC; v++) {
-        beta[v] = ctl->beta[c0 + v];
-        live |= ctl->active[c0 + v] != 0;
+        beta[v] = __ldcg(&ctl->beta[c0 + v]);
+        live |= __ldcg(&ctl->active[c0 + v]) != 0;
     }
     double acc[1][KC] = {};
     if (live) {
@@ -449,16 +449,16 @@ __global__ void __launch_bounds__(kCT) k_cq(int n, int nb, int K, const int32_t 
         if (threadIdx.x == 0) {
             int any = 0;
             for (int c = 0; c < K; c++) {
-                if (ctl->active[c]) {
+                if (__ldcg(&ctl->active[c])) {
                     double pq = res[c];
                     if (pq > 0.0 && isfinite(pq)) {
                         ctl->pq[c] = pq;
-                        ctl->alpha[c] = ctl->rho[c] / pq;
+                        ctl->alpha[c] = __ldcg(&ctl->rho[c]) / pq;
                     } else {
                         ctl->active[c] = 0;
                     }
                 }
-                any |= ctl->active[c];
+                any |= __ldcg(&ctl->active[c]);
             }
             ctl->any = any;
             ctl->counter[1] = 0;
@@ -489,15 +489,15 @@ __global__ void __launch_bounds__(kCT) k_cx(int n, int nb, int K, const double *
     r = after_wait(r);
     z = after_wait(z);
     xo = after_wait(xo);
-    if (!ctl->any) return;
+    if (!__ldcg(&ctl->any)) return;
     int c0 = it.g * KC;
     double alpha[KC];
     bool act[KC];
     bool live = false;
 #pragma unroll
     for (int v = 0; v < KC; v++) {
-        act[v] = ctl->active[c0 + v] != 0;
-        alpha[v] = act[v] ? ctl->alpha[c0 + v] : 0.0;
+        act[v] = __ldcg(&ctl->active[c0 + v]) != 0;
+        alpha[v] = act[v] ? __ldcg(&ctl->alpha[c0 + v]) : 0.0;
         live |= act[v];
     }
     double acc[3][KC] = {};
@@ -540,17 +540,17 @@ __global__ void __launch_bounds__(kCT) k_cx(int n, int nb, int K, const double *
         if (threadIdx.x == 0) {
             int any = 0;
             for (int c = 0; c < K; c++) {
-                if (ctl->active[c]) {
+                if (__ldcg(&ctl->active[c])) {
                     ctl->its[c] = iter;
                     double rn = sqrt(res[c]), rz = res[K + c], zq = res[2 * K + c];
-                    if (rn <= tol * ctl->bn[c] || iter >= maxit || !(rz > 0.0) || !isfinite(rz)) {
+                    if (rn <= tol * __ldcg(&ctl->bn[c]) || iter >= maxit || !(rz > 0.0) || !isfinite(rz)) {
                         ctl->active[c] = 0;
                     } else {
-                        ctl->beta[c] = -zq / ctl->pq[c];
+                        ctl->beta[c] = -zq / __ldcg(&ctl->pq[c]);
                         ctl->rho[c] = rz;
                     }
                 }
-                any |= ctl->active[c];
+                any |= __ldcg(&ctl->active[c]);
             }
             ctl->any = any;
             ctl->counter[0] = 0;

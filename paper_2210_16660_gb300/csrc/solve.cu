@@ -66,6 +66,15 @@ __device__ __forceinline__ bool publish_partials(double (&a)[NV], double *partia
     return last;
 }
 
+// Reads of the solve's state go to L2. A kernel launched with programmatic
+// dependence starts, and drops its SM's L1 lines, while its predecessor still
+// runs: a block of the predecessor on that SM may then bring a line of Ctl
+// into L1 before another block changes it, and nothing shows that a plain
+// load after the wait cannot still hit that line.
+template <typename T>
+__device__ __forceinline__ T state(const T *p) { return __ldcg(p); }
+__device__ __forceinline__ int halted(const Ctl *c) { return state(&c->halt); }
+
 // Ctl::halt: whether the iteration's kernels run
 constexpr int kRun = 0, kCheck = 1, kEnded = 2;
 
@@ -84,29 +93,41 @@ __device__ __forceinline__ void fail(Ctl *c, int status) {
 // Outcome of the iteration whose update left g partial sums of ||r||^2:
 // kRun, or why the kernels that follow must not run (kCheck: rtol met, the
 // true residual is formed next; kEnded). Called by every thread of every block
-// of one kernel; one thread records the outcome in ctl->halt (one word, so a
-// block that reads it already takes the same way as on its own).
+// of one kernel; one thread records the outcome in ctl->halt. A block that
+// starts after that finds it there, and takes the same way as on its own: the
+// flag is read by one thread for the whole block, as another block may be
+// writing it.
 __device__ __forceinline__ int step_outcome(const double *pc, int g, Ctl *ctl, double *hist) {
     __shared__ int out;
     __shared__ double srr;
-    const double stop2 = ctl->stop2;
-    const int it = ctl->iter, maxit = ctl->maxit;
+    int halt = kRun, it = 0, maxit = 0;
+    double stop2 = 0.0;
+    if (threadIdx.x == 0) {
+        halt = halted(ctl);
+        it = state(&ctl->iter);
+        maxit = state(&ctl->maxit);
+        stop2 = state(&ctl->stop2);
+    }
     double rr[1];
     sum_partials<1>(pc, g, rr);
     if (threadIdx.x == 0) {
-        const int o = !isfinite(rr[0]) ? kEnded : rr[0] <= stop2 ? kCheck : it >= maxit ? kEnded : kRun;
-        out = o;
-        if (blockIdx.x == 0) {
-            if (o == kCheck) ctl->halt = kCheck;
-            else if (o == kEnded) fail(ctl, isfinite(rr[0]) ? AMG_ERR_NOCONV : AMG_ERR_NAN);
-            srr = rr[0];
+        int o = halt;
+        if (o == kRun) {
+            o = !isfinite(rr[0]) ? kEnded : rr[0] <= stop2 ? kCheck : it >= maxit ? kEnded : kRun;
+            if (blockIdx.x == 0) {
+                if (o == kCheck) ctl->halt = kCheck;
+                else if (o == kEnded) fail(ctl, isfinite(rr[0]) ? AMG_ERR_NOCONV : AMG_ERR_NAN);
+            }
         }
+        out = o;
+        srr = halt == kRun ? rr[0] : -1.0;
     }
     __syncthreads();
-    if (blockIdx.x == 0 && threadIdx.x == 32) {  // off the block's way: nothing waits for it
-        const double rel = sqrt(srr) / ctl->bnorm;
+    // the history's root and quotient in a thread that nothing waits for
+    if (blockIdx.x == 0 && threadIdx.x == 32 && !(srr < 0.0)) {
+        const double rel = sqrt(srr) / state(&ctl->bnorm);
         ctl->rel = rel;
-        hist[it] = rel;
+        hist[state(&ctl->iter)] = rel;
     }
     return out;
 }
@@ -157,7 +178,8 @@ __global__ void __launch_bounds__(kBlock, SweepOcc<T, U>::kMinBlocks) k_down(
     xpre = after_wait(xpre);
     b = after_wait(b);
     ctl = after_wait(ctl);
-    if (ctl->halt) return;
+    // a kernel that takes an outcome may write the flag: it is read there
+    if (!STEP && halted(ctl)) return;
     if (STEP && step_outcome(after_wait(pc), gc, ctl, hist) != kRun) return;
     for (; i < n; i += stride) {
         T acc = R.dot(i, [&](int j) { return ldg(xpre + j); });
@@ -192,7 +214,7 @@ __global__ void __launch_bounds__(kBlock) k_down_ml(int n, const int32_t *__rest
     xpre = after_wait(xpre);
     b = after_wait(b);
     ctl = after_wait(ctl);
-    if (ctl->halt) return;
+    if (halted(ctl)) return;
     T acc = R.dot(row, [&](int j) { return ldg(xpre + j); });
     if (live && q == 0) t[row] = pi * (ldg(b + row) - acc);
 }
@@ -215,7 +237,7 @@ __global__ void __launch_bounds__(kBlock) k_post_ml(int n, const int32_t *__rest
     xp = after_wait(xp);
     b = after_wait(b);
     ctl = after_wait(ctl);
-    if (ctl->halt) return;
+    if (halted(ctl)) return;
     T acc = R.dot(row, [&](int j) { return ldg(xp + j); });
     if (live && q == 0) z[row] = ldg(xp + row) + di * (ldg(b + row) - acc);
 }
@@ -237,7 +259,7 @@ __global__ void __launch_bounds__(kBlock) k_prolong(int n, const T *__restrict__
     xpre = after_wait(xpre);
     xc = after_wait(xc);
     ctl = after_wait(ctl);
-    if (ctl->halt) return;
+    if (halted(ctl)) return;
     for (; i < n; i += stride) {
         T x = ldg(xpre + i);
         if (a >= 0) x += pw * ldg(xc + a);
@@ -272,7 +294,7 @@ __global__ void __launch_bounds__(kBlock, SweepOcc<T, U>::kMinBlocks) k_post(
     r64 = after_wait(r64);
     qold = after_wait(qold);
     ctl = after_wait(ctl);
-    if (ctl->halt) return;
+    if (halted(ctl)) return;
     double rz = 0.0, zq = 0.0;
     for (; i < n; i += stride) {
         T acc = R.dot(i, [&](int j) { return ldg(xp + j); });
@@ -318,7 +340,7 @@ __global__ void __launch_bounds__(kBlock) k_restrict(int nc, const int32_t *__re
     pdl_enter();
     t = after_wait(t);
     ctl = after_wait(ctl);
-    if (ctl->halt || I >= nc) return;
+    if (halted(ctl) || I >= nc) return;
     T tv[M];
 #pragma unroll
     for (int u = 0; u < M; u++) tv[u] = k0 + u < k1 ? ldg(t + m[u]) : T(0);
@@ -341,7 +363,7 @@ __global__ void __launch_bounds__(kBlock) k_restrict_sa(int nc, const int32_t *_
                                                         const T *__restrict__ dinvc, T *__restrict__ xprec,
                                                         const Ctl *__restrict__ ctl) {
     pdl_enter();
-    if (ctl->halt) return;
+    if (halted(ctl)) return;
     int I = blockIdx.x * blockDim.x + threadIdx.x;
     if (I >= nc) return;
     T s = 0;
@@ -357,7 +379,7 @@ __global__ void __launch_bounds__(kBlock) k_prolong_sa(int n, const int32_t *__r
                                                        const T *__restrict__ xpre, const T *__restrict__ xc,
                                                        T *__restrict__ xp, const Ctl *__restrict__ ctl) {
     pdl_enter();
-    if (ctl->halt) return;
+    if (halted(ctl)) return;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         T s = 0;
         for (int32_t q = ldg(prp + i); q < ldg(prp + i + 1); q++) s += ldg(pv + q) * ldg(xc + ldg(pci + q));
@@ -400,7 +422,7 @@ __global__ void __launch_bounds__(kBlock) k_down_restrict(int nc, const int32_t 
     xpre = after_wait(xpre);
     b = after_wait(b);
     ctl = after_wait(ctl);
-    if (ctl->halt || I >= nc) return;
+    if (halted(ctl) || I >= nc) return;
     T sum = 0;
     for (int32_t q = q0; q < q1; q++) {
         T acc = R.dot(i, [&](int j) { return ldg(xpre + j); });
@@ -441,7 +463,7 @@ __global__ void __launch_bounds__(kBlock) k_prolong_post(int n, const int32_t *_
     xc = after_wait(xc);
     b = after_wait(b);
     ctl = after_wait(ctl);
-    if (ctl->halt) return;
+    if (halted(ctl)) return;
     auto xp = [&](int j) {
         T x = ldg(xpre + j);
         int a = ldg(agg + j);
@@ -474,7 +496,7 @@ __global__ void __launch_bounds__(kBlock) k_gs_sweep(int n, int nb, const int32_
                                                      const T *__restrict__ dinv, const T *__restrict__ b,
                                                      const T *__restrict__ xo, T *xn, const Ctl *__restrict__ ctl) {
     pdl_enter();
-    if (ctl->halt) return;
+    if (halted(ctl)) return;
     int64_t lo64 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * nb;
     if (lo64 >= n) return;
     const int lo = (int)lo64, hi = (int)min((int64_t)n, lo64 + nb);
@@ -507,7 +529,7 @@ __global__ void __launch_bounds__(kBlock, Occ<T>::kMinBlocks) k_gs_offsum(
     int n, int nb, const int32_t *__restrict__ sptr, const IDX *__restrict__ col, const T *__restrict__ val,
     const T *__restrict__ xo, T *__restrict__ acc, const Ctl *__restrict__ ctl) {
     pdl_enter();
-    if (ctl->halt) return;
+    if (halted(ctl)) return;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         SELL_ROW_BEGIN
         const int lo = (i / nb) * nb, hi = min(n, lo + nb);
@@ -535,7 +557,7 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_block(int n, int nb, int w, c
                                                          const Ctl *__restrict__ ctl) {
     __shared__ T win[kGsThreads * 33];
     pdl_enter();
-    if (ctl->halt) return;
+    if (halted(ctl)) return;
     int64_t lo64 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * nb;
     if (lo64 >= n) return;
     const int lo = (int)lo64, hi = (int)min((int64_t)n, lo64 + nb);
@@ -575,7 +597,7 @@ __global__ void __launch_bounds__(kBlock, Occ<T>::kMinBlocks) k_gs_warp(
     const int32_t *__restrict__ pci, const T *__restrict__ pv, const T *__restrict__ dinv, const T *__restrict__ b,
     const T *__restrict__ xo, T *__restrict__ xn, const Ctl *__restrict__ ctl) {
     pdl_enter();
-    if (ctl->halt) return;
+    if (halted(ctl)) return;
     const int lane = threadIdx.x & 31;
     const int nsl = (n + 31) >> 5;
     const int wstride = (int)(((int64_t)gridDim.x * blockDim.x) >> 5);
@@ -652,7 +674,7 @@ __global__ void __launch_bounds__(kBlock, Occ<T>::kMinBlocks) k_gs_finish0(int n
                                                                            double *__restrict__ z, double *partials,
                                                                            Ctl *ctl) {
     pdl_enter();
-    if (ctl->halt) return;
+    if (halted(ctl)) return;
     double rz = 0.0, zq = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         double zo = (double)ldg(x + i);
@@ -672,7 +694,7 @@ __global__ void __launch_bounds__(kBlock) k_coarse(int nL, const double *__restr
                                                    const double *__restrict__ bL, TO *__restrict__ xL,
                                                    const Ctl *__restrict__ ctl) {
     pdl_enter();
-    if (ctl->halt) return;
+    if (halted(ctl)) return;
     int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (row >= nL) return;
     const double *a = ainv + (int64_t)row * nL;
@@ -691,7 +713,7 @@ __global__ void __launch_bounds__(kBlock) k_coarse_only(int n, const double *__r
                                                         const double *__restrict__ qold, double *partials,
                                                         Ctl *ctl) {
     pdl_enter();
-    if (ctl->halt) return;
+    if (halted(ctl)) return;
     double rz = 0.0, zq = 0.0;
     int lane = threadIdx.x & 31;
     int wpb = blockDim.x >> 5;
@@ -731,14 +753,19 @@ __global__ void __launch_bounds__(kVecBlock) k_axpy_p(int n, const double *__res
     pdl_enter();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int stride = gridDim.x * blockDim.x;
-    const int halt = ctl->halt, restart = ctl->restart;
-    const double pq_old = ctl->pq_old, rho_old = ctl->rho_old;
+    int halt = kRun, restart = 0;
+    double pq_old = 0.0, rho_old = 0.0;
+    if (threadIdx.x == 0) {  // read once per block: block 0 may be writing (step_outcome)
+        halt = halted(ctl);
+        restart = state(&ctl->restart);
+        pq_old = state(&ctl->pq_old);
+        rho_old = state(&ctl->rho_old);
+    }
     double zi = 0.0, pi = 0.0;
     if (i < n) {
         zi = z[i];
         pi = p[i];
     }
-    if (halt) return;
     __shared__ double sbeta;
     __shared__ bool ok;
     double sums[FCG ? 2 : 1];
@@ -746,9 +773,9 @@ __global__ void __launch_bounds__(kVecBlock) k_axpy_p(int n, const double *__res
     if (threadIdx.x == 0) {
         const double rz = sums[0], zq = FCG ? sums[FCG ? 1 : 0] : 0.0;
         const bool finite = isfinite(rz) && isfinite(zq);
-        ok = finite && rz > 0.0;
+        ok = halt == kRun && finite && rz > 0.0;
         sbeta = restart ? 0.0 : FCG ? -zq / pq_old : rz / rho_old;
-        if (blockIdx.x == 0) {
+        if (blockIdx.x == 0 && halt == kRun) {
             if (ok) {
                 ctl->rho = rz;
                 ctl->zq = zq;
@@ -783,7 +810,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_spmv(int n, const int32_t *__rest
     pdl_enter();
     p = after_wait(p);
     ctl = after_wait(ctl);
-    if (ctl->halt) return;
+    if (halted(ctl)) return;
     double pq = 0.0;
     for (; i < n; i += stride) {
         double acc = R.dot(i, [&](int j) { return ldg(p + j); });
@@ -829,9 +856,13 @@ __global__ void __launch_bounds__(kVecBlock) k_update(int n, const double *__res
     pdl_enter();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int stride = gridDim.x * blockDim.x;
-    const int halt = ctl->halt;
-    const double rho = ctl->rho;
-    const int iter = ctl->iter;
+    int halt = kRun, iter = 0;
+    double rho = 0.0;
+    if (threadIdx.x == 0) {
+        halt = halted(ctl);
+        rho = state(&ctl->rho);
+        iter = state(&ctl->iter);
+    }
     double pi = 0.0, qi = 0.0, xi = 0.0, ro = 0.0;
     if (i < n) {
         pi = p[i];
@@ -839,7 +870,6 @@ __global__ void __launch_bounds__(kVecBlock) k_update(int n, const double *__res
         xi = x[i];
         ro = r[i];
     }
-    if (halt) return;
     __shared__ double salpha;
     __shared__ bool ok;
     double sums[1];
@@ -847,9 +877,9 @@ __global__ void __launch_bounds__(kVecBlock) k_update(int n, const double *__res
     if (threadIdx.x == 0) {
         const double pq = sums[0];
         const bool finite = isfinite(pq);
-        ok = finite && pq > 0.0;
+        ok = halt == kRun && finite && pq > 0.0;
         salpha = rho / pq;
-        if (blockIdx.x == 0) {
+        if (blockIdx.x == 0 && halt == kRun) {
             if (ok) {
                 ctl->pq = pq;
                 ctl->alpha = salpha;
@@ -895,11 +925,11 @@ struct Cond {
 __device__ __forceinline__ void set_cond(const Cond &c, Ctl *ctl, bool body) {
     if (!c.set) return;
     if (body) {
-        const int b = ctl->bodies + 1;
+        const int b = state(&ctl->bodies) + 1;
         ctl->bodies = b;
-        if (!ctl->done && b > ctl->maxit + 1) fail(ctl, AMG_ERR_NOCONV);
+        if (!state(&ctl->done) && b > state(&ctl->maxit) + 1) fail(ctl, AMG_ERR_NOCONV);
     }
-    cudaGraphSetConditional(c.hc, ctl->done ? 0u : 1u);
+    cudaGraphSetConditional(c.hc, state(&ctl->done) ? 0u : 1u);
 }
 
 // r = b - A x, ||r||^2 (and ||b||^2 on INIT); also the mode's copy of r.
@@ -916,9 +946,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_residual(int n, const int32_t *__
                                                         Ctl *ctl, double *hist, Cond cond) {
     pdl_enter();
     if (!INIT) {
-        int h = ctl->halt;
-        if (h == kRun) h = step_outcome(pc, gc, ctl, hist);
-        if (h != kCheck) {
+        if (step_outcome(pc, gc, ctl, hist) != kCheck) {
             if (blockIdx.x == 0 && threadIdx.x == 0) set_cond(cond, ctl, true);
             return;
         }
@@ -942,11 +970,11 @@ __global__ void __launch_bounds__(kBlock, 4) k_residual(int n, const int32_t *__
         const double a = sums[0], bsq = sums[1];
         ctl->counter = 0;
         if (INIT) {
-            const double bn0 = sqrt(bsq), stop = ctl->rtol * bn0;
+            const double bn0 = sqrt(bsq), stop = state(&ctl->rtol) * bn0;
             ctl->bnorm = bn0;
             ctl->stop2 = stop * stop;
         }
-        const double bn = ctl->bnorm, rel = sqrt(a) / bn;
+        const double bn = state(&ctl->bnorm), rel = sqrt(a) / bn;
         if (INIT && (!isfinite(bn) || !isfinite(a))) {
             fail(ctl, AMG_ERR_NAN);
         } else if (INIT && bn == 0.0) {
@@ -958,14 +986,15 @@ __global__ void __launch_bounds__(kBlock, 4) k_residual(int n, const int32_t *__
             if (INIT) ctl->rel = rel;
             if (!isfinite(rel)) {
                 fail(ctl, AMG_ERR_NAN);
-            } else if (rel <= ctl->rtol) {
+            } else if (rel <= state(&ctl->rtol)) {
                 if (INIT) hist[0] = rel;
                 finish(ctl);
             } else {
                 ctl->restart = 1;
                 ctl->halt = kRun;
-                hist[ctl->iter] = rel;
-                if (ctl->iter >= ctl->maxit) fail(ctl, AMG_ERR_NOCONV);
+                const int it = state(&ctl->iter);
+                hist[it] = rel;
+                if (it >= state(&ctl->maxit)) fail(ctl, AMG_ERR_NOCONV);
             }
         }
         set_cond(cond, ctl, !INIT);

@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(kTThreads, 1) k_tail_smem(SmemTailPlan plan, c
     bF = after_wait(bF);
     xpreF = after_wait(xpreF);
     xF = after_wait(xF);
-    if (ctl->halt) {
+    if (__ldcg(&ctl->halt)) {
         asm volatile("cp.async.wait_all;" ::: "memory");  // no copy may outlive the block
         return;
     }

@@ -56,3 +56,25 @@ def test_non_finite_sums_end_the_solve(bad):
     b[prob.A.n - 1] = bad
     r, _ = _solve(amg, b, torch.zeros_like(b))
     assert r.status == B.ERR_NAN
+
+
+def test_outcomes_do_not_depend_on_when_blocks_start():
+    """Branches of a batch delay one another's blocks, so a block may start
+    after the one that records an iteration's outcome: every repetition still
+    equals the systems' own solves bit for bit."""
+    probs = [W.make_problem(N, 1.04, seed=60 + N) for N in (61, 44, 38, 31, 29, 45, 52)]
+    amgs = [B.AMG.from_csr(p.A, mode="fcg32") for p in probs]
+    bs = [torch.from_numpy(p.b).cuda() for p in probs]
+    alone = []
+    for a, b in zip(amgs, bs):
+        r, y = _solve(a, b, torch.zeros_like(b))
+        assert r.status == 0
+        alone.append((r.iters, y))
+    batch = B.Batch(amgs)
+    for _ in range(12):
+        xs = [torch.zeros_like(b) for b in bs]
+        st, it, _ = batch.solve(bs, xs)
+        assert st == 0
+        for k, (iters, y) in enumerate(alone):
+            assert it[k] == iters and torch.equal(xs[k], y), k
+    batch.close()
