@@ -18,6 +18,7 @@ constexpr int kBlock = 256;       // threads per block of the streaming kernels
 constexpr int kDenseMax = 4096;   // largest coarsest level solved densely
 constexpr int kCoarseBlock = 32;  // rows per block-Jacobi block of the iterative coarsest solve
 constexpr int kMaxPass = 8;
+constexpr int kSmallRows = 65536; // levels up to this many rows wait for latency rather than bandwidth
 
 // ------------------------------------------------------------------ errors
 void set_error(const char *fmt, ...);
@@ -150,6 +151,13 @@ struct Level {
     float *p32 = nullptr;
     int32_t *rptr = nullptr;  // members of each coarse row: rptr[nc+1], ridx[...]
     int32_t *ridx = nullptr;
+    // rows in the order of the coarse rows they restrict to (down sweeps that
+    // restrict in the same launch): mslot positions per coarse row (a power
+    // of two), its members in increasing order, -1 pads; then, from position
+    // mmain (a multiple of 32) to mpos, the rows left out of the coarse space.
+    // mslot = 0: the level restricts and prolongs in launches of their own.
+    int mslot = 0, mmain = 0, mpos = 0;
+    int32_t *mrow = nullptr;
     float *v32csr = nullptr;  // float32 copy of A.v (CSR order), for the Gauss-Seidel sweeps
     // smoothed aggregation (amg_params.smoothed): the explicit prolongator P
     // (n_l x n_{l+1}, columns sorted) and its transpose Pt (rows of each
@@ -305,7 +313,14 @@ struct amg_hier {
     int smoothed = 0;         // smoothed-aggregation prolongators (amg_params.smoothed)
     pcgamg::CoarseIter cit;
     pcgamg::CoarseWS cws;
-    double *bL = nullptr;     // coarsest right-hand side in float64
+    double *bL = nullptr;     // right-hand side of the directly solved level in float64
+    // The V-cycle from level op_first down as one explicit matrix (a fixed
+    // linear operator with the dense coarsest solve), row-major float64:
+    // op[l] for l = op_first..L-1, and the coarsest inverse itself at L.
+    // op_first = 0: none (iterative coarsest solve, or no room under the budget).
+    int op_first = 0;
+    std::vector<double *> op;
+    size_t col_bytes = 0;     // device bytes given back by dropping int32 columns beside int16 ones
     // Krylov workspace (level-0 length)
     double *b = nullptr, *x = nullptr, *r = nullptr, *z = nullptr, *q = nullptr, *p = nullptr;
     float *r32 = nullptr;        // float32 copy of r read by the float32 V-cycle
@@ -316,6 +331,7 @@ struct amg_hier {
     pcgamg::Ctl *ctl_host = nullptr;  // pinned mirror
     int nblk = 0;                // largest level-0 grid (sizes the partial sums)
     int grid32 = 0, grid64 = 0, gridp = 0;  // one wave of the float32 sweeps, float64 sweeps, prolongation
+    int block0 = 0;                         // threads per block of the level-0 matrix kernels
     int gridv = 0, blockv = 0;              // vector kernels
     int wave[2][2][2] = {};      // blocks in one wave: [float, double][down, post][4- or 16-entry chunks]
     double last_true_rel = 0.0;
@@ -352,6 +368,7 @@ struct amg_hier {
     int gs_fused = 1;  // one-launch warp sweeps where the blocks fit the slices (PCGAMG_GS_FUSED=0: off)
     double refresh_ms = 0;  // host time of the last amg_refresh
     int use_graph = 1;
+    int fuse = 1;  // transfers inside the sweeps (PCGAMG_TAIL=0: every sweep and transfer its own launch)
     int no_col16 = 0;
     int no_uniform = 0;  // PCGAMG_UNIFORM=0: no shared offset patterns on level 0
     int pdl = 1;  // programmatic dependent launch between solve kernels
@@ -376,6 +393,8 @@ int refresh_impl(amg_hier *h, const amg_csr *A, cudaStream_t s);
 int set_smoother_impl(amg_hier *h, int nu, int nblocks, cudaStream_t s);
 int gs_rows(int n, int nblocks);
 int fill_gs_parts(Level &lv, int nblocks, cudaStream_t s);
+int ops_alloc(amg_hier *h);
+int ops_build(amg_hier *h, int nu, int nblocks, cudaStream_t s);
 int refresh_smem_tail(amg_hier *h);
 int solve_impl(amg_hier *h, const double *b, double *x, double rtol, int maxit, int *iters,
                double *res_hist, cudaStream_t s);

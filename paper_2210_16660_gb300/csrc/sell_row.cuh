@@ -15,7 +15,9 @@ namespace pcgamg {
 // U = 16 so a row's loads take about two dependent round trips.
 constexpr int kUnroll = 4;
 constexpr int kUnrollSmall = 16;
-constexpr int kSmallRows = 65536;
+// Coarse-level sweeps whose rows are read whole: one chunk holds a row of up
+// to 28 entries (most rows of a Galerkin level of a 27-point operator).
+constexpr int kWholeRow = 28;
 
 // Loads of the matrix stream: level-0 sweeps use evict-first loads (the
 // matrix is read once per sweep and is larger than L2), coarser levels keep
@@ -316,7 +318,75 @@ struct MlRow {
     }
 };
 
+// Rows read whole (one thread per row of a small level): load() takes the
+// columns and values of the first kWholeRow entries before the wait, and
+// dot() gathers x for all of them at once, so a row costs one round trip to
+// L2 and not one per chunk; a longer row goes on chunk by chunk. Entries are
+// summed one by one in storage order.
+template <bool STREAM, typename IDX, typename T>
+struct WholeRow {
+    const IDX *c;
+    const T *a;
+    int w, cs, rb;
+    int j[kWholeRow];
+    T v[kWholeRow];
+
+    __device__ __forceinline__ void chunk(int k, int row) {
+#pragma unroll
+        for (int u = 0; u < kWholeRow; u++) {
+            if (k + u < w) {
+                j[u] = rb + (int)ld_mat<STREAM>(c + cs * (k + u));
+                v[u] = ld_mat<STREAM>(a + 32 * (k + u));
+            } else {
+                j[u] = row;
+                v[u] = T(0);
+            }
+        }
+    }
+
+    __device__ __forceinline__ void load(const int32_t *__restrict__ sptr, const IDX *__restrict__ col,
+                                         const T *__restrict__ val, int row,
+                                         const IDX *__restrict__ upat = nullptr) {
+        const int s = row >> 5, lane = row & 31;
+        const int32_t base = __ldg(sptr + s);
+        w = (__ldg(sptr + s + 1) - base) >> 5;
+        a = val + base + lane;
+        c = col + base + lane;
+        cs = 32;
+        rb = col_base<IDX>(row);
+        if (upat && __ldg(upat + (base >> 5)) != kNoPattern<IDX>) {
+            c = upat + (base >> 5);
+            cs = 1;
+            rb = row;
+        }
+        chunk(0, row);
+    }
+
+    template <typename F>
+    __device__ __forceinline__ T dot(int row, F xval) {
+        T acc = 0;
+        for (int k = 0;;) {
+            T x[kWholeRow];
+#pragma unroll
+            for (int u = 0; u < kWholeRow; u++) x[u] = k + u < w ? xval(j[u]) : T(0);
+#pragma unroll
+            for (int u = 0; u < kWholeRow; u++)
+                if (k + u < w) acc += v[u] * x[u];
+            k += kWholeRow;
+            if (k >= w) break;
+            chunk(k, row);
+        }
+        return acc;
+    }
+};
+
 template <int U, bool STREAM, typename IDX, typename T>
-using RowOf = typename std::conditional<U == kPatRow, PatRow<STREAM, IDX, T>, SellRow<U, STREAM, IDX, T>>::type;
+struct RowKind { using type = SellRow<U, STREAM, IDX, T>; };
+template <bool STREAM, typename IDX, typename T>
+struct RowKind<kPatRow, STREAM, IDX, T> { using type = PatRow<STREAM, IDX, T>; };
+template <bool STREAM, typename IDX, typename T>
+struct RowKind<kWholeRow, STREAM, IDX, T> { using type = WholeRow<STREAM, IDX, T>; };
+template <int U, bool STREAM, typename IDX, typename T>
+using RowOf = typename RowKind<U, STREAM, IDX, T>::type;
 
 }  // namespace pcgamg

@@ -568,6 +568,27 @@ __global__ void k_fill_members(int n, const int32_t *__restrict__ agg, const int
     ridx[rptr[a] + pos] = i;
 }
 
+__global__ void k_max_members(int nc, const int32_t *__restrict__ rptr, int *most) {
+    int I = blockIdx.x * blockDim.x + threadIdx.x;
+    if (I < nc) atomicMax(most, rptr[I + 1] - rptr[I]);
+}
+
+// Positions of the member order: slot of them per coarse row, -1 past its
+// members (and past the last coarse row).
+__global__ void k_member_rows(int nc, int slot, int npos, const int32_t *__restrict__ rptr,
+                              const int32_t *__restrict__ ridx, int32_t *__restrict__ mrow) {
+    int pos = blockIdx.x * blockDim.x + threadIdx.x;
+    if (pos >= npos) return;
+    int I = pos / slot, k = pos % slot;
+    mrow[pos] = I < nc && rptr[I] + k < rptr[I + 1] ? ridx[rptr[I] + k] : -1;
+}
+
+// The rows left out of the coarse space, in any order (each is copied alone).
+__global__ void k_left_out(int n, const int32_t *__restrict__ agg, int32_t *__restrict__ out, int *cur) {
+    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n && agg[i] < 0) out[atomicAdd(cur, 1)] = i;
+}
+
 __global__ void k_sort_members(int nc, const int32_t *__restrict__ rptr, int32_t *__restrict__ ridx) {
     int I = blockIdx.x * blockDim.x + threadIdx.x;
     if (I >= nc) return;
@@ -928,6 +949,42 @@ int pairwise_pass(amg_hier *h, const DevCSR &cur, const double *w, int32_t **agg
     return AMG_OK;
 }
 
+// Rows in member order (Level::mrow) on the levels that wait for latency (up
+// to kSmallRows rows), where a launch and its round trips to L2 cost more than
+// the sweep's scattered rows. On larger levels they cost more than they save:
+// in member order the down sweep of 2,097,152 rows took 86 us (57 in row order
+// and 7 for the restriction), and 520,192 rows 31.6 us (26.1 and 4.4). The
+// largest aggregate has to fit a warp.
+int member_order(amg_hier *h, Level &lv, int members, cudaStream_t s) {
+    Mem &M = h->mem;
+    const int n = lv.A.n, nc = lv.nc;
+    lv.mslot = 0;
+    if (h->smoothed || n > kSmallRows) return AMG_OK;
+    int *dmax = nullptr;
+    PCG_TRY(alloc(M, &dmax, 2));
+    PCG_CK(cudaMemsetAsync(dmax, 0, 2 * sizeof(int), s));
+    k_max_members<<<grid_for(nc), kBlock, 0, s>>>(nc, lv.rptr, dmax);
+    PCG_LAUNCH_CK();
+    int most = 0;
+    PCG_TRY(read_flag(dmax, s, &most));
+    int slot = 1;
+    while (slot < most) slot <<= 1;
+    const int64_t want = (int64_t)slot * nc;
+    if (slot <= 32) {
+        lv.mslot = slot;
+        lv.mmain = (int)((want + 31) / 32 * 32);
+        lv.mpos = lv.mmain + (n - members + 31) / 32 * 32;
+        PCG_TRY(alloc(M, &lv.mrow, lv.mpos));
+        h->col_bytes -= std::min(h->col_bytes, sizeof(int32_t) * (size_t)lv.mpos);
+        k_member_rows<<<grid_for(lv.mpos), kBlock, 0, s>>>(nc, slot, lv.mpos, lv.rptr, lv.ridx, lv.mrow);
+        k_left_out<<<grid_for(n), kBlock, 0, s>>>(n, lv.agg, lv.mrow + lv.mmain, dmax + 1);
+        PCG_LAUNCH_CK();
+    }
+    PCG_CK(cudaStreamSynchronize(s));
+    release(M, dmax);
+    return AMG_OK;
+}
+
 int finish_level(amg_hier *h, Level &lv, bool coarsest, cudaStream_t s) {
     Mem &M = h->mem;
     int n = lv.A.n;
@@ -1020,6 +1077,12 @@ int finish_level(amg_hier *h, Level &lv, bool coarsest, cudaStream_t s) {
             }
         }
     }
+    // every kernel of a level with 16-bit offsets reads those
+    if (S.col16) {
+        PCG_CK(cudaStreamSynchronize(s));
+        release(M, S.col);
+        h->col_bytes += sizeof(int32_t) * (size_t)tot;
+    }
     // work vectors
     PCG_TRY(alloc(M, &lv.b64, n));
     PCG_TRY(alloc(M, &lv.x64, n));
@@ -1054,6 +1117,8 @@ int finish_level(amg_hier *h, Level &lv, bool coarsest, cudaStream_t s) {
         PCG_TRY(alloc(M, &lv.ridx, nm));
         k_fill_members<<<grid_for(n), kBlock, 0, s>>>(n, lv.agg, lv.rptr, cur, lv.ridx);
         k_sort_members<<<grid_for(lv.nc), kBlock, 0, s>>>(lv.nc, lv.rptr, lv.ridx);
+        PCG_LAUNCH_CK();
+        PCG_TRY(member_order(h, lv, (int)nm, s));
         PCG_LAUNCH_CK();
         PCG_CK(cudaStreamSynchronize(s));
         release(M, cnt);
@@ -1261,6 +1326,7 @@ int setup_impl(amg_hier *h, const amg_csr *A, const amg_params *prm, cudaStream_
     PCG_CK(cudaStreamSynchronize(s));
     release(M, ad);
     PCG_TRY(alloc_solve_workspace(h));
+    PCG_TRY(ops_build(h, 0, 0, s));
     PCG_CK(cudaStreamSynchronize(s));
     h->setup_ms[0] = now_ms() - t_begin;
     h->setup_ms[1] = t_match;
@@ -1455,6 +1521,8 @@ int refresh_impl(amg_hier *h, const amg_csr *A, cudaStream_t s) {
     PCG_CK(cudaStreamSynchronize(s));
     release(M, ad);
     PCG_TRY(refresh_smem_tail(h));
+    PCG_TRY(ops_build(h, h->gs_nu, h->gs_blocks, s));
+    PCG_CK(cudaStreamSynchronize(s));
     h->invalid = 0;
     h->refresh_ms = now_ms() - t_begin;
     return AMG_OK;
@@ -1553,6 +1621,8 @@ int set_smoother_impl(amg_hier *h, int nu, int nblocks, cudaStream_t s) {
     // the cluster tail's shared-memory image holds the small levels' D^-1:
     // form it again from the diagonals now in place (used while nu = 0)
     PCG_TRY(refresh_smem_tail(h));
+    PCG_TRY(ops_build(h, nu, nblocks, s));
+    PCG_CK(cudaStreamSynchronize(s));
     h->gs_nu = nu;
     h->gs_blocks = nu > 0 ? nblocks : 0;
     return AMG_OK;

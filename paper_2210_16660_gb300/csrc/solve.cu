@@ -50,6 +50,11 @@ constexpr int kVecBlock = 1024;  // largest block of the vector kernels (k_axpy_
 template <typename T>
 __device__ __forceinline__ T ldg(const T *p) { return __ldg(p); }
 
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+
 // As write_partials, and true in every thread of the last block to finish,
 // after which all partials are complete: for the true residual, whose outcome
 // decides whether the loop goes on.
@@ -147,6 +152,7 @@ struct Occ { static constexpr int kMinBlocks = sizeof(T) == 4 ? 6 : 4; };
 template <typename T, int U>
 struct SweepOcc {
     static constexpr int kMinBlocks = U <= 4 ? Occ<T>::kMinBlocks
+                                      : U == kWholeRow ? 1
                                       : U == kPatRow ? (sizeof(T) == 4 ? 3 : 1)
                                                      : (sizeof(T) == 4 ? 2 : 1);
 };
@@ -179,15 +185,98 @@ __global__ void __launch_bounds__(kBlock, SweepOcc<T, U>::kMinBlocks) k_down(
     b = after_wait(b);
     ctl = after_wait(ctl);
     // a kernel that takes an outcome may write the flag: it is read there
-    if (!STEP && halted(ctl)) return;
+    const int halt = STEP ? 0 : halted(ctl);
+    if (U != kWholeRow && halt) return;
     if (STEP && step_outcome(after_wait(pc), gc, ctl, hist) != kRun) return;
     for (; i < n; i += stride) {
+        const T bi = ldg(b + i);
         T acc = R.dot(i, [&](int j) { return ldg(xpre + j); });
-        t[i] = pi * (ldg(b + i) - acc);
+        if (U == kWholeRow && halt) return;
+        t[i] = pi * (bi - acc);
         if (i + stride < n) {
             R.load(sptr, col, val, i + stride, upat);
             pi = ldg(p + i + stride);
         }
+    }
+}
+
+// Down sweep and the restriction it feeds in one launch: thread <-> position of
+// the member order (Level::mrow), so the members of a coarse row are slot
+// consecutive lanes. t_i = p_i (b_i - sum_j a_ij xpre_j) as in k_down, then
+// the slot's lanes are added in member order by shuffles to b_c and
+// (dinvc given) xpre_c = dinv_c b_c; t is never stored. Rows left out of the
+// coarse space take xp = xpre, for the prolongation by the coarser level's
+// kernel (Up). Same values as k_down followed by k_restrict.
+template <typename T, typename TO, typename IDX>
+struct DownR {
+    const int32_t *mrow;
+    int npos, nmain, lg;  // positions, positions of members, log2 of the slot
+    const int32_t *sptr;
+    const IDX *col;
+    const T *val;
+    const IDX *upat;
+    const T *xpre, *b, *p;
+    TO *bc;
+    const T *dinvc;
+    T *xprec, *xp;
+    const double *pc;
+    int gc;
+    Ctl *ctl;
+    double *hist;
+};
+
+template <typename T, typename TO, typename IDX, int U, bool STREAM, bool STEP>
+__global__ void __launch_bounds__(kBlock, SweepOcc<T, U>::kMinBlocks) k_down_r(DownR<T, TO, IDX> a) {
+    int pos = blockIdx.x * blockDim.x + threadIdx.x;
+    const int stride = gridDim.x * blockDim.x;
+    const int slot = 1 << a.lg;
+    RowOf<U, STREAM, IDX, T> R;
+    int row = -1, next = -1;
+    T pi = 0, dc = 0;
+    auto fetch = [&](int q) {  // static data of position q, whose row is `row`
+        if (row >= 0 && q < a.nmain) {
+            R.load(a.sptr, a.col, a.val, row, a.upat);
+            pi = ldg(a.p + row);
+            if (a.dinvc && (q & (slot - 1)) == 0) dc = ldg(a.dinvc + (q >> a.lg));
+        }
+    };
+    if (pos < a.npos) {
+        row = ldg(a.mrow + pos);
+        fetch(pos);
+    }
+    pdl_enter();
+    const T *xpre = after_wait(a.xpre), *b = after_wait(a.b);
+    Ctl *ctl = after_wait(a.ctl);
+    const int halt = STEP ? 0 : halted(ctl);
+    if (U != kWholeRow && halt) return;
+    if (STEP && step_outcome(after_wait(a.pc), a.gc, ctl, a.hist) != kRun) return;
+    for (; pos < a.npos; pos += stride) {  // npos and nmain are multiples of 32: a warp stays whole
+        if (pos + stride < a.npos) next = ldg(a.mrow + pos + stride);
+        if (pos >= a.nmain) {
+            if (row >= 0) {
+                const T x = ldg(xpre + row);
+                if (U == kWholeRow && halt) return;
+                a.xp[row] = x;
+            }
+        } else {
+            T t = 0;
+            if (row >= 0) {
+                const T bi = ldg(b + row);
+                const T acc = R.dot(row, [&](int j) { return ldg(xpre + j); });
+                // rounded product (never contracted into the sum), as k_down stores t
+                t = mul_rn(pi, bi - acc);
+            }
+            T sum = T(0) + t;
+            for (int u = 1; u < slot; u++) sum += __shfl_down_sync(0xffffffffu, t, u);
+            if (U == kWholeRow && halt) return;
+            if (row >= 0 && (pos & (slot - 1)) == 0) {
+                const int I = pos >> a.lg;
+                a.bc[I] = (TO)sum;
+                if (a.dinvc) a.xprec[I] = dc * sum;
+            }
+        }
+        row = next;
+        if (pos + stride < a.npos) fetch(pos + stride);
     }
 }
 
@@ -262,7 +351,7 @@ __global__ void __launch_bounds__(kBlock) k_prolong(int n, const T *__restrict__
     if (halted(ctl)) return;
     for (; i < n; i += stride) {
         T x = ldg(xpre + i);
-        if (a >= 0) x += pw * ldg(xc + a);
+        if (a >= 0) x = fma_rn(pw, ldg(xc + a), x);
         xp[i] = x;
         if (i + stride < n) {
             a = ldg(agg + i + stride);
@@ -271,22 +360,70 @@ __global__ void __launch_bounds__(kBlock) k_prolong(int n, const T *__restrict__
     }
 }
 
-// Post-smooth z_i = xp_i + dinv_i (b_i - sum_j a_ij xp_j). On level 0 (DOT)
+// Prolongation to the finer level by the kernel that forms x: coarse row I's
+// members are mrow[slot I ..] of that level (see Level::mrow), and
+// xp_m = xpre_m + p_m x_I for each (the rows left out of the coarse space take
+// xp = xpre from that level's down sweep). The first four members and their
+// weights are static and loaded before the wait, their xpre with the gathers.
+template <typename T>
+struct Up {
+    const int32_t *mrow;
+    int slot;
+    const T *p;
+    const T *xpre;
+    T *xp;
+};
+
+template <typename T>
+struct UpRow {
+    int m[4];
+    T p[4], x[4];
+    __device__ __forceinline__ void load(const Up<T> &u, int I) {
+        const int32_t *src = u.mrow + (int64_t)u.slot * I;
+        if (u.slot >= 4) {
+            const int4 q = __ldg(reinterpret_cast<const int4 *>(src));
+            m[0] = q.x; m[1] = q.y; m[2] = q.z; m[3] = q.w;
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; k++) m[k] = k < u.slot ? ldg(src + k) : -1;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; k++) p[k] = m[k] >= 0 ? ldg(u.p + m[k]) : T(0);
+    }
+    __device__ __forceinline__ void gather(const Up<T> &u) {
+#pragma unroll
+        for (int k = 0; k < 4; k++) x[k] = m[k] >= 0 ? ldg(u.xpre + m[k]) : T(0);
+    }
+    __device__ __forceinline__ void store(const Up<T> &u, int I, T xc) const {
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+            if (m[k] >= 0) u.xp[m[k]] = fma_rn(p[k], xc, x[k]);
+        for (int k = 4; k < u.slot; k++) {
+            const int q = ldg(u.mrow + (int64_t)u.slot * I + k);
+            if (q >= 0) u.xp[q] = fma_rn(ldg(u.p + q), xc, ldg(u.xpre + q));
+        }
+    }
+};
+
+// Post-smooth z_i = xp_i + dinv_i (b_i - sum_j a_ij xp_j); UP also prolongs
+// z to the next finer level. On level 0 (DOT)
 // z is written in float64 and the kernel also leaves partial sums of r.z
 // (float64 r) and, for FCG(1), z.q_old for k_axpy_p.
-template <typename T, typename TZ, bool DOT, bool FCG, typename IDX, int U, bool STREAM>
+template <typename T, typename TZ, bool DOT, bool FCG, typename IDX, int U, bool STREAM, bool UP>
 __global__ void __launch_bounds__(kBlock, SweepOcc<T, U>::kMinBlocks) k_post(
     int n, const int32_t *__restrict__ sptr, const IDX *__restrict__ col, const T *__restrict__ val,
     const IDX *__restrict__ upat, const T *__restrict__ xp, const T *__restrict__ b,
     const T *__restrict__ dinv, TZ *__restrict__ z, const double *__restrict__ r64,
-    const double *__restrict__ qold, double *partials, Ctl *ctl) {
+    const double *__restrict__ qold, double *partials, const Ctl *ctl, Up<T> up) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int stride = gridDim.x * blockDim.x;
     RowOf<U, STREAM, IDX, T> R;
+    UpRow<T> ur;
     T di = 0;
     if (i < n) {
         R.load(sptr, col, val, i, upat);
         di = ldg(dinv + i);
+        if (UP) ur.load(up, i);
     }
     pdl_enter();
     xp = after_wait(xp);
@@ -294,12 +431,19 @@ __global__ void __launch_bounds__(kBlock, SweepOcc<T, U>::kMinBlocks) k_post(
     r64 = after_wait(r64);
     qold = after_wait(qold);
     ctl = after_wait(ctl);
-    if (halted(ctl)) return;
+    up.xpre = after_wait(up.xpre);
+    // a whole row's gathers do not wait for the flag: it is read beside them
+    const int halt = halted(ctl);
+    if (U != kWholeRow && halt) return;
     double rz = 0.0, zq = 0.0;
     for (; i < n; i += stride) {
+        if (UP) ur.gather(up);
+        const T bi = ldg(b + i), xi = ldg(xp + i);
         T acc = R.dot(i, [&](int j) { return ldg(xp + j); });
-        TZ zo = (TZ)(ldg(xp + i) + di * (ldg(b + i) - acc));
+        if (U == kWholeRow && halt) return;
+        TZ zo = (TZ)(xi + di * (bi - acc));
         z[i] = zo;
+        if (UP) ur.store(up, i, (T)zo);
         if (DOT) {
             rz += ldg(r64 + i) * (double)zo;
             if (FCG) zq += (double)zo * ldg(qold + i);
@@ -307,6 +451,7 @@ __global__ void __launch_bounds__(kBlock, SweepOcc<T, U>::kMinBlocks) k_post(
         if (i + stride < n) {
             R.load(sptr, col, val, i + stride, upat);
             di = ldg(dinv + i + stride);
+            if (UP) ur.load(up, i + stride);
         }
     }
     if (DOT) {
@@ -387,9 +532,6 @@ __global__ void __launch_bounds__(kBlock) k_prolong_sa(int n, const int32_t *__r
     }
 }
 
-__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
-
 // Down sweep fused with the restriction it feeds, one thread per coarse row
 // I: t_i = p_i (b_i - sum_j a_ij xpre_j) for each member i of aggregate I
 // (members in increasing index order), summed into b_c[I] (and, with PRE,
@@ -467,7 +609,7 @@ __global__ void __launch_bounds__(kBlock) k_prolong_post(int n, const int32_t *_
     auto xp = [&](int j) {
         T x = ldg(xpre + j);
         int a = ldg(agg + j);
-        if (a >= 0) x += ldg(p + j) * ldg(xc + a);
+        if (a >= 0) x = fma_rn(ldg(p + j), ldg(xc + a), x);
         return x;
     };
     for (; i < n; i += stride) {
@@ -689,20 +831,80 @@ __global__ void __launch_bounds__(kBlock, Occ<T>::kMinBlocks) k_gs_finish0(int n
 }
 
 // x_L = A_L^{-1} b_L, one warp per row; TO = float rounds the float64 result.
-template <typename TO>
+// UP also prolongs x_L to the next finer level.
+template <typename TO, bool UP>
 __global__ void __launch_bounds__(kBlock) k_coarse(int nL, const double *__restrict__ ainv,
                                                    const double *__restrict__ bL, TO *__restrict__ xL,
-                                                   const Ctl *__restrict__ ctl) {
-    pdl_enter();
-    if (halted(ctl)) return;
+                                                   const Ctl *__restrict__ ctl, Up<TO> up) {
     int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    UpRow<TO> ur;
+    if (UP && row < nL && lane == 0) ur.load(up, row);
+    pdl_enter();
+    ctl = after_wait(ctl);
+    bL = after_wait(bL);
+    up.xpre = after_wait(up.xpre);
+    if (halted(ctl)) return;
     if (row >= nL) return;
     const double *a = ainv + (int64_t)row * nL;
+    if (UP && lane == 0) ur.gather(up);
     double s = 0.0;
     for (int j = lane; j < nL; j += 32) s += ldg(a + j) * ldg(bL + j);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) xL[row] = (TO)s;
+    if (lane == 0) {
+        xL[row] = (TO)s;
+        if (UP) ur.store(up, row, (TO)s);
+    }
+}
+
+// x = B b on the directly solved level (B: op[op_first], or the coarsest
+// inverse), float64; TO = float rounds the result. W warps share a row, a lane
+// takes entries lane, lane + 32 W, ... (kOpAhead of them at most: rows of up
+// to 512 W entries), all loaded before the wait since B is static, so after it
+// the product costs the load of b, the FMAs and the sums. Bound: the float64
+// pipe, n^2 FMAs (1,036 rows: 1.7 us).
+constexpr int kOpAhead = 16;
+template <typename TO, bool UP, int W>
+__global__ void __launch_bounds__(kBlock) k_op(int n, const double *__restrict__ B, const double *__restrict__ b,
+                                               TO *__restrict__ x, const Ctl *__restrict__ ctl, Up<TO> up) {
+    __shared__ double sh[kBlock / 32];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, wr = w % W;
+    const int row = blockIdx.x * (kBlock / 32 / W) + w / W;
+    const int j0 = 32 * wr + lane;
+    double v[kOpAhead];
+    UpRow<TO> ur;
+    if (row < n) {
+        const double *a = B + (int64_t)row * n;
+#pragma unroll
+        for (int k = 0; k < kOpAhead; k++) v[k] = j0 + 32 * W * k < n ? ldg(a + j0 + 32 * W * k) : 0.0;
+        if (UP && j0 == 0) ur.load(up, row);
+    }
+    pdl_enter();
+    b = after_wait(b);
+    ctl = after_wait(ctl);
+    up.xpre = after_wait(up.xpre);
+    const int halt = halted(ctl);
+    double s = 0.0;
+    if (row < n) {
+        double bv[kOpAhead];
+#pragma unroll
+        for (int k = 0; k < kOpAhead; k++) bv[k] = j0 + 32 * W * k < n ? ldg(b + j0 + 32 * W * k) : 0.0;
+        if (UP && j0 == 0) ur.gather(up);
+#pragma unroll
+        for (int k = 0; k < kOpAhead; k++)
+            if (32 * W * k < n) s = fma(v[k], bv[k], s);
+    }
+    s = warp_sum(s);
+    if (W > 1) {
+        if (lane == 0) sh[w] = s;
+        __syncthreads();
+        if (j0 == 0)
+            for (int q = 1; q < W; q++) s += sh[w + q];
+    }
+    if (row < n && j0 == 0 && !halt) {
+        x[row] = (TO)s;
+        if (UP) ur.store(up, row, (TO)s);
+    }
 }
 
 // Single-level hierarchy: z = A^{-1} r (through float32 as the float32
@@ -798,24 +1000,27 @@ __global__ void __launch_bounds__(kVecBlock) k_axpy_p(int n, const double *__res
 }
 
 // q = A p and the partial sums of p.q.
-template <typename IDX>
-__global__ void __launch_bounds__(kBlock, 4) k_spmv(int n, const int32_t *__restrict__ sptr,
+template <typename IDX, int U>
+__global__ void __launch_bounds__(kBlock, U == kWholeRow ? 1 : 4) k_spmv(int n, const int32_t *__restrict__ sptr,
                                                     const IDX *__restrict__ col, const double *__restrict__ val,
                                                     const IDX *__restrict__ upat, const double *__restrict__ p,
                                                     double *__restrict__ q, double *partials, const Ctl *ctl) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int stride = gridDim.x * blockDim.x;
-    SellRow<kUnroll, true, IDX, double> R;
+    RowOf<U, U != kWholeRow, IDX, double> R;
     if (i < n) R.load(sptr, col, val, i, upat);
     pdl_enter();
     p = after_wait(p);
     ctl = after_wait(ctl);
-    if (halted(ctl)) return;
+    const int halt = halted(ctl);
+    if (U != kWholeRow && halt) return;
     double pq = 0.0;
     for (; i < n; i += stride) {
+        const double pi = ldg(p + i);
         double acc = R.dot(i, [&](int j) { return ldg(p + j); });
+        if (U == kWholeRow && halt) return;
         q[i] = acc;
-        pq += ldg(p + i) * acc;
+        pq += pi * acc;
         if (i + stride < n) R.load(sptr, col, val, i + stride, upat);
     }
     double sums[1] = {pq};
@@ -1121,11 +1326,46 @@ REmit remit(amg_hier *h) {
 template <typename T>
 constexpr int prec_index() { return sizeof(T) == 4 ? 0 : 1; }
 
-int shape_grid(const amg_hier *h, int n, int pi, int sweep, unsigned char shape) {
-    int g = grid_rows(n);
-    if (shape & 2) return g;
-    int w = h->wave[pi][sweep][shape & 1];
-    return w > 0 && w < g ? w : g;
+// Sections of the partial sums, 2 h->nblk values each: what k_post left for
+// k_axpy_p, k_spmv for k_update, k_update for the next iteration's first
+// kernel or k_residual, and k_residual's own.
+inline double *parts(const amg_hier *h, int section) { return h->partials + 2 * (size_t)h->nblk * section; }
+constexpr int kPartsRz = 0, kPartsPq = 1, kPartsRr = 2, kPartsTrue = 3, kPartSections = 4;
+
+// Threads per block of a sweep with one thread per row: small levels spread
+// over the SMs (4,096 rows are 64 blocks of 64 rows, not 16 of 256).
+int small_block(int n) { return n <= 152 * 64 ? 64 : n <= 152 * 128 ? 128 : kBlock; }
+
+// Rows up to which a level's rows are read whole (WholeRow: one thread per
+// row, ~100 registers in float32); above, 16-entry chunks keep more warps
+// resident (64,512 rows: 9.9 us whole, 6.7 us in chunks).
+constexpr int kWholeRows = 32768;
+// A solve that shares the device (batches, serving lanes: no_tail) is short of
+// registers and float64 cycles rather than waiting for latency: twelve systems
+// of 24^3 to 72^3 at once ran 14.2 ms with the limits of a lone solve, 13.1
+// with these (the bits are the same).
+constexpr int kWholeRowsShared = 1024;
+constexpr int kFuseRowsShared = 16384;
+int whole_rows(const amg_hier *h) { return h->no_tail ? kWholeRowsShared : kWholeRows; }
+
+// Blocks and threads of a coarse-level sweep over n rows (or positions).
+struct Geo {
+    int grid, block;
+};
+Geo shape_geo(const amg_hier *h, int n, int pi, int sweep, unsigned char shape) {
+    const int blk = shape & 1 ? small_block(n) : kBlock;
+    const int g = (n + blk - 1) / blk;
+    if (shape & 2) return {g, blk};
+    const int w = h->wave[pi][sweep][shape & 1] * (kBlock / blk);
+    return {w > 0 && w < g ? w : g, blk};
+}
+
+// Whether level l's down sweep restricts in the same launch (member order);
+// l >= 1 only with a down shape that is not one of the older forms.
+bool down_fused(const amg_hier *h, int l, int pi) {
+    const Level &lv = h->lev[l];
+    return h->fuse && lv.mslot > 0 && !h->smoothed && !h->gs_nu && !(h->no_tail && lv.A.n > kFuseRowsShared) &&
+           (l == 0 || !(lv.shape[pi][0] & 12));
 }
 
 // Weight of the down sweep's output t = w (b - A xpre): the tentative
@@ -1164,18 +1404,25 @@ void launch_down(amg_hier *h, int l, unsigned char shape, cudaStream_t s) {
                                   P::t(lv), (const Ctl *)h->ctl)));
         return;
     }
-    int g = shape_grid(h, n, prec_index<T>(), 0, shape);
-    if (shape & 1)
-        WITH_COLS(lv.S, (launch_k(h->pdl, k_down<T, IDX, kUnrollSmall, false, false>, g, kBlock, s, n, lv.S.sptr,
+    const Geo g = shape_geo(h, n, prec_index<T>(), 0, shape);
+    if ((shape & 1) && n <= whole_rows(h))
+        WITH_COLS(lv.S, (launch_k(h->pdl, k_down<T, IDX, kWholeRow, false, false>, g.grid, g.block, s, n, lv.S.sptr,
                                   cols, P::val(lv), pats, P::xpre(lv), P::b(lv), pdown<T>(h, lv), P::t(lv),
                                   (const double *)nullptr, 0, h->ctl, (double *)nullptr)));
+    else if (shape & 1)
+        WITH_COLS(lv.S, (launch_k(h->pdl, k_down<T, IDX, kUnrollSmall, false, false>, g.grid, g.block, s, n,
+                                  lv.S.sptr, cols, P::val(lv), pats, P::xpre(lv), P::b(lv), pdown<T>(h, lv),
+                                  P::t(lv), (const double *)nullptr, 0, h->ctl, (double *)nullptr)));
     else
-        WITH_COLS(lv.S, (launch_k(h->pdl, k_down<T, IDX, kUnroll, false, false>, g, kBlock, s, n, lv.S.sptr, cols,
+        WITH_COLS(lv.S, (launch_k(h->pdl, k_down<T, IDX, kUnroll, false, false>, g.grid, g.block, s, n, lv.S.sptr, cols,
                                   P::val(lv), pats, P::xpre(lv), P::b(lv), pdown<T>(h, lv), P::t(lv),
                                   (const double *)nullptr, 0, h->ctl, (double *)nullptr)));
 }
 
-// Restriction from level l to l+1 (the coarsest gets float64 b_L).
+// The level whose right-hand side is float64: solved directly.
+inline int direct_level(const amg_hier *h) { return h->op_first ? h->op_first : (int)h->lev.size() - 1; }
+
+// Restriction from level l to l+1 (the directly solved one gets float64 b_L).
 template <typename T>
 void launch_restrict(amg_hier *h, int l, cudaStream_t s) {
     using P = LP<T>;
@@ -1183,7 +1430,7 @@ void launch_restrict(amg_hier *h, int l, cudaStream_t s) {
     Level &lv = lev[l];
     const Ctl *ctl = h->ctl;
     if (h->smoothed) {
-        if (l + 2 == (int)lev.size())
+        if (l + 1 == direct_level(h))
             launch_k(h->pdl, k_restrict_sa<T, double, false>, grid_rows(lv.nc), kBlock, s, lv.nc,
                      (const int32_t *)lv.Pt.rp, (const int32_t *)lv.Pt.ci, P::Ptv(lv), (const T *)P::t(lv), h->bL,
                      (const T *)nullptr, (T *)nullptr, ctl);
@@ -1193,7 +1440,7 @@ void launch_restrict(amg_hier *h, int l, cudaStream_t s) {
                      P::b(lev[l + 1]), P::dinv(lev[l + 1]), P::xpre(lev[l + 1]), ctl);
         return;
     }
-    if (l + 2 == (int)lev.size())
+    if (l + 1 == direct_level(h))
         launch_k(h->pdl, k_restrict<T, double, false>, grid_rows(lv.nc), kBlock, s, lv.nc, lv.rptr, lv.ridx,
                  (const T *)P::t(lv), h->bL, (const T *)nullptr, (T *)nullptr, ctl);
     else
@@ -1201,11 +1448,58 @@ void launch_restrict(amg_hier *h, int l, cudaStream_t s) {
                  (const T *)P::t(lv), P::b(lev[l + 1]), P::dinv(lev[l + 1]), P::xpre(lev[l + 1]), ctl);
 }
 
-// Down phase of level l >= 1: down sweep then restriction, or (shape bit 2)
-// both in one launch by aggregate.
+// Level `to`'s target of a prolongation by the kernel that forms x_{to+1}.
 template <typename T>
-void launch_down_phase(amg_hier *h, int l, unsigned char shape, cudaStream_t s) {
+Up<T> up_of(amg_hier *h, int to) {
     using P = LP<T>;
+    Level &lv = h->lev[to];
+    return Up<T>{lv.mrow, lv.mslot, P::p(lv), P::xpre(lv), P::xp(lv)};
+}
+
+// Down sweep of level l with its restriction in one launch (down_fused).
+template <typename T, typename TO, int U, bool STREAM, bool STEP>
+void launch_down_r(amg_hier *h, int l, const T *b, TO *bc, bool pre, Geo g, cudaStream_t s) {
+    using P = LP<T>;
+    Level &lv = h->lev[l];
+    Level &nx = h->lev[l + 1];
+    int lg = 0;
+    while ((1 << lg) < lv.mslot) lg++;
+    WITH_COLS(lv.S, (launch_k(h->pdl, k_down_r<T, TO, IDX, U, STREAM, STEP>, g.grid, g.block, s,
+                              DownR<T, TO, IDX>{lv.mrow, lv.mpos, lv.mmain, lg, lv.S.sptr, cols, P::val(lv), pats,
+                                                P::xpre(lv), b, P::p(lv), bc, pre ? P::dinv(nx) : nullptr,
+                                                pre ? P::xpre(nx) : nullptr, P::xp(lv),
+                                                (const double *)parts(h, kPartsRr), h->gridv, h->ctl,
+                                                h->hist})));
+}
+
+// Down phase of level l >= 1: one launch in member order where the level has
+// one (down_fused); else down sweep then restriction, or (shape bit 2) both in
+// one launch by aggregate. Adds the kernels launched to *kernels.
+template <typename T>
+void launch_down_phase(amg_hier *h, int l, unsigned char shape, cudaStream_t s, int *kernels) {
+    using P = LP<T>;
+    if (down_fused(h, l, prec_index<T>()) && !(shape & 12)) {
+        Level &lv = h->lev[l];
+        const Geo g = shape_geo(h, lv.mpos, prec_index<T>(), 0, shape);
+        const T *b = P::b(lv);
+        *kernels += 1;
+        if (l + 1 == direct_level(h)) {
+            if ((shape & 1) && lv.A.n <= whole_rows(h))
+                launch_down_r<T, double, kWholeRow, false, false>(h, l, b, h->bL, false, g, s);
+            else if (shape & 1)
+                launch_down_r<T, double, kUnrollSmall, false, false>(h, l, b, h->bL, false, g, s);
+            else launch_down_r<T, double, kUnroll, false, false>(h, l, b, h->bL, false, g, s);
+        } else {
+            T *bc = P::b(h->lev[l + 1]);
+            if ((shape & 1) && lv.A.n <= whole_rows(h))
+                launch_down_r<T, T, kWholeRow, false, false>(h, l, b, bc, true, g, s);
+            else if (shape & 1)
+                launch_down_r<T, T, kUnrollSmall, false, false>(h, l, b, bc, true, g, s);
+            else launch_down_r<T, T, kUnroll, false, false>(h, l, b, bc, true, g, s);
+        }
+        return;
+    }
+    *kernels += (shape & 4) && !h->smoothed ? 1 : 2;
     if (!(shape & 4) || h->smoothed) {
         launch_down<T>(h, l, shape, s);
         launch_restrict<T>(h, l, s);
@@ -1215,7 +1509,7 @@ void launch_down_phase(amg_hier *h, int l, unsigned char shape, cudaStream_t s) 
     Level &lv = lev[l];
     const Ctl *ctl = h->ctl;
     int g = grid_rows(lv.nc);
-    bool last = l + 2 == (int)lev.size();
+    bool last = l + 1 == direct_level(h);
 #define PCG_DR(U)                                                                                                   \
     do {                                                                                                            \
         if (last)                                                                                                   \
@@ -1232,8 +1526,9 @@ void launch_down_phase(amg_hier *h, int l, unsigned char shape, cudaStream_t s) 
 #undef PCG_DR
 }
 
-// Post sweep of level l >= 1 (z = x_l) with the given launch shape.
-template <typename T>
+// Post sweep of level l >= 1 (z = x_l) with the given launch shape; up: it
+// prolongs to level l - 1 too (not in shape 8).
+template <typename T, bool UP>
 void launch_post(amg_hier *h, int l, unsigned char shape, cudaStream_t s) {
     using P = LP<T>;
     Level &lv = h->lev[l];
@@ -1244,56 +1539,104 @@ void launch_post(amg_hier *h, int l, unsigned char shape, cudaStream_t s) {
                                   (const Ctl *)h->ctl)));
         return;
     }
-    int g = shape_grid(h, n, prec_index<T>(), 1, shape);
-    if (shape & 1)
-        WITH_COLS(lv.S, (launch_k(h->pdl, k_post<T, T, false, false, IDX, kUnrollSmall, false>, g, kBlock, s, n,
-                                  lv.S.sptr, cols, P::val(lv), pats, P::xp(lv), P::b(lv), P::dinv(lv), P::x(lv),
-                                  (const double *)nullptr, (const double *)nullptr, (double *)nullptr, h->ctl)));
+    const Up<T> up = UP ? up_of<T>(h, l - 1) : Up<T>{};
+    const Geo g = shape_geo(h, n, prec_index<T>(), 1, shape);
+    if ((shape & 1) && n <= whole_rows(h))
+        WITH_COLS(lv.S, (launch_k(h->pdl, k_post<T, T, false, false, IDX, kWholeRow, false, UP>, g.grid, g.block, s,
+                                  n, lv.S.sptr, cols, P::val(lv), pats, P::xp(lv), P::b(lv), P::dinv(lv), P::x(lv),
+                                  (const double *)nullptr, (const double *)nullptr, (double *)nullptr, h->ctl, up)));
+    else if (shape & 1)
+        WITH_COLS(lv.S, (launch_k(h->pdl, k_post<T, T, false, false, IDX, kUnrollSmall, false, UP>, g.grid, g.block,
+                                  s, n, lv.S.sptr, cols, P::val(lv), pats, P::xp(lv), P::b(lv), P::dinv(lv),
+                                  P::x(lv), (const double *)nullptr, (const double *)nullptr, (double *)nullptr,
+                                  h->ctl, up)));
     else
-        WITH_COLS(lv.S, (launch_k(h->pdl, k_post<T, T, false, false, IDX, kUnroll, false>, g, kBlock, s, n,
+        WITH_COLS(lv.S, (launch_k(h->pdl, k_post<T, T, false, false, IDX, kUnroll, false, UP>, g.grid, g.block, s, n,
                                   lv.S.sptr, cols, P::val(lv), pats, P::xp(lv), P::b(lv), P::dinv(lv), P::x(lv),
-                                  (const double *)nullptr, (const double *)nullptr, (double *)nullptr, h->ctl)));
+                                  (const double *)nullptr, (const double *)nullptr, (double *)nullptr, h->ctl, up)));
 }
 
-// Up phase of level l >= 1: prolongation then post sweep, or (shape bit 2)
-// the prolongation formed per gathered entry inside the post sweep.
+// Up phase of level l >= 1: prolongation (unless xp_ready: the kernel that
+// formed x_{l+1} has done it) then post sweep, or (shape bit 2) the
+// prolongation formed per gathered entry inside the post sweep. Returns
+// whether it has prolonged to level l - 1 as well; adds to *kernels.
 template <typename T>
-void launch_up_phase(amg_hier *h, int l, unsigned char shape, cudaStream_t s) {
+bool launch_up_phase(amg_hier *h, int l, unsigned char shape, bool xp_ready, cudaStream_t s, int *kernels) {
     using P = LP<T>;
     auto &lev = h->lev;
     Level &lv = lev[l];
     int n = lv.A.n;
     const Ctl *ctl = h->ctl;
+    *kernels += 1;
     if (!(shape & 4) || h->smoothed) {
-        launch_prolong<T>(h, l, grid_rows(n), s);
-        launch_post<T>(h, l, shape, s);
-        return;
+        if (!xp_ready) {
+            launch_prolong<T>(h, l, grid_rows(n), s);
+            *kernels += 1;
+        }
+        if (!(shape & 8) && down_fused(h, l - 1, prec_index<T>())) {
+            launch_post<T, true>(h, l, shape, s);
+            return true;
+        }
+        launch_post<T, false>(h, l, shape, s);
+        return false;
     }
-    int g = shape_grid(h, n, prec_index<T>(), 1, shape);
+    const Geo g = shape_geo(h, n, prec_index<T>(), 1, (unsigned char)(shape & 2));
     if (shape & 1)
-        WITH_COLS(lv.S, (launch_k(h->pdl, k_prolong_post<T, IDX, kUnrollSmall>, g, kBlock, s, n, lv.S.sptr, cols,
-                                  P::val(lv), (const T *)P::xpre(lv), P::p(lv), lv.agg, (const T *)P::x(lev[l + 1]),
-                                  (const T *)P::b(lv), P::dinv(lv), P::x(lv), ctl)));
+        WITH_COLS(lv.S, (launch_k(h->pdl, k_prolong_post<T, IDX, kUnrollSmall>, g.grid, g.block, s, n, lv.S.sptr,
+                                  cols, P::val(lv), (const T *)P::xpre(lv), P::p(lv), lv.agg,
+                                  (const T *)P::x(lev[l + 1]), (const T *)P::b(lv), P::dinv(lv), P::x(lv), ctl)));
     else
-        WITH_COLS(lv.S, (launch_k(h->pdl, k_prolong_post<T, IDX, kUnroll>, g, kBlock, s, n, lv.S.sptr, cols,
+        WITH_COLS(lv.S, (launch_k(h->pdl, k_prolong_post<T, IDX, kUnroll>, g.grid, g.block, s, n, lv.S.sptr, cols,
                                   P::val(lv), (const T *)P::xpre(lv), P::p(lv), lv.agg, (const T *)P::x(lev[l + 1]),
                                   (const T *)P::b(lv), P::dinv(lv), P::x(lv), ctl)));
+    return false;
 }
 
-// Coarsest solve of the single-column V-cycle: x_L = A_L^{-1} b_L with the
-// dense inverse, or the iterative solve (FCG + block-Jacobi ILU(1)). Adds
-// the kernels launched to *kernels.
+template <typename T, bool UP>
+void launch_op(amg_hier *h, int D, const Up<T> &up, cudaStream_t s) {
+    using P = LP<T>;
+    Level &ld = h->lev[D];
+    const int n = ld.A.n;
+    const double *B = h->op[D] ? h->op[D] : h->Ainv;
+#define PCG_OP(W)                                                                                                   \
+    launch_k(h->pdl, k_op<T, UP, W>, (n + kBlock / 32 / W - 1) / (kBlock / 32 / W), kBlock, s, n, B, h->bL, P::x(ld), \
+             (const Ctl *)h->ctl, up)
+    if (n <= 32 * kOpAhead) PCG_OP(1);
+    else if (n <= 64 * kOpAhead) PCG_OP(2);
+    else if (n <= 128 * kOpAhead) PCG_OP(4);
+    else PCG_OP(8);
+#undef PCG_OP
+}
+
+// The directly solved level of the single-column V-cycle: x = B b with the
+// explicit operator of the small levels, or x_L = A_L^{-1} b_L with the dense
+// inverse, or the iterative solve (FCG + block-Jacobi ILU(1)). Adds the
+// kernels launched to *kernels; *prolonged: x has been prolonged too.
 template <typename T>
-int launch_coarsest(amg_hier *h, cudaStream_t s, int *kernels) {
+int launch_direct(amg_hier *h, cudaStream_t s, int *kernels, bool *prolonged) {
     using P = LP<T>;
     Level &lc = h->lev.back();
+    const int D = direct_level(h);
+    *prolonged = false;
     if (h->coarse_iter) {
         PCG_TRY(launch_coarse_iter<T>(h, h->cws, h->bL, P::x(lc), &h->ctl->halt, nullptr, s));
         *kernels += coarse_iter_launches(h);
         return AMG_OK;
     }
-    launch_k(h->pdl, k_coarse<T>, (h->nL * 32 + kBlock - 1) / kBlock, kBlock, s, h->nL, h->Ainv, h->bL, P::x(lc),
-             (const Ctl *)h->ctl);
+    const bool up = down_fused(h, D - 1, prec_index<T>());
+    if (h->op_first) {
+        if (up) launch_op<T, true>(h, D, up_of<T>(h, D - 1), s);
+        else launch_op<T, false>(h, D, Up<T>{}, s);
+    } else {
+        const int g = (h->nL * 32 + kBlock - 1) / kBlock;
+        if (up)
+            launch_k(h->pdl, k_coarse<T, true>, g, kBlock, s, h->nL, h->Ainv, h->bL, P::x(lc), (const Ctl *)h->ctl,
+                     up_of<T>(h, D - 1));
+        else
+            launch_k(h->pdl, k_coarse<T, false>, g, kBlock, s, h->nL, h->Ainv, h->bL, P::x(lc), (const Ctl *)h->ctl,
+                     Up<T>{});
+    }
+    *prolonged = up;
     *kernels += 1;
     return AMG_OK;
 }
@@ -1306,12 +1649,6 @@ int grid0(const amg_hier *h) { return sizeof(T) == 4 ? h->grid32 : h->grid64; }
 // offset patterns (PatRow), else 4-entry chunks.
 inline bool pat_rows(const amg_hier *h) { return h->lev[0].S.upat != nullptr; }
 
-// Sections of the partial sums, 2 h->nblk values each: what k_post left for
-// k_axpy_p, k_spmv for k_update, k_update for the next iteration's first
-// kernel or k_residual, and k_residual's own.
-inline double *parts(const amg_hier *h, int section) { return h->partials + 2 * (size_t)h->nblk * section; }
-constexpr int kPartsRz = 0, kPartsPq = 1, kPartsRr = 2, kPartsTrue = 3, kPartSections = 4;
-
 // Level-0 down sweep t = p (b - A xpre) (evict-first matrix stream, shared
 // offset patterns where level 0 has them). step: it takes the outcome of the
 // iteration before it.
@@ -1320,15 +1657,26 @@ void launch_down0_t(amg_hier *h, const T *b0, cudaStream_t s) {
     using P = LP<T>;
     Level &l0 = h->lev[0];
     const double *pc = parts(h, kPartsRr);
+    if (down_fused(h, 0, prec_index<T>())) {
+        const int blk = std::min(h->block0, small_block(l0.mpos));
+        const Geo g{(l0.mpos + blk - 1) / blk, blk};
+        T *bc = P::b(h->lev[1]);
+        const bool direct = direct_level(h) == 1, whole = l0.A.n <= whole_rows(h);
+        if (direct && whole) launch_down_r<T, double, kWholeRow, false, STEP>(h, 0, b0, h->bL, false, g, s);
+        else if (direct) launch_down_r<T, double, kUnrollSmall, false, STEP>(h, 0, b0, h->bL, false, g, s);
+        else if (whole) launch_down_r<T, T, kWholeRow, false, STEP>(h, 0, b0, bc, true, g, s);
+        else launch_down_r<T, T, kUnrollSmall, false, STEP>(h, 0, b0, bc, true, g, s);
+        return;
+    }
     if constexpr (sizeof(T) == 4) {
         if (pat_rows(h)) {
-            WITH_COLS(l0.S, (launch_k(h->pdl, k_down<T, IDX, kPatRow, true, STEP>, grid0<T>(h), kBlock, s, l0.A.n,
+            WITH_COLS(l0.S, (launch_k(h->pdl, k_down<T, IDX, kPatRow, true, STEP>, grid0<T>(h), h->block0, s, l0.A.n,
                                       l0.S.sptr, cols, P::val(l0), pats, (const T *)P::xpre(l0), b0,
                                       pdown<T>(h, l0), P::t(l0), pc, h->gridv, h->ctl, h->hist)));
             return;
         }
     }
-    WITH_COLS(l0.S, (launch_k(h->pdl, k_down<T, IDX, kUnroll, true, STEP>, grid0<T>(h), kBlock, s, l0.A.n, l0.S.sptr,
+    WITH_COLS(l0.S, (launch_k(h->pdl, k_down<T, IDX, kUnroll, true, STEP>, grid0<T>(h), h->block0, s, l0.A.n, l0.S.sptr,
                               cols, P::val(l0), pats, (const T *)P::xpre(l0), b0, pdown<T>(h, l0), P::t(l0), pc,
                               h->gridv, h->ctl, h->hist)));
 }
@@ -1344,17 +1692,24 @@ template <typename T, bool FCG>
 void launch_post0(amg_hier *h, const T *b0, cudaStream_t s) {
     using P = LP<T>;
     Level &l0 = h->lev[0];
+    if (l0.A.n <= whole_rows(h)) {
+        WITH_COLS(l0.S, (launch_k(h->pdl, k_post<T, double, true, FCG, IDX, kWholeRow, false, false>, grid0<T>(h),
+                                  h->block0, s, l0.A.n, l0.S.sptr, cols, P::val(l0), pats, P::xp(l0), b0,
+                                  P::dinv(l0), h->z, h->r, h->q, parts(h, kPartsRz), h->ctl, Up<T>{})));
+        return;
+    }
     if constexpr (sizeof(T) == 4) {
         if (pat_rows(h)) {
-            WITH_COLS(l0.S, (launch_k(h->pdl, k_post<T, double, true, FCG, IDX, kPatRow, true>, grid0<T>(h), kBlock,
+            WITH_COLS(l0.S, (launch_k(h->pdl, k_post<T, double, true, FCG, IDX, kPatRow, true, false>, grid0<T>(h), h->block0,
                                       s, l0.A.n, l0.S.sptr, cols, P::val(l0), pats, P::xp(l0), b0, P::dinv(l0), h->z,
-                                      h->r, h->q, parts(h, kPartsRz), h->ctl)));
+                                      h->r, h->q, parts(h, kPartsRz), h->ctl,
+                                      Up<T>{})));
             return;
         }
     }
-    WITH_COLS(l0.S, (launch_k(h->pdl, k_post<T, double, true, FCG, IDX, kUnroll, true>, grid0<T>(h), kBlock, s,
+    WITH_COLS(l0.S, (launch_k(h->pdl, k_post<T, double, true, FCG, IDX, kUnroll, true, false>, grid0<T>(h), h->block0, s,
                                   l0.A.n, l0.S.sptr, cols, P::val(l0), pats, P::xp(l0), b0, P::dinv(l0), h->z, h->r,
-                                  h->q, parts(h, kPartsRz), h->ctl)));
+                                  h->q, parts(h, kPartsRz), h->ctl, Up<T>{})));
 }
 
 // z = B r (one V-cycle in precision T), including rho / beta. Kernels are
@@ -1363,15 +1718,15 @@ template <typename T, bool FCG>
 int launch_vcycle(amg_hier *h, bool step, cudaStream_t s) {
     using P = LP<T>;
     auto &lev = h->lev;
-    int L = (int)lev.size() - 1;
     const T *b0 = P::r0(h);
     int sp1 = prof_begin(h, 0, s);
     launch_down0<T>(h, b0, step, s);
     prof_end(h, sp1, s);
     int sp2 = prof_begin(h, 5, s);
-    // levels handled by separate launches: 0..F-1; the tail runs F..L
-    int tf = h->no_tail ? 0 : h->tail_first[prec_index<T>()];
-    int F = tf > 0 ? tf : L;
+    // levels handled by separate launches: 0..F-1; the explicit operator (or
+    // the tail, or the coarsest solve) takes F..L
+    int tf = h->no_tail || h->op_first ? 0 : h->tail_first[prec_index<T>()];
+    int F = tf > 0 ? tf : direct_level(h);
     // per-level spans (profiling only): level l's down phase is its down
     // sweep and the restriction that leaves it (level 0: the restriction)
     int kernels = 1;  // down sweep of level 0
@@ -1380,35 +1735,38 @@ int launch_vcycle(amg_hier *h, bool step, cudaStream_t s) {
         int spl = prof_begin(h, kLevelSpan + 3 * l, s);
         unsigned char sh = lv.shape[prec_index<T>()][0];
         if (l == 0) {
-            launch_restrict<T>(h, 0, s);
-            kernels += 1;
+            if (!down_fused(h, 0, prec_index<T>())) {
+                launch_restrict<T>(h, 0, s);
+                kernels += 1;
+            }
         } else {
-            launch_down_phase<T>(h, l, sh, s);
-            kernels += (sh & 4) ? 1 : 2;
+            launch_down_phase<T>(h, l, sh, s, &kernels);
         }
         prof_end(h, spl, s);
     }
     int spc = prof_begin(h, kLevelSpan + 3 * F + 2, s);
-    if (F < L) {
+    bool xp_ready = false;
+    if (tf > 0) {
         PCG_TRY(launch_smem_tail<T>(h, s));
         kernels += 1;
     } else {
-        PCG_TRY(launch_coarsest<T>(h, s, &kernels));
+        PCG_TRY(launch_direct<T>(h, s, &kernels, &xp_ready));
     }
     prof_end(h, spc, s);
     for (int l = F - 1; l >= 1; l--) {
         Level &lv = lev[l];
         int spl = prof_begin(h, kLevelSpan + 3 * l + 1, s);
-        unsigned char sh = lv.shape[prec_index<T>()][1];
-        launch_up_phase<T>(h, l, sh, s);
-        kernels += (sh & 4) ? 1 : 2;
+        xp_ready = launch_up_phase<T>(h, l, lv.shape[prec_index<T>()][1], xp_ready, s, &kernels);
         prof_end(h, spl, s);
     }
-    kernels += 2;  // prolongation and post sweep of level 0
+    kernels += 1;  // post sweep of level 0
     prof_end(h, sp2, s);
-    int sp7 = prof_begin(h, 7, s);
-    launch_prolong<T>(h, 0, h->gridp, s);
-    prof_end(h, sp7, s);
+    if (!xp_ready) {
+        int sp7 = prof_begin(h, 7, s);
+        launch_prolong<T>(h, 0, h->gridp, s);
+        prof_end(h, sp7, s);
+        kernels += 1;
+    }
     int sp3 = prof_begin(h, 1, s);
     launch_post0<T, FCG>(h, b0, s);
     prof_end(h, sp3, s);
@@ -1536,7 +1894,7 @@ template <typename T, bool FCG>
 int launch_vcycle_gs(amg_hier *h, cudaStream_t s) {
     using P = LP<T>;
     auto &lev = h->lev;
-    int L = (int)lev.size() - 1;
+    const int L = direct_level(h);  // smoothed levels: 0..L-1
     Ctl *ctl = h->ctl;
     Level &l0 = lev[0];
     const T *b0 = P::r0(h);
@@ -1556,13 +1914,13 @@ int launch_vcycle_gs(amg_hier *h, cudaStream_t s) {
             kernels += 1;
         } else {
             kernels += launch_gs<T>(h, l, true, P::b(lev[l]), P::xpre(lev[l]), s);
-            launch_down_phase<T>(h, l, sh, s);
-            kernels += (sh & 4) ? 1 : 2;
+            launch_down_phase<T>(h, l, sh, s, &kernels);
         }
         prof_end(h, spl, s);
     }
     int spc = prof_begin(h, kLevelSpan + 3 * L + 2, s);
-    PCG_TRY(launch_coarsest<T>(h, s, &kernels));
+    bool prolonged = false;
+    PCG_TRY(launch_direct<T>(h, s, &kernels, &prolonged));
     prof_end(h, spc, s);
     for (int l = L - 1; l >= 1; l--) {
         Level &lv = lev[l];
@@ -1576,7 +1934,7 @@ int launch_vcycle_gs(amg_hier *h, cudaStream_t s) {
     launch_prolong<T>(h, 0, h->gridp, s);
     kernels += 1 + launch_gs<T>(h, 0, false, b0, P::x(l0), s);
     // the post sweep's grid, so rho is summed in the same order as there
-    launch_k(pdl, k_gs_finish0<T, FCG>, grid0<T>(h), kBlock, s, l0.A.n, (const T *)P::x(l0), (const double *)h->r,
+    launch_k(pdl, k_gs_finish0<T, FCG>, grid0<T>(h), h->block0, s, l0.A.n, (const T *)P::x(l0), (const double *)h->r,
              (const double *)h->q, h->z, parts(h, kPartsRz), ctl);
     kernels += 1;
     prof_end(h, sp3, s);
@@ -1622,8 +1980,12 @@ int launch_iteration_t(amg_hier *h, bool first, bool last, const Cond &cond, cud
         launch_k(pdl, k_axpy_p<false>, h->gridv, h->blockv, s, n, h->z, h->p, parts(h, kPartsRz), ga, h->ctl);
     prof_end(h, sp4, s);
     int sp5 = prof_begin(h, 2, s);
-    WITH_COLS(l0.S, (launch_k(pdl, k_spmv<IDX>, h->grid64, kBlock, s, n, l0.S.sptr, cols, l0.S.v64, pats, h->p, h->q,
-                              parts(h, kPartsPq), h->ctl)));
+    if (n <= whole_rows(h))
+        WITH_COLS(l0.S, (launch_k(pdl, k_spmv<IDX, kWholeRow>, h->grid64, h->block0, s, n, l0.S.sptr, cols, l0.S.v64,
+                                  pats, h->p, h->q, parts(h, kPartsPq), h->ctl)));
+    else
+        WITH_COLS(l0.S, (launch_k(pdl, k_spmv<IDX, kUnroll>, h->grid64, h->block0, s, n, l0.S.sptr, cols, l0.S.v64,
+                                  pats, h->p, h->q, parts(h, kPartsPq), h->ctl)));
     prof_end(h, sp5, s);
     int sp6 = prof_begin(h, 3, s);
     launch_k(pdl, k_update<MODE>, h->gridv, h->blockv, s, n, h->p, h->q, h->x, h->r, remit(h), parts(h, kPartsPq),
@@ -1632,7 +1994,7 @@ int launch_iteration_t(amg_hier *h, bool first, bool last, const Cond &cond, cud
     h->launches += 3;
     if (last || !takes) {
         int sp7 = prof_begin(h, 4, s);
-        WITH_COLS(l0.S, (launch_k(pdl, k_residual<false, MODE, IDX>, h->grid64, kBlock, s, n, l0.S.sptr, cols,
+        WITH_COLS(l0.S, (launch_k(pdl, k_residual<false, MODE, IDX>, h->grid64, h->block0, s, n, l0.S.sptr, cols,
                                   l0.S.v64, h->b, h->x, h->r, remit(h), parts(h, kPartsRr), h->gridv,
                                   parts(h, kPartsTrue), h->ctl, h->hist, last ? cond : Cond{})));
         prof_end(h, sp7, s);
@@ -1653,11 +2015,11 @@ int launch_prefix(amg_hier *h, const Cond &cond, cudaStream_t s) {
     k_zero<<<grid_rows(n), kBlock, 0, s>>>(h->p, n);
     k_zero<<<grid_rows(n), kBlock, 0, s>>>(h->q, n);
     if (h->mode == AMG_MODE_FCG32)
-        WITH_COLS(l0.S, (launch_k(h->pdl, k_residual<true, AMG_MODE_FCG32, IDX>, h->grid64, kBlock, s, n, l0.S.sptr,
+        WITH_COLS(l0.S, (launch_k(h->pdl, k_residual<true, AMG_MODE_FCG32, IDX>, h->grid64, h->block0, s, n, l0.S.sptr,
                                   cols, l0.S.v64, h->b, h->x, h->r, remit(h), (const double *)nullptr, 0,
                                   parts(h, kPartsTrue), h->ctl, h->hist, cond)));
     else
-        WITH_COLS(l0.S, (launch_k(h->pdl, k_residual<true, AMG_MODE_PCG64, IDX>, h->grid64, kBlock, s, n, l0.S.sptr,
+        WITH_COLS(l0.S, (launch_k(h->pdl, k_residual<true, AMG_MODE_PCG64, IDX>, h->grid64, h->block0, s, n, l0.S.sptr,
                                   cols, l0.S.v64, h->b, h->x, h->r, remit(h), (const double *)nullptr, 0,
                                   parts(h, kPartsTrue), h->ctl, h->hist, cond)));
     h->launches += 3;
@@ -1711,7 +2073,7 @@ int capture_solve_prefix(amg_hier *h, int mode, cudaStream_t cs, PendingBody *pb
 // Fills the while node's body: kBodyIters iterations, the last kernel of which
 // sets the loop condition, captured on s (not capturing). Kernel count of one
 // body to *body_k.
-constexpr int kBodyIters = 2;
+constexpr int kBodyIters = 4;
 int capture_solve_body(const PendingBody &pb, cudaStream_t s, int *body_k) {
     amg_hier *h = pb.h;
     int saved_mode = h->mode;
@@ -1785,10 +2147,13 @@ bool is_device_ptr(const void *p) {
 // separately instead.
 int setup_tail(amg_hier *h) {
     h->tail_first[0] = h->tail_first[1] = 0;
-    // the tail holds a dense coarsest inverse and aggregate-map transfers
-    if (h->coarse_iter || h->smoothed) return AMG_OK;
     const char *e = getenv("PCGAMG_TAIL");
-    if (e && e[0] == '0') return AMG_OK;
+    if (e && e[0] == '0') {
+        h->fuse = 0;
+        return AMG_OK;
+    }
+    // the tail holds a dense coarsest inverse and aggregate-map transfers
+    if (h->coarse_iter || h->smoothed || h->op_first) return AMG_OK;
     return setup_smem_tail(h);
 }
 
@@ -1819,10 +2184,12 @@ int alloc_solve_workspace(amg_hier *h) {
     h->device = dev;
     // One wave of resident blocks per level-0 kernel family (grid = SMs x
     // blocks resident per SM), capped by the rows available.
+    // A mesh of less than a full block per SM takes smaller blocks, one per SM.
+    h->block0 = std::min(kBlock, std::max(64, ((n + sms - 1) / sms + 31) / 32 * 32));
     auto wave = [&](const void *fn, int *grid) -> int {
         int per = 0;
-        PCG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, kBlock, 0));
-        int64_t want = ((int64_t)n + kBlock - 1) / kBlock;
+        PCG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, h->block0, 0));
+        int64_t want = ((int64_t)n + h->block0 - 1) / h->block0;
         int64_t g = (int64_t)sms * (per > 0 ? per : 1);
         *grid = (int)(want < g ? want : g);
         if (*grid < 1) *grid = 1;
@@ -1834,14 +2201,14 @@ int alloc_solve_workspace(amg_hier *h) {
         int gd = 0, gp = 0;
         if (h->lev[0].S.col16) {
             PCG_TRY(wave((const void *)k_down<float, int16_t, kPatRow, true, true>, &gd));
-            PCG_TRY(wave((const void *)k_post<float, double, true, true, int16_t, kPatRow, true>, &gp));
+            PCG_TRY(wave((const void *)k_post<float, double, true, true, int16_t, kPatRow, true, false>, &gp));
         } else {
             PCG_TRY(wave((const void *)k_down<float, int32_t, kPatRow, true, true>, &gd));
-            PCG_TRY(wave((const void *)k_post<float, double, true, true, int32_t, kPatRow, true>, &gp));
+            PCG_TRY(wave((const void *)k_post<float, double, true, true, int32_t, kPatRow, true, false>, &gp));
         }
         h->grid32 = std::min(gd, gp);
     }
-    PCG_TRY(wave((const void *)k_spmv<int32_t>, &h->grid64));
+    PCG_TRY(wave((const void *)k_spmv<int32_t, kUnroll>, &h->grid64));
     PCG_TRY(wave((const void *)k_prolong<float>, &h->gridp));
     // the vector kernels: at most two blocks per SM (their consumers read one
     // partial per block), the block as large as the rows fill
@@ -1852,12 +2219,14 @@ int alloc_solve_workspace(amg_hier *h) {
     h->nblk = std::max(h->grid32, std::max(h->grid64, h->gridv));
     // One wave of each coarse-level sweep variant, and the fixed shape rule.
     const void *fns[2][2][2] = {
-        {{(const void *)k_down<float, int16_t, kUnroll, false, false>, (const void *)k_down<float, int16_t, kUnrollSmall, false, false>},
-         {(const void *)k_post<float, float, false, false, int16_t, kUnroll, false>,
-          (const void *)k_post<float, float, false, false, int16_t, kUnrollSmall, false>}},
-        {{(const void *)k_down<double, int16_t, kUnroll, false, false>, (const void *)k_down<double, int16_t, kUnrollSmall, false, false>},
-         {(const void *)k_post<double, double, false, false, int16_t, kUnroll, false>,
-          (const void *)k_post<double, double, false, false, int16_t, kUnrollSmall, false>}}};
+        {{(const void *)k_down_r<float, float, int16_t, kUnroll, false, false>,
+          (const void *)k_down_r<float, float, int16_t, kUnrollSmall, false, false>},
+         {(const void *)k_post<float, float, false, false, int16_t, kUnroll, false, true>,
+          (const void *)k_post<float, float, false, false, int16_t, kUnrollSmall, false, true>}},
+        {{(const void *)k_down_r<double, double, int16_t, kUnroll, false, false>,
+          (const void *)k_down_r<double, double, int16_t, kUnrollSmall, false, false>},
+         {(const void *)k_post<double, double, false, false, int16_t, kUnroll, false, true>,
+          (const void *)k_post<double, double, false, false, int16_t, kUnrollSmall, false, true>}}};
     for (int a = 0; a < 2; a++)
         for (int b = 0; b < 2; b++)
             for (int c = 0; c < 2; c++) {
@@ -1883,6 +2252,7 @@ int alloc_solve_workspace(amg_hier *h) {
     h->hist_cap = 1001;
     PCG_TRY(alloc(M, &h->hist, h->hist_cap));
     if (h->coarse_iter) PCG_TRY(cws_alloc(h, M, h->cws, 1));
+    PCG_TRY(ops_alloc(h));
     PCG_TRY(setup_tail(h));
     return AMG_OK;
 }
@@ -1902,12 +2272,12 @@ int tune_level(amg_hier *h, int l, cudaStream_t s, int reps, cudaEvent_t e0, cud
     Level &lv = h->lev[l];
     for (int sweep = 0; sweep < 2; sweep++) {
         float best = 0.0f, cur = 0.0f;
-        int pick = -1;
+        int pick = -1, kernels = 0;
         for (int shape = 0; shape < kShapes; shape++) {
             for (int r = -1; r < reps; r++) {
                 if (r == 0) PCG_CK(cudaEventRecord(e0, s));
-                if (sweep == 0) launch_down_phase<T>(h, l, (unsigned char)shape, s);
-                else launch_up_phase<T>(h, l, (unsigned char)shape, s);
+                if (sweep == 0) launch_down_phase<T>(h, l, (unsigned char)shape, s, &kernels);
+                else launch_up_phase<T>(h, l, (unsigned char)shape, down_fused(h, l, pi), s, &kernels);
             }
             PCG_CK(cudaEventRecord(e1, s));
             PCG_CK(cudaEventSynchronize(e1));
@@ -1947,7 +2317,7 @@ int autotune_impl(amg_hier *h, cudaStream_t s, int reps, int *changed) {
     cudaError_t ce = cudaEventCreate(&e0);
     if (ce == cudaSuccess) ce = cudaEventCreate(&e1);
     if (ce != cudaSuccess) st = cuda_fail(ce, "autotune events", __FILE__, __LINE__);
-    for (int l = 1; l < L && !st; l++) {
+    for (int l = 1; l < direct_level(h) && !st; l++) {
         st = tune_level<float>(h, l, s, reps, e0, e1, changed);
         if (!st) st = tune_level<double>(h, l, s, reps, e0, e1, changed);
     }

@@ -1,0 +1,84 @@
+"""Transfers inside the small levels' sweeps, and the small levels as one matrix.
+
+The down sweep that restricts in the same launch (member order) and the
+kernels that prolong the x they form give the bits of the separate launches
+(PCGAMG_TAIL=0): checked for aggregates of 2 to 64 rows (slots of 2 to 32, and
+past a warp the separate launches), ragged sizes and both column widths. The
+explicit matrix of the small levels (left out under a byte budget that has no
+room for it) is the same operator as the levels one by one, up to rounding.
+"""
+import os
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+from paper_2210_16660_gb300 import binding as B  # noqa: E402
+from paper_2210_16660_gb300 import workloads as W  # noqa: E402
+
+
+def _amg(A, env=(), **kw):
+    old = {k: os.environ.get(k) for k, _ in env}
+    os.environ.update(dict(env))
+    try:
+        return B.AMG.from_csr(A, **kw)
+    finally:
+        for k, v in old.items():
+            if v is None:
+                del os.environ[k]
+            else:
+                os.environ[k] = v
+
+
+def _solve(amg, b):
+    x = torch.zeros_like(b)
+    return amg.solve(b, x, rtol=1e-8), x
+
+
+@pytest.mark.parametrize("mode", ["pcg64", "fcg32"])
+@pytest.mark.parametrize("N,npass,cmax,env", [
+    (9, 1, 10, ()), (14, 2, 20, ()), (24, 3, 30, (("PCGAMG_COL16", "0"),)), (33, 4, 20, (("PCGAMG_UNIFORM", "0"),)),
+    (24, 5, 5, ()), (24, 6, 5, ()), (41, 2, 200, ()), (33, 1, 3000, ())])
+def test_fused_transfers_give_the_bits_of_separate_launches(N, npass, cmax, env, mode):
+    prob = W.make_problem(N, 1.04, seed=3)
+    b = torch.from_numpy(prob.b).cuda()
+    kw = dict(mode=mode, n_pass=npass, coarse_max=cmax)
+    r1, x1 = _solve(_amg(prob.A, env, **kw), b)
+    r2, x2 = _solve(_amg(prob.A, tuple(env) + (("PCGAMG_TAIL", "0"),), **kw), b)
+    assert r1.status == r2.status == 0 and r1.iters == r2.iters
+    assert np.array_equal(r1.hist, r2.hist) and torch.equal(x1, x2)
+
+
+@pytest.mark.parametrize("mode", ["pcg64", "fcg32"])
+@pytest.mark.parametrize("N,kw,nu,rows", [
+    (24, {}, 0, 1), (33, {}, 0, 1), (24, {}, 2, 5), (28, {}, 4, 32), (24, {"smoothed": True, "n_pass": 3}, 0, 1),
+    (20, {"coarse_max": 20}, 1, 1)])
+def test_small_levels_as_one_matrix(N, kw, nu, rows, mode):
+    prob = W.make_problem(N, 1.04, seed=4)
+    b = torch.from_numpy(prob.b).cuda()
+    A2 = W.rescaled(prob.A, seed=9)
+    amgs = [B.AMG.from_csr(prob.A, mode=mode, **kw), B.AMG.from_csr(prob.A, mode=mode, hbm_budget=1 << 34, **kw)]
+    for step in ("setup", "refresh"):
+        out = []
+        for a in amgs:
+            if step == "refresh":
+                a.refresh(A2)
+            elif nu:
+                a.set_smoother(nu, -(-prob.A.n // rows))
+            n0 = a.launch_count()
+            r, x = _solve(a, b)
+            assert r.status == 0, r.message
+            out.append((r, x, a.launch_count() - n0))
+        (r1, x1, n1), (r2, x2, n2) = out
+        assert abs(r1.iters - r2.iters) <= 1
+        # the two V-cycles differ by rounding alone: u = 2^-53 per operation in
+        # float64 (2^-24 in float32), a few hundred operations deep, so the
+        # residuals of the first iterations agree to 1e-10 (1e-4)
+        k = min(5, r1.iters, r2.iters)
+        assert np.allclose(r1.hist[:k], r2.hist[:k], rtol=1e-10 if mode == "pcg64" else 1e-4, atol=0)
+        assert (x1 - x2).norm().item() <= 1e-6 * x2.norm().item()
+    for a in amgs:
+        a.close()
