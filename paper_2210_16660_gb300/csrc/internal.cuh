@@ -271,7 +271,7 @@ struct MultiLevel {
 };
 
 struct MultiWS {
-    int K = 0, hist_cap = 0, grid = 0;
+    int K = 0, hist_cap = 0, grid = 0, sms = 1;
     double *b = nullptr, *x = nullptr, *r = nullptr, *z = nullptr, *p = nullptr, *q = nullptr;
     float *r32 = nullptr;
     std::vector<MultiLevel> lev;

@@ -11,12 +11,14 @@
 // residual history and status; a column that has converged or failed stops
 // changing (alpha = 0) while the others go on. Same V-cycle structure and
 // reading of the method as the single right-hand-side path.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <vector>
 
 #include "internal.cuh"
+#include "reduce.cuh"
 #include "sell_row.cuh"
 
 namespace pcgamg {
@@ -70,7 +72,9 @@ __device__ __forceinline__ void st_vec(T *p, const T (&o)[V]) {
 }
 
 // acc[v] += sum_k a_k x(j_k)[v] over one sliced-ELL row, entries in storage
-// order; U entries' columns and values are loaded before their gathers.
+// order; U entries' columns and values are loaded before their gathers (level
+// 0, Gauss-Seidel: a second chunk in flight costs more in registers than it
+// gains there).
 template <int U, bool STREAM, int V, typename IDX, typename T, typename F>
 __device__ __forceinline__ void sell_row_vec(const IDX *__restrict__ c, const T *__restrict__ a, int w, int row,
                                              F xvec, T (&acc)[V]) {
@@ -113,12 +117,24 @@ __device__ __forceinline__ void sell_row_vec(const IDX *__restrict__ c, const T 
     int c0 = (int)(g_ % (K / (V))) * (V);                                                     \
     int64_t e0 = (int64_t)i * K + c0;
 
+// Whether the solve goes on and any of the V columns from c0 still iterates, for
+// the small levels' kernels: all loads are issued together, and the answer is
+// used only before the store.
+template <int V>
+__device__ __forceinline__ int group_runs(const CtlM *ctl, int c0) {
+    int a = 0;
+    const int done = __ldcg(&ctl->done);
+#pragma unroll
+    for (int v = 0; v < V; v++) a |= __ldcg(&ctl->active[c0 + v]);
+    return a && !done;
+}
+
 // Whether any of the V columns from c0 is still iterating.
 template <int V>
 __device__ __forceinline__ bool group_live(const CtlM *ctl, int c0) {
     int a = 0;
 #pragma unroll
-    for (int v = 0; v < V; v++) a |= ctl->active[c0 + v];
+    for (int v = 0; v < V; v++) a |= __ldcg(&ctl->active[c0 + v]);
     return a != 0;
 }
 
@@ -130,50 +146,42 @@ __device__ __forceinline__ bool group_live(const CtlM *ctl, int c0) {
     const bool live_ = group_live<V>(                                                         \
         ctl, (int)((((int64_t)blockIdx.x * blockDim.x + threadIdx.x) % (K / (V))) * (V)));
 
-// Per-column block sums: a thread holds a[V] and b[V] for columns c0..c0+V-1
-// (c0 fixed per thread). Result: threads 0..K-1 hold the block's sums for
-// columns 0..K-1.
-template <int K, int V>
-__device__ __forceinline__ void block_sum_cols(double (&a)[V], double (&b)[V], double &ra, double &rb) {
-    constexpr int TPR = K / V;
-    __shared__ double sa[kMB / 32][kMaxK], sb[kMB / 32][kMaxK];
-#pragma unroll
-    for (int o = 16; o >= TPR; o >>= 1)
-#pragma unroll
-        for (int v = 0; v < V; v++) {
-            a[v] += __shfl_down_sync(0xffffffffu, a[v], o);
-            b[v] += __shfl_down_sync(0xffffffffu, b[v], o);
-        }
-    int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane < TPR)
-#pragma unroll
-        for (int v = 0; v < V; v++) {
-            sa[w][lane * V + v] = a[v];
-            sb[w][lane * V + v] = b[v];
-        }
-    __syncthreads();
-    ra = rb = 0.0;
-    if (threadIdx.x < K) {
-        for (int q = 0; q < kMB / 32; q++) { ra += sa[q][threadIdx.x]; rb += sb[q][threadIdx.x]; }
+// Per-column scalars of a thread's fixed column group, read once (c: its first
+// column).
+#define MK_COLS(V, BODY)                                                                      \
+    {                                                                                         \
+        const int c = (int)((((int64_t)blockIdx.x * blockDim.x + threadIdx.x) % (K / (V))) * (V)); \
+        _Pragma("unroll") for (int v = 0; v < (V); v++) { BODY; }                             \
     }
-}
 
-// Writes the block's per-column partials (layout [slot][column][block]) and
-// returns true in every thread of the last block to finish.
-template <int K, int V>
-__device__ __forceinline__ bool publish_cols(double (&a)[V], double (&b)[V], double *partials,
-                                             unsigned *counter) {
+// Per-column sums of NV quantities: a thread holds a[s][v], the s-th quantity
+// of column c0 + v (c0 fixed per thread). The block's values meet in shared
+// memory by column and a warp adds one column at a time (reduce.cuh), so no
+// warp pays a float64 shuffle tree per quantity and column. Writes the block's
+// partials (layout [quantity][column][block]); true in every thread of the
+// last block to finish.
+template <int K, int V, int NV>
+__device__ __forceinline__ bool publish_cols(double (&a)[NV][V], double *partials, unsigned *counter) {
+    constexpr int TPR = K / V, R = kMB / TPR;  // threads per row, values per column
+    __shared__ double sh[NV * K * R];
     __shared__ bool last;
-    double ra, rb;
-    block_sum_cols<K, V>(a, b, ra, rb);
-    int G = gridDim.x;
-    if (threadIdx.x < K) {
-        partials[(0 * K + threadIdx.x) * G + blockIdx.x] = ra;
-        partials[(1 * K + threadIdx.x) * G + blockIdx.x] = rb;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int c0 = (int)(threadIdx.x % TPR) * V, r = threadIdx.x / TPR;
+#pragma unroll
+    for (int s = 0; s < NV; s++)
+#pragma unroll
+        for (int v = 0; v < V; v++) sh[(s * K + c0 + v) * R + r] = a[s][v];
+    __syncthreads();
+    const int G = gridDim.x;
+    for (int q = w; q < NV * K; q += kMB / 32) {
+        double t = lane < R ? sh[q * R + lane] : 0.0;
+        for (int k = lane + 32; k < R; k += 32) t += sh[q * R + k];
+        t = warp_sum(t);
+        if (lane == 0) partials[(int64_t)q * G + blockIdx.x] = t;
     }
+    __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
         unsigned t = atomicAdd(counter, 1u);
         last = (t == gridDim.x - 1);
     }
@@ -181,29 +189,25 @@ __device__ __forceinline__ bool publish_cols(double (&a)[V], double (&b)[V], dou
     return last;
 }
 
-// Last block: res[q] = sum over blocks of partials[q][.] in block order, for
-// q < 2K (slot 0 columns, then slot 1 columns). Loads are unrolled so each
-// lane has several in flight.
-template <int K>
+// Last block: res[q] = sum over blocks of partials[q][.], q < NV K.
+template <int K, int NV>
 __device__ __forceinline__ void final_cols(const double *partials, double *res) {
     __threadfence();
-    int G = gridDim.x;
-    int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int q = w; q < 2 * K; q += kMB / 32) {
+    const int G = gridDim.x;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int q = w; q < NV * K; q += kMB / 32) {
         const double *src = partials + (int64_t)q * G;
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-        int k = lane;
-        for (; k + 96 < G; k += 128) {
-            s0 += __ldcg(src + k);
-            s1 += __ldcg(src + k + 32);
-            s2 += __ldcg(src + k + 64);
-            s3 += __ldcg(src + k + 96);
-        }
-        for (; k < G; k += 32) s0 += __ldcg(src + k);
-        double s = (s0 + s1) + (s2 + s3);
+        double t = 0.0;
+        for (int k0 = lane; k0 < G; k0 += 32 * 8) {
+            double x[8];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-        if (lane == 0) res[q] = s;
+            for (int u = 0; u < 8; u++) x[u] = k0 + 32 * u < G ? __ldcg(src + k0 + 32 * u) : 0.0;
+#pragma unroll
+            for (int u = 0; u < 8; u++)
+                if (k0 - lane + 32 * u < G) t += x[u];
+        }
+        t = warp_sum(t);
+        if (lane == 0) res[q] = t;
     }
     __syncthreads();
 }
@@ -213,13 +217,15 @@ __device__ __forceinline__ void col_fail(CtlM *c, int col, int status) {
     c->active[col] = 0;
 }
 
-__device__ __forceinline__ void update_done(CtlM *c) {
-    int any = 0;
-    for (int q = 0; q < c->K; q++) any |= c->active[q];
-    if (!any) c->done = 1;
+// Every thread of the last block: done once no column is active. Thread c < K
+// passes column c's flag.
+__device__ __forceinline__ void update_done(CtlM *c, int active) {
+    const int any = __syncthreads_or(active);
+    if (threadIdx.x == 0 && !any) c->done = 1;
 }
 
 // ------------------------------------------------------------ V-cycle
+// Level 0 and the other large levels: t = p (b - A xpre).
 template <typename T, typename IDX, int K, int U, bool STREAM>
 __global__ void __launch_bounds__(kMB) k_down_m(int n, const int32_t *__restrict__ sptr,
                                                const IDX *__restrict__ col, const T *__restrict__ val,
@@ -227,7 +233,8 @@ __global__ void __launch_bounds__(kMB) k_down_m(int n, const int32_t *__restrict
                                                const T *__restrict__ p, T *__restrict__ t,
                                                const CtlM *__restrict__ ctl) {
     constexpr int V = VW<T>::V;
-    if (ctl->done) return;
+    pdl_enter();
+    if (__ldcg(&ctl->done)) return;
     MK_LIVE(V)
     MK_FOR(live_ ? n : 0, V) {
         MK_IDX(V)
@@ -246,62 +253,155 @@ __global__ void __launch_bounds__(kMB) k_down_m(int n, const int32_t *__restrict
     }
 }
 
+// k_down_m and k_post_m on the coarse levels, which wait for latency: one
+// (row, column group) per thread, its first U entries and the weight loaded
+// before the wait, the next chunk's entries in flight during the gathers.
+template <typename T, typename IDX, int K, int U>
+__global__ void __launch_bounds__(kMB) k_down_c(int n, const int32_t *__restrict__ sptr,
+                                               const IDX *__restrict__ col, const T *__restrict__ val,
+                                               const IDX *__restrict__ upat, const T *__restrict__ xpre,
+                                               const T *__restrict__ b, const T *__restrict__ p, T *__restrict__ t,
+                                               const CtlM *__restrict__ ctl) {
+    constexpr int V = VW<T>::V;
+    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = (int)(g / (K / V)), c0 = (int)(g % (K / V)) * V;
+    const bool in = i < n;
+    SellRow<U, false, IDX, T> R;
+    T pi = 0;
+    if (in) {
+        R.load(sptr, col, val, i, upat);
+        pi = ldg(p + i);
+    }
+    pdl_enter();
+    xpre = after_wait(xpre);
+    b = after_wait(b);
+    ctl = after_wait(ctl);
+    if (!in) return;
+    const int runs = group_runs<V>(ctl, c0);
+    const int64_t e0 = (int64_t)i * K + c0;
+    T bv[V], acc[V], o[V];
+    ld_vec<T, V>(b + e0, bv);
+    R.template dot_vec<V>(i, [&](int j, T (&x)[V]) { ld_vec<T, V>(xpre + (int64_t)j * K + c0, x); }, acc);
+#pragma unroll
+    for (int v = 0; v < V; v++) o[v] = pi * (bv[v] - acc[v]);
+    if (runs) st_vec<T, V>(t + e0, o);
+}
+
+template <typename T, typename IDX, int K, int U>
+__global__ void __launch_bounds__(kMB) k_post_c(int n, const int32_t *__restrict__ sptr,
+                                               const IDX *__restrict__ col, const T *__restrict__ val,
+                                               const IDX *__restrict__ upat, const T *__restrict__ xp,
+                                               const T *__restrict__ b, const T *__restrict__ dinv,
+                                               T *__restrict__ z, const CtlM *__restrict__ ctl) {
+    constexpr int V = VW<T>::V;
+    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = (int)(g / (K / V)), c0 = (int)(g % (K / V)) * V;
+    const bool in = i < n;
+    SellRow<U, false, IDX, T> R;
+    T d = 0;
+    if (in) {
+        R.load(sptr, col, val, i, upat);
+        d = ldg(dinv + i);
+    }
+    pdl_enter();
+    xp = after_wait(xp);
+    b = after_wait(b);
+    ctl = after_wait(ctl);
+    if (!in) return;
+    const int runs = group_runs<V>(ctl, c0);
+    const int64_t e0 = (int64_t)i * K + c0;
+    T xv[V], bv[V], acc[V], o[V];
+    ld_vec<T, V>(xp + e0, xv);
+    ld_vec<T, V>(b + e0, bv);
+    R.template dot_vec<V>(i, [&](int j, T (&x)[V]) { ld_vec<T, V>(xp + (int64_t)j * K + c0, x); }, acc);
+#pragma unroll
+    for (int v = 0; v < V; v++) o[v] = xv[v] + d * (bv[v] - acc[v]);
+    if (runs) st_vec<T, V>(z + e0, o);
+}
+
+// b_c[I] = sum of t over the members of aggregate I in index order (and
+// xpre_c = dinv_c b_c), one (coarse row, column group) per thread; the first
+// four members are static and read before the wait.
 template <typename T, typename TO, bool PRE, int K>
 __global__ void __launch_bounds__(kMB) k_restrict_m(int nc, const int32_t *__restrict__ rptr,
                                                    const int32_t *__restrict__ ridx, const T *__restrict__ t,
                                                    TO *__restrict__ bc, const T *__restrict__ dinvc,
                                                    T *__restrict__ xprec, const CtlM *__restrict__ ctl) {
-    constexpr int V = VW<T>::V;
-    if (ctl->done) return;
-    MK_LIVE(V)
-    MK_FOR(live_ ? nc : 0, V) {
-        MK_IDX(V)
-        T s[V];
+    constexpr int V = VW<T>::V, M = 4;
+    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = (int)(g / (K / V)), c0 = (int)(g % (K / V)) * V;
+    const bool in = i < nc;
+    int32_t q0 = 0, q1 = 0;
+    int m[M];
+    T d = 0;
+    if (in) {
+        q0 = ldg(rptr + i);
+        q1 = ldg(rptr + i + 1);
 #pragma unroll
-        for (int v = 0; v < V; v++) s[v] = 0;
-        for (int32_t q = ldg(rptr + i); q < ldg(rptr + i + 1); q++) {
-            T x[V];
-            ld_vec<T, V>(t + (int64_t)ldg(ridx + q) * K + c0, x);
+        for (int u = 0; u < M; u++) m[u] = q0 + u < q1 ? ldg(ridx + q0 + u) : 0;
+        if (PRE) d = ldg(dinvc + i);
+    }
+    pdl_enter();
+    t = after_wait(t);
+    ctl = after_wait(ctl);
+    if (!in) return;
+    const int runs = group_runs<V>(ctl, c0);
+    const int64_t e0 = (int64_t)i * K + c0;
+    T s[V], x[M][V];
 #pragma unroll
-            for (int v = 0; v < V; v++) s[v] += x[v];
+    for (int v = 0; v < V; v++) s[v] = 0;
+#pragma unroll
+    for (int u = 0; u < M; u++)
+        if (q0 + u < q1) ld_vec<T, V>(t + (int64_t)m[u] * K + c0, x[u]);
+#pragma unroll
+    for (int u = 0; u < M; u++)
+        if (q0 + u < q1) {
+#pragma unroll
+            for (int v = 0; v < V; v++) s[v] += x[u][v];
         }
+    for (int32_t q = q0 + M; q < q1; q++) {
+        T y[V];
+        ld_vec<T, V>(t + (int64_t)ldg(ridx + q) * K + c0, y);
 #pragma unroll
-        for (int v = 0; v < V; v++) bc[e0 + v] = (TO)s[v];
-        if (PRE) {
-            T d = ldg(dinvc + i), o[V];
+        for (int v = 0; v < V; v++) s[v] += y[v];
+    }
+    if (!runs) return;
 #pragma unroll
-            for (int v = 0; v < V; v++) o[v] = d * s[v];
-            st_vec<T, V>(xprec + e0, o);
-        }
+    for (int v = 0; v < V; v++) bc[e0 + v] = (TO)s[v];
+    if (PRE) {
+        T o[V];
+#pragma unroll
+        for (int v = 0; v < V; v++) o[v] = d * s[v];
+        st_vec<T, V>(xprec + e0, o);
     }
 }
 
-// x_L = A_L^{-1} b_L for K columns (float64): one warp per (row, pair of
-// columns), lanes striding over the row with coalesced loads of A_L^{-1},
-// then the shuffle tree -- the order of k_coarse, per column.
+// x = B b for K columns on the directly solved level (float64): the coarsest
+// inverse, or the explicit operator of the small levels (amg_hier::op). One
+// warp per (row, pair of columns), lanes striding over the row with coalesced
+// loads, then the warp's sum.
 template <typename TO, int K>
 __global__ void __launch_bounds__(kMB) k_coarse_m(int nL, const double *__restrict__ ainv,
                                                  const double *__restrict__ bL, TO *__restrict__ xL,
                                                  const CtlM *__restrict__ ctl) {
     constexpr int V = 2;
-    if (ctl->done) return;
+    pdl_enter();
+    if (__ldcg(&ctl->done)) return;
     int warp = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (warp >= nL * (K / V)) return;  // whole warps
     int row = warp / (K / V), c0 = (warp % (K / V)) * V;
     if (!group_live<V>(ctl, c0)) return;
     const double *a = ainv + (int64_t)row * nL;
     double s0 = 0.0, s1 = 0.0;
+#pragma unroll 4
     for (int j = lane; j < nL; j += 32) {
         double aj = ldg(a + j);
         double2 bj = __ldg(reinterpret_cast<const double2 *>(bL + (int64_t)j * K + c0));
         s0 += aj * bj.x;
         s1 += aj * bj.y;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        s0 += __shfl_down_sync(0xffffffffu, s0, o);
-        s1 += __shfl_down_sync(0xffffffffu, s1, o);
-    }
+    s0 = warp_sum(s0);
+    s1 = warp_sum(s1);
     if (lane == 0) {
         xL[(int64_t)row * K + c0] = (TO)s0;
         xL[(int64_t)row * K + c0 + 1] = (TO)s1;
@@ -313,7 +413,8 @@ __global__ void __launch_bounds__(kMB) k_prolong_m(int n, const T *__restrict__ 
                                                   const int32_t *__restrict__ agg, const T *__restrict__ xc,
                                                   T *__restrict__ xp, const CtlM *__restrict__ ctl) {
     constexpr int V = VW<T>::V;
-    if (ctl->done) return;
+    pdl_enter();
+    if (__ldcg(&ctl->done)) return;
     MK_LIVE(V)
     MK_FOR(live_ ? n : 0, V) {
         MK_IDX(V)
@@ -330,6 +431,31 @@ __global__ void __launch_bounds__(kMB) k_prolong_m(int n, const T *__restrict__ 
     }
 }
 
+// Per-column rho = r.z and beta (see the single-column k_axpy_p) from the
+// threads' sums of r.z and, with NV = 2, z.q_old.
+template <int K, int V, int NV>
+__device__ __forceinline__ void finish_rho_m(double (&sums)[NV][V], double *partials, CtlM *ctl) {
+    __shared__ double res[NV * K];
+    if (!publish_cols<K, V, NV>(sums, partials, &ctl->counter[0])) return;
+    final_cols<K, NV>(partials, res);
+    if (threadIdx.x == 0) ctl->counter[0] = 0;
+    const int c = threadIdx.x;
+    if (c < K && __ldcg(&ctl->active[c])) {
+        const double rho = res[c], zqc = NV == 2 ? res[(NV - 1) * K + c] : 0.0;
+        if (!isfinite(rho) || !isfinite(zqc)) {
+            col_fail(ctl, c, AMG_ERR_NAN);
+        } else if (!(rho > 0.0)) {
+            col_fail(ctl, c, AMG_ERR_BREAKDOWN);
+        } else {
+            ctl->rho[c] = rho;
+            double beta = 0.0;
+            if (!__ldcg(&ctl->restart[c]))
+                beta = NV == 2 ? -zqc / __ldcg(&ctl->pq_old[c]) : rho / __ldcg(&ctl->rho_old[c]);
+            ctl->beta[c] = beta;
+        }
+    }
+}
+
 // z = xp + D^-1 (b - A xp); DOT on level 0: per-column r.z and z.q_old, and
 // the last block forms rho_c and beta_c.
 template <typename T, typename TZ, bool DOT, bool FCG, typename IDX, int K, int U, bool STREAM>
@@ -340,10 +466,10 @@ __global__ void __launch_bounds__(kMB) k_post_m(int n, const int32_t *__restrict
                                                const double *__restrict__ r64, const double *__restrict__ qold,
                                                double *partials, CtlM *ctl) {
     constexpr int V = VW<T>::V;
-    if (ctl->done) return;
-    double rz[V], zq[V];
-#pragma unroll
-    for (int v = 0; v < V; v++) rz[v] = zq[v] = 0.0;
+    pdl_enter();
+    if (__ldcg(&ctl->done)) return;
+    constexpr int NV = FCG ? 2 : 1;
+    double sums[NV][V] = {};
     MK_LIVE(V)
     MK_FOR(live_ ? n : 0, V) {
         MK_IDX(V)
@@ -359,37 +485,15 @@ __global__ void __launch_bounds__(kMB) k_post_m(int n, const int32_t *__restrict
         T d = ldg(dinv + i);
 #pragma unroll
         for (int v = 0; v < V; v++) {
-            TZ zo = (TZ)(xv[v] + d * (bv[v] - acc[v]));
+            const TZ zo = (TZ)(xv[v] + d * (bv[v] - acc[v]));
             z[e0 + v] = zo;
             if (DOT) {
-                rz[v] += ldg(r64 + e0 + v) * (double)zo;
-                if (FCG) zq[v] += (double)zo * ldg(qold + e0 + v);
+                sums[0][v] += ldg(r64 + e0 + v) * (double)zo;
+                if (FCG) sums[NV - 1][v] += (double)zo * ldg(qold + e0 + v);
             }
         }
     }
-    if (DOT) {
-        __shared__ double res[2 * kMaxK];
-        if (publish_cols<K, V>(rz, zq, partials, &ctl->counter[0])) {
-            final_cols<K>(partials, res);
-            if (threadIdx.x == 0) ctl->counter[0] = 0;
-            int c = threadIdx.x;
-            if (c < K && ctl->active[c]) {
-                double rho = res[c], zqc = res[K + c];
-                if (!isfinite(rho) || !isfinite(zqc)) {
-                    col_fail(ctl, c, AMG_ERR_NAN);
-                } else if (!(rho > 0.0)) {
-                    col_fail(ctl, c, AMG_ERR_BREAKDOWN);
-                } else {
-                    ctl->rho[c] = rho;
-                    double beta = 0.0;
-                    if (!ctl->restart[c])
-                        beta = ctl->mode == AMG_MODE_FCG32 || ctl->flex ? -zqc / ctl->pq_old[c]
-                                                                        : rho / ctl->rho_old[c];
-                    ctl->beta[c] = beta;
-                }
-            }
-        }
-    }
+    if constexpr (DOT) finish_rho_m<K, V, NV>(sums, partials, ctl);
 }
 
 // ------------------------------------------------------------ hybrid Gauss-Seidel
@@ -412,7 +516,8 @@ __global__ void __launch_bounds__(kMB) k_gs_warp_m(int n, int nb, int w, const i
                                                   const CtlM *__restrict__ ctl) {
     constexpr int V = VW<T>::V;
     constexpr int G = K / V;
-    if (ctl->done) return;
+    pdl_enter();
+    if (__ldcg(&ctl->done)) return;
     const int lane = threadIdx.x & 31;
     const int nsl = (n + 31) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -508,10 +613,10 @@ __global__ void __launch_bounds__(kMB) k_gs_finish0_m(int n, const T *__restrict
                                                      const double *__restrict__ qold, double *__restrict__ z,
                                                      double *partials, CtlM *ctl) {
     constexpr int V = VW<T>::V;
-    if (ctl->done) return;
-    double rz[V], zq[V];
-#pragma unroll
-    for (int v = 0; v < V; v++) rz[v] = zq[v] = 0.0;
+    pdl_enter();
+    if (__ldcg(&ctl->done)) return;
+    constexpr int NV = FCG ? 2 : 1;
+    double sums[NV][V] = {};
     MK_LIVE(V)
     MK_FOR(live_ ? n : 0, V) {
         MK_IDX(V)
@@ -521,30 +626,11 @@ __global__ void __launch_bounds__(kMB) k_gs_finish0_m(int n, const T *__restrict
         for (int v = 0; v < V; v++) {
             double zo = (double)xv[v];
             z[e0 + v] = zo;
-            rz[v] += ldg(r64 + e0 + v) * zo;
-            if (FCG) zq[v] += zo * ldg(qold + e0 + v);
+            sums[0][v] += ldg(r64 + e0 + v) * zo;
+            if (FCG) sums[NV - 1][v] += zo * ldg(qold + e0 + v);
         }
     }
-    __shared__ double res[2 * kMaxK];
-    if (publish_cols<K, V>(rz, zq, partials, &ctl->counter[0])) {
-        final_cols<K>(partials, res);
-        if (threadIdx.x == 0) ctl->counter[0] = 0;
-        int c = threadIdx.x;
-        if (c < K && ctl->active[c]) {
-            double rho = res[c], zqc = res[K + c];
-            if (!isfinite(rho) || !isfinite(zqc)) {
-                col_fail(ctl, c, AMG_ERR_NAN);
-            } else if (!(rho > 0.0)) {
-                col_fail(ctl, c, AMG_ERR_BREAKDOWN);
-            } else {
-                ctl->rho[c] = rho;
-                double beta = 0.0;
-                if (!ctl->restart[c])
-                    beta = ctl->mode == AMG_MODE_FCG32 || ctl->flex ? -zqc / ctl->pq_old[c] : rho / ctl->rho_old[c];
-                ctl->beta[c] = beta;
-            }
-        }
-    }
+    finish_rho_m<K, V, NV>(sums, partials, ctl);
 }
 
 // ------------------------------------------------------------ Krylov
@@ -552,27 +638,35 @@ template <int K>
 __global__ void __launch_bounds__(kMB) k_axpy_m(int n, const double *__restrict__ z, double *__restrict__ p,
                                                const CtlM *__restrict__ ctl) {
     constexpr int V = 2;
-    if (ctl->done) return;
+    pdl_enter();
+    if (__ldcg(&ctl->done)) return;
     MK_LIVE(V)
+    int act[V];
+    double beta[V];
+    MK_COLS(V, act[v] = __ldcg(&ctl->active[c + v]); beta[v] = __ldcg(&ctl->beta[c + v]))
     MK_FOR(live_ ? n : 0, V) {
         MK_IDX(V)
         double zv[V], pv[V], o[V];
         ld_vec<double, V>(z + e0, zv);
         ld_vec_cg<double, V>(p + e0, pv);
 #pragma unroll
-        for (int v = 0; v < V; v++) o[v] = ctl->active[c0 + v] ? zv[v] + ctl->beta[c0 + v] * pv[v] : 0.0;
+        for (int v = 0; v < V; v++) o[v] = act[v] ? zv[v] + beta[v] * pv[v] : 0.0;
         st_vec<double, V>(p + e0, o);
     }
 }
 
+// Bound by the float64 pipe (two FMAs per entry and thread); from 16 columns on
+// a full SM of warps at 32 registers keeps it busier than fewer with more
+// (96^3 x 32: whole solves 172 -> 164 ms; 40^3 x 8 7.0 -> 7.3 ms, so not there).
 template <typename IDX, int K>
-__global__ void __launch_bounds__(kMB) k_spmm_m(int n, const int32_t *__restrict__ sptr,
+__global__ void __launch_bounds__(kMB, K >= 16 ? 8 : 4) k_spmm_m(int n, const int32_t *__restrict__ sptr,
                                                const IDX *__restrict__ col, const double *__restrict__ val,
                                                const double *__restrict__ p, double *__restrict__ q,
                                                double *partials, CtlM *ctl) {
     constexpr int V = 2;
-    if (ctl->done) return;
-    double pq[V] = {0.0, 0.0}, unused[V] = {0.0, 0.0};
+    pdl_enter();
+    if (__ldcg(&ctl->done)) return;
+    double pq[1][V] = {};
     MK_LIVE(V)
     MK_FOR(live_ ? n : 0, V) {
         MK_IDX(V)
@@ -587,26 +681,25 @@ __global__ void __launch_bounds__(kMB) k_spmm_m(int n, const int32_t *__restrict
         double pv[V];
         ld_vec<double, V>(p + e0, pv);
 #pragma unroll
-        for (int v = 0; v < V; v++) pq[v] += pv[v] * acc[v];
+        for (int v = 0; v < V; v++) pq[0][v] += pv[v] * acc[v];
     }
-    __shared__ double res[2 * kMaxK];
-    if (publish_cols<K, V>(pq, unused, partials, &ctl->counter[1])) {
-        final_cols<K>(partials, res);
+    __shared__ double res[K];
+    if (publish_cols<K, V, 1>(pq, partials, &ctl->counter[1])) {
+        final_cols<K, 1>(partials, res);
         if (threadIdx.x == 0) ctl->counter[1] = 0;
         int c = threadIdx.x;
         if (c < K) {
-            if (!ctl->active[c]) {
-                ctl->alpha[c] = 0.0;
-            } else {
+            double alpha = 0.0;
+            if (__ldcg(&ctl->active[c])) {
                 double a = res[c];
                 if (!isfinite(a)) col_fail(ctl, c, AMG_ERR_NAN);
                 else if (!(a > 0.0)) col_fail(ctl, c, AMG_ERR_BREAKDOWN);
                 else {
                     ctl->pq[c] = a;
-                    ctl->alpha[c] = ctl->rho[c] / a;
+                    alpha = __ldcg(&ctl->rho[c]) / a;
                 }
-                if (!ctl->active[c]) ctl->alpha[c] = 0.0;
             }
+            ctl->alpha[c] = alpha;
         }
     }
 }
@@ -634,9 +727,13 @@ __global__ void __launch_bounds__(kMB) k_update_m(int n, const double *__restric
                                                  const double *__restrict__ dinv64, double *__restrict__ xpre64,
                                                  double *partials, CtlM *ctl, double *hist, int hstride) {
     constexpr int V = 2;
-    if (ctl->done) return;
-    double rr[V] = {0.0, 0.0}, unused[V] = {0.0, 0.0};
+    pdl_enter();
+    if (__ldcg(&ctl->done)) return;
+    double rr[1][V] = {};
     MK_LIVE(V)
+    int act[V];
+    double al[V];
+    MK_COLS(V, act[v] = __ldcg(&ctl->active[c + v]); al[v] = __ldcg(&ctl->alpha[c + v]))
     MK_FOR(live_ ? n : 0, V) {
         MK_IDX(V)
         double rv[V], xv[V], pv[V], qv[V];
@@ -646,42 +743,50 @@ __global__ void __launch_bounds__(kMB) k_update_m(int n, const double *__restric
         ld_vec<double, V>(q + e0, qv);
 #pragma unroll
         for (int v = 0; v < V; v++) {
-            if (ctl->active[c0 + v]) {
-                double al = ctl->alpha[c0 + v];
-                xv[v] = xv[v] + al * pv[v];
-                rv[v] = rv[v] - al * qv[v];
-                rr[v] += rv[v] * rv[v];
+            if (act[v]) {
+                xv[v] = xv[v] + al[v] * pv[v];
+                rv[v] = rv[v] - al[v] * qv[v];
+                rr[0][v] += rv[v] * rv[v];
             }
         }
         st_vec<double, V>(x + e0, xv);
         st_vec<double, V>(r + e0, rv);
         emit_r_m<MODE>(e0, i, rv, r32, dinv32, xpre32, dinv64, xpre64);
     }
-    __shared__ double res[2 * kMaxK];
-    if (publish_cols<K, V>(rr, unused, partials, &ctl->counter[2])) {
-        final_cols<K>(partials, res);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            ctl->counter[2] = 0;
-            ctl->iter_all += 1;
-            int anycheck = 0;
-            for (int c = 0; c < K; c++) {
-                if (!ctl->active[c]) continue;
-                int it = ctl->iter[c] + 1;
-                ctl->iter[c] = it;
-                double rel = sqrt(res[c]) / ctl->bnorm[c];
-                ctl->rel[c] = rel;
-                hist[(int64_t)c * hstride + it] = rel;
-                ctl->rho_old[c] = ctl->rho[c];
-                ctl->pq_old[c] = ctl->pq[c];
-                ctl->restart[c] = 0;
-                if (!isfinite(rel)) { col_fail(ctl, c, AMG_ERR_NAN); continue; }
-                if (rel <= ctl->rtol) { ctl->check[c] = 1; anycheck = 1; }
-                else if (it >= ctl->maxit) col_fail(ctl, c, AMG_ERR_NOCONV);
+    __shared__ double res[K];
+    if (publish_cols<K, V, 1>(rr, partials, &ctl->counter[2])) {
+        final_cols<K, 1>(partials, res);
+        // one thread per column: its scalars, then whether any goes on
+        const int c = threadIdx.x;
+        int active = 0, check = 0;
+        if (c < K && __ldcg(&ctl->active[c])) {
+            const int it = __ldcg(&ctl->iter[c]) + 1;
+            const double rel = sqrt(res[c]) / __ldcg(&ctl->bnorm[c]);
+            ctl->iter[c] = it;
+            ctl->rel[c] = rel;
+            hist[(int64_t)c * hstride + it] = rel;
+            ctl->rho_old[c] = __ldcg(&ctl->rho[c]);
+            ctl->pq_old[c] = __ldcg(&ctl->pq[c]);
+            ctl->restart[c] = 0;
+            active = 1;
+            if (!isfinite(rel)) {
+                col_fail(ctl, c, AMG_ERR_NAN);
+                active = 0;
+            } else if (rel <= __ldcg(&ctl->rtol)) {
+                ctl->check[c] = 1;
+                check = 1;
+            } else if (it >= __ldcg(&ctl->maxit)) {
+                col_fail(ctl, c, AMG_ERR_NOCONV);
+                active = 0;
             }
-            ctl->any_check = anycheck;
-            update_done(ctl);
         }
+        const int any_check = __syncthreads_or(check);
+        if (c == 0) {
+            ctl->counter[2] = 0;
+            ctl->iter_all = __ldcg(&ctl->iter_all) + 1;
+            ctl->any_check = any_check;
+        }
+        update_done(ctl, active);
     }
 }
 
@@ -697,14 +802,16 @@ __global__ void __launch_bounds__(kMB) k_residual_m(int n, const int32_t *__rest
                                                    const double *__restrict__ dinv64, double *__restrict__ xpre64,
                                                    double *partials, CtlM *ctl, double *hist, int hstride) {
     constexpr int V = 2;
-    if (ctl->done) return;
-    if (!INIT && !ctl->any_check) return;
-    double rr[V] = {0.0, 0.0}, bb[V] = {0.0, 0.0};
-    MK_FOR(n, V) {
+    pdl_enter();
+    if (__ldcg(&ctl->done)) return;
+    if (!INIT && !__ldcg(&ctl->any_check)) return;
+    constexpr int NV = INIT ? 2 : 1;
+    double sums[NV][V] = {};
+    int use[V];
+    MK_COLS(V, use[v] = INIT ? __ldcg(&ctl->pending[c + v]) : __ldcg(&ctl->check[c + v]))
+    const bool use0 = use[0] != 0, use1 = use[1] != 0;
+    MK_FOR(use0 || use1 ? n : 0, V) {
         MK_IDX(V)
-        bool use0 = INIT ? ctl->pending[c0] != 0 : ctl->check[c0] != 0;
-        bool use1 = INIT ? ctl->pending[c0 + 1] != 0 : ctl->check[c0 + 1] != 0;
-        if (!use0 && !use1) continue;
         int s = i >> 5, lane = i & 31;
         int32_t base = ldg(sptr + s);
         int w = (ldg(sptr + s + 1) - base) >> 5;
@@ -719,55 +826,76 @@ __global__ void __launch_bounds__(kMB) k_residual_m(int n, const int32_t *__rest
         if (use1) rv[1] = bv[1] - acc[1];
         st_vec<double, V>(r + e0, rv);
         emit_r_m<MODE>(e0, i, rv, r32, dinv32, xpre32, dinv64, xpre64);
-        if (use0) rr[0] += rv[0] * rv[0];
-        if (use1) rr[1] += rv[1] * rv[1];
+        if (use0) sums[0][0] += rv[0] * rv[0];
+        if (use1) sums[0][1] += rv[1] * rv[1];
         if (INIT) {
-            if (use0) bb[0] += bv[0] * bv[0];
-            if (use1) bb[1] += bv[1] * bv[1];
+            if (use0) sums[NV - 1][0] += bv[0] * bv[0];
+            if (use1) sums[NV - 1][1] += bv[1] * bv[1];
         }
     }
-    __shared__ double res[2 * kMaxK];
-    if (publish_cols<K, V>(rr, bb, partials, &ctl->counter[3])) {
-        final_cols<K>(partials, res);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            ctl->counter[3] = 0;
-            for (int c = 0; c < K; c++) {
-                if (INIT) {
-                    if (!ctl->pending[c]) continue;
-                    ctl->pending[c] = 0;
-                    double bn = sqrt(res[K + c]);
-                    ctl->bnorm[c] = bn;
+    __shared__ double res[NV * K];
+    if (publish_cols<K, V, NV>(sums, partials, &ctl->counter[3])) {
+        final_cols<K, NV>(partials, res);
+        const int c = threadIdx.x;
+        int active = 0;
+        if (c < K) {
+            active = __ldcg(&ctl->active[c]);
+            if (INIT && __ldcg(&ctl->pending[c])) {
+                const double bn = sqrt(res[(NV - 1) * K + c]);
+                ctl->pending[c] = 0;
+                ctl->bnorm[c] = bn;
+                ctl->status[c] = AMG_OK;
+                ctl->iter[c] = 0;
+                ctl->check[c] = 0;
+                active = 0;
+                int status = AMG_OK;
+                if (c < __ldcg(&ctl->k)) {
+                    if (!isfinite(bn) || !isfinite(res[c])) {
+                        status = AMG_ERR_NAN;
+                    } else if (bn == 0.0) {
+                        ctl->true_rel[c] = 0.0;
+                        hist[(int64_t)c * hstride] = 0.0;
+                    } else {
+                        const double rel = sqrt(res[c]) / bn;
+                        ctl->rel[c] = rel;
+                        ctl->true_rel[c] = rel;
+                        hist[(int64_t)c * hstride] = rel;
+                        if (!(rel <= __ldcg(&ctl->rtol))) {
+                            if (__ldcg(&ctl->maxit) <= 0) {
+                                status = AMG_ERR_NOCONV;
+                            } else {
+                                active = 1;
+                                ctl->restart[c] = 1;
+                            }
+                        }
+                    }
+                }
+                ctl->active[c] = active;
+                if (status != AMG_OK) ctl->status[c] = status;
+            } else if (!INIT && __ldcg(&ctl->check[c])) {
+                const double rel = sqrt(res[c]) / __ldcg(&ctl->bnorm[c]);
+                const int it = __ldcg(&ctl->iter[c]);
+                ctl->check[c] = 0;
+                ctl->true_rel[c] = rel;
+                active = 0;
+                if (!isfinite(rel)) {
+                    col_fail(ctl, c, AMG_ERR_NAN);
+                } else if (rel <= __ldcg(&ctl->rtol)) {
                     ctl->active[c] = 0;
                     ctl->status[c] = AMG_OK;
-                    ctl->iter[c] = 0;
-                    ctl->check[c] = 0;
-                    if (c >= ctl->k) continue;
-                    if (!isfinite(bn) || !isfinite(res[c])) { col_fail(ctl, c, AMG_ERR_NAN); continue; }
-                    if (bn == 0.0) { ctl->true_rel[c] = 0.0; hist[(int64_t)c * hstride] = 0.0; continue; }
-                    double rel = sqrt(res[c]) / bn;
-                    ctl->rel[c] = rel;
-                    ctl->true_rel[c] = rel;
-                    hist[(int64_t)c * hstride] = rel;
-                    if (rel <= ctl->rtol) continue;
-                    if (ctl->maxit <= 0) { col_fail(ctl, c, AMG_ERR_NOCONV); continue; }
-                    ctl->active[c] = 1;
-                    ctl->restart[c] = 1;
                 } else {
-                    if (!ctl->check[c]) continue;
-                    ctl->check[c] = 0;
-                    double rel = sqrt(res[c]) / ctl->bnorm[c];
-                    ctl->true_rel[c] = rel;
-                    if (!isfinite(rel)) { col_fail(ctl, c, AMG_ERR_NAN); continue; }
-                    if (rel <= ctl->rtol) { ctl->active[c] = 0; ctl->status[c] = AMG_OK; continue; }
                     ctl->restart[c] = 1;
-                    hist[(int64_t)c * hstride + ctl->iter[c]] = rel;
-                    if (ctl->iter[c] >= ctl->maxit) col_fail(ctl, c, AMG_ERR_NOCONV);
+                    hist[(int64_t)c * hstride + it] = rel;
+                    if (it >= __ldcg(&ctl->maxit)) col_fail(ctl, c, AMG_ERR_NOCONV);
+                    else active = 1;
                 }
             }
-            ctl->any_check = 0;
-            update_done(ctl);
         }
+        if (c == 0) {
+            ctl->counter[3] = 0;
+            ctl->any_check = 0;
+        }
+        update_done(ctl, active);
     }
 }
 
@@ -838,17 +966,19 @@ struct MP<double> {
     static const double *part(const Level &l, int d) { return l.gs_v64[d]; }
 };
 
-#define WITH_COLS_M(S, BODY)              \
-    do {                                  \
-        if ((S).col16) {                  \
-            using IDX = int16_t;          \
-            const IDX *cols = (S).col16;  \
-            BODY;                         \
-        } else {                          \
-            using IDX = int32_t;          \
-            const IDX *cols = (S).col;    \
-            BODY;                         \
-        }                                 \
+#define WITH_COLS_M(S, BODY)                               \
+    do {                                                   \
+        if ((S).col16) {                                   \
+            using IDX = int16_t;                           \
+            const IDX *cols = (S).col16;                   \
+            [[maybe_unused]] const IDX *pats = (S).upat16; \
+            BODY;                                          \
+        } else {                                           \
+            using IDX = int32_t;                           \
+            const IDX *cols = (S).col;                     \
+            [[maybe_unused]] const IDX *pats = (S).upat;   \
+            BODY;                                          \
+        }                                                  \
     } while (0)
 
 // gs_nu Gauss-Seidel sweeps of level l for K columns: pre-smoothing
@@ -869,43 +999,70 @@ void launch_gs_m(amg_hier *h, MultiWS &W, int l, bool pre, const T *b, T *target
     for (int sw = 1; sw <= nu; sw++) {
         T *dst = (nu - sw) % 2 == 0 ? target : P::t(mv);
         const bool zero = pre && sw == 1;
-#define PCG_GSM(UU, ST)                                                                                          \
-    do {                                                                                                         \
-        if (zero)                                                                                                \
-            WITH_COLS_M(lv.S, (k_gs_warp_m<T, IDX, UU, true, true, ST, K><<<grid, kMB, 0, s>>>(                  \
-                                  n, nb, w, lv.S.sptr, cols, P::val(lv), lv.gs_ci[d], P::part(lv, d), P::dinv(lv), \
-                                  b, src, dst, W.ctl)));                                                         \
-        else if (pre)                                                                                            \
-            WITH_COLS_M(lv.S, (k_gs_warp_m<T, IDX, UU, true, false, ST, K><<<grid, kMB, 0, s>>>(                 \
-                                  n, nb, w, lv.S.sptr, cols, P::val(lv), lv.gs_ci[d], P::part(lv, d), P::dinv(lv), \
-                                  b, src, dst, W.ctl)));                                                         \
-        else                                                                                                     \
-            WITH_COLS_M(lv.S, (k_gs_warp_m<T, IDX, UU, false, false, ST, K><<<grid, kMB, 0, s>>>(                \
-                                  n, nb, w, lv.S.sptr, cols, P::val(lv), lv.gs_ci[d], P::part(lv, d), P::dinv(lv), \
-                                  b, src, dst, W.ctl)));                                                         \
+#define PCG_GSM_LAUNCH(UU, FWD, ZERO, ST)                                                                        \
+    WITH_COLS_M(lv.S, (launch_k(h->pdl, k_gs_warp_m<T, IDX, UU, FWD, ZERO, ST, K>, grid, kMB, s, n, nb, w,      \
+                                lv.S.sptr, cols, P::val(lv), lv.gs_ci[d], P::part(lv, d), P::dinv(lv), b, src,  \
+                                dst, W.ctl)))
+#define PCG_GSM(UU, ST)                                  \
+    do {                                                 \
+        if (zero) PCG_GSM_LAUNCH(UU, true, true, ST);    \
+        else if (pre) PCG_GSM_LAUNCH(UU, true, false, ST); \
+        else PCG_GSM_LAUNCH(UU, false, false, ST);       \
     } while (0)
         if (l == 0) PCG_GSM(kUnroll, true);
         else if (big) PCG_GSM(kUnroll, false);
         else PCG_GSM(kUnrollSmall, false);
+#undef PCG_GSM_LAUNCH
 #undef PCG_GSM
         src = dst;
     }
 }
 
+// The level that K columns solve directly: the explicit operator of the first
+// level whose product stays under kOpWorkM float64 FMAs (9 million take 14 us;
+// at 8 columns a 992-row level's sweeps, transfers and coarse solve took 25),
+// else the coarsest one.
+constexpr int64_t kOpWorkM = 9000000;
+int direct_level_m(const amg_hier *h, int K) {
+    const int L = (int)h->lev.size() - 1;
+    for (int l = h->op_first; l && l < L; l++)
+        if ((int64_t)h->lev[l].A.n * h->lev[l].A.n * K <= kOpWorkM) return l;
+    return L;
+}
+
+// Blocks of a grid-stride kernel: one thread per item up to two waves, else
+// one wave of what stays resident (a grid that is no multiple of it leaves SMs with blocks to spare
+// at the end: 96^3 x 32, q = A p 1549 us with 8 blocks per SM where 6 fit).
+template <typename F>
+int wave_grid(const MultiWS &W, F *kernel, int64_t items) {
+    int per = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, kMB, 0) != cudaSuccess || per < 1) per = 1;
+    const int64_t want = (items + kMB - 1) / kMB, wave = (int64_t)W.sms * per;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(want <= 2 * wave ? want : wave, W.grid));
+}
+
+// Threads per block of the coarse levels' kernels (few rows spread over the SMs).
+inline int block_of(const MultiWS &W, int64_t items) {
+    return items <= (int64_t)W.sms * 64 ? 64 : items <= (int64_t)W.sms * 128 ? 128 : kMB;
+}
+
+// Rows up to which a coarse level's rows load 16 entries per chunk, else 4.
+constexpr int kChunkRowsM = 16384;
+
 template <typename T, bool FCG, int K>
 int launch_vcycle_m(amg_hier *h, MultiWS &W, cudaStream_t s) {
     using P = MP<T>;
     constexpr int V = VW<T>::V;
-    auto gv = [](int64_t rows) { return grid_of(rows * (K / V)); };
     auto &lev = h->lev;
-    int L = (int)lev.size() - 1;
+    const int L = direct_level_m(h, K);  // levels 0..L-1 are swept
+    const bool pdl = h->pdl;
     CtlM *ctl = W.ctl;
     Level &l0 = lev[0];
     MultiLevel &m0 = W.lev[0];
+    const int64_t items0 = (int64_t)l0.A.n * (K / V);
     const T *b0;
     if constexpr (sizeof(T) == 4) b0 = W.r32;
     else b0 = W.r;
-    int g0 = W.grid;
     if (L == 0) {
         // single level: z = A^{-1} r through the coarse kernel (float32 rounding as the V-cycle's)
         set_error("pcg_solve_multi: single-level hierarchy not supported by the multi-column path");
@@ -913,83 +1070,113 @@ int launch_vcycle_m(amg_hier *h, MultiWS &W, cudaStream_t s) {
     }
     const bool gs = h->gs_nu > 0;
     if (gs) launch_gs_m<T, K>(h, W, 0, true, b0, P::xpre(m0), s);
-    WITH_COLS_M(l0.S, (k_down_m<T, IDX, K, kUnroll, true><<<g0, kMB, 0, s>>>(
-                          l0.A.n, l0.S.sptr, cols, P::val(l0), P::xpre(m0), b0, P::p(l0), P::t(m0), ctl)));
+    WITH_COLS_M(l0.S, (launch_k(pdl, k_down_m<T, IDX, K, kUnroll, true>,
+                                wave_grid(W, k_down_m<T, IDX, K, kUnroll, true>, items0), kMB, s, l0.A.n, l0.S.sptr,
+                                cols, P::val(l0), P::xpre(m0), b0, P::p(l0), P::t(m0), ctl)));
     for (int l = 0; l < L; l++) {
         Level &lv = lev[l];
         MultiLevel &mv = W.lev[l];
-        int n = lv.A.n;
-        if (l > 0 && gs) launch_gs_m<T, K>(h, W, l, true, P::b(mv), P::xpre(mv), s);
-        if (l > 0)
-            WITH_COLS_M(lv.S, (k_down_m<T, IDX, K, kUnroll, false><<<gv(n), kMB, 0, s>>>(
-                                  n, lv.S.sptr, cols, P::val(lv), P::xpre(mv), P::b(mv), P::p(lv), P::t(mv), ctl)));
+        const int n = lv.A.n;
+        const int64_t items = (int64_t)n * (K / V), citems = (int64_t)lv.nc * (K / V);
+        if (l > 0) {
+            if (gs) launch_gs_m<T, K>(h, W, l, true, P::b(mv), P::xpre(mv), s);
+            const int blk = block_of(W, items), g = (int)((items + blk - 1) / blk);
+            if (n <= kChunkRowsM)
+                WITH_COLS_M(lv.S, (launch_k(pdl, k_down_c<T, IDX, K, kUnrollSmall>, g, blk, s, n, lv.S.sptr, cols,
+                                            P::val(lv), pats, P::xpre(mv), P::b(mv), P::p(lv), P::t(mv), ctl)));
+            else
+                WITH_COLS_M(lv.S, (launch_k(pdl, k_down_m<T, IDX, K, kUnroll, false>, grid_of(items), kMB, s, n,
+                                            lv.S.sptr, cols, P::val(lv), P::xpre(mv), P::b(mv), P::p(lv), P::t(mv),
+                                            ctl)));
+        }
+        const int cblk = block_of(W, citems), cg = (int)((citems + cblk - 1) / cblk);
         if (l + 1 == L)
-            k_restrict_m<T, double, false, K><<<gv(lv.nc), kMB, 0, s>>>(
-                lv.nc, lv.rptr, lv.ridx, P::t(mv), W.bL, nullptr, nullptr, ctl);
+            launch_k(pdl, k_restrict_m<T, double, false, K>, cg, cblk, s, lv.nc, lv.rptr, lv.ridx, P::t(mv), W.bL,
+                     nullptr, nullptr, ctl);
         else
-            k_restrict_m<T, T, true, K><<<gv(lv.nc), kMB, 0, s>>>(
-                lv.nc, lv.rptr, lv.ridx, P::t(mv), P::b(W.lev[l + 1]), P::dinv(lev[l + 1]), P::xpre(W.lev[l + 1]),
-                ctl);
+            launch_k(pdl, k_restrict_m<T, T, true, K>, cg, cblk, s, lv.nc, lv.rptr, lv.ridx, P::t(mv),
+                     P::b(W.lev[l + 1]), P::dinv(lev[l + 1]), P::xpre(W.lev[l + 1]), ctl);
     }
     if (h->coarse_iter)
         PCG_TRY(launch_coarse_iter<T>(h, W.cws, W.bL, P::x(W.lev[L]), &ctl->done, ctl->active, s));
     else
-        k_coarse_m<T, K><<<grid_of((int64_t)h->nL * (K / 2) * 32), kMB, 0, s>>>(h->nL, h->Ainv, W.bL,
-                                                                                P::x(W.lev[L]), ctl);
+        launch_k(pdl, k_coarse_m<T, K>, grid_of((int64_t)lev[L].A.n * (K / 2) * 32), kMB, s, lev[L].A.n,
+                 h->op_first && h->op[L] ? h->op[L] : h->Ainv, W.bL, P::x(W.lev[L]), ctl);
     for (int l = L - 1; l >= 1; l--) {
         Level &lv = lev[l];
         MultiLevel &mv = W.lev[l];
-        int n = lv.A.n;
-        k_prolong_m<T, K><<<gv(n), kMB, 0, s>>>(n, P::xpre(mv), P::p(lv), lv.agg,
-                                                                  P::x(W.lev[l + 1]), P::xp(mv), ctl);
-        if (gs) {
+        const int n = lv.A.n;
+        const int64_t items = (int64_t)n * (K / V);
+        const int blk = block_of(W, items), g = (int)((items + blk - 1) / blk);
+        launch_k(pdl, k_prolong_m<T, K>, g, blk, s, n, P::xpre(mv), P::p(lv), lv.agg, P::x(W.lev[l + 1]), P::xp(mv),
+                 ctl);
+        if (gs)
             launch_gs_m<T, K>(h, W, l, false, P::b(mv), P::x(mv), s);
-            continue;
-        }
-        WITH_COLS_M(lv.S, (k_post_m<T, T, false, false, IDX, K, kUnroll, false>
-                           <<<gv(n), kMB, 0, s>>>(n, lv.S.sptr, cols, P::val(lv), P::xp(mv),
-                                                                    P::b(mv), P::dinv(lv), P::x(mv), nullptr,
-                                                                    nullptr, nullptr, ctl)));
+        else if (n <= kChunkRowsM)
+            WITH_COLS_M(lv.S, (launch_k(pdl, k_post_c<T, IDX, K, kUnrollSmall>, g, blk, s, n, lv.S.sptr, cols,
+                                        P::val(lv), pats, P::xp(mv), P::b(mv), P::dinv(lv), P::x(mv), ctl)));
+        else
+            WITH_COLS_M(lv.S, (launch_k(pdl, k_post_m<T, T, false, false, IDX, K, kUnroll, false>, grid_of(items),
+                                        kMB, s, n, lv.S.sptr, cols, P::val(lv), P::xp(mv), P::b(mv), P::dinv(lv),
+                                        P::x(mv), (const double *)nullptr, (const double *)nullptr,
+                                        (double *)nullptr, ctl)));
     }
-    k_prolong_m<T, K><<<g0, kMB, 0, s>>>(l0.A.n, P::xpre(m0), P::p(l0), l0.agg, P::x(W.lev[1]), P::xp(m0), ctl);
+    launch_k(pdl, k_prolong_m<T, K>, wave_grid(W, k_prolong_m<T, K>, items0), kMB, s, l0.A.n, P::xpre(m0), P::p(l0),
+             l0.agg, P::x(W.lev[1]), P::xp(m0), ctl);
     if (gs) {
         launch_gs_m<T, K>(h, W, 0, false, b0, P::x(m0), s);
-        k_gs_finish0_m<T, FCG, K><<<g0, kMB, 0, s>>>(l0.A.n, (const T *)P::x(m0), W.r, W.q, W.z, W.partials, ctl);
+        launch_k(pdl, k_gs_finish0_m<T, FCG, K>, wave_grid(W, k_gs_finish0_m<T, FCG, K>, items0), kMB, s, l0.A.n,
+                 (const T *)P::x(m0), W.r, W.q, W.z, W.partials, ctl);
         PCG_LAUNCH_CK();
         return AMG_OK;
     }
-    WITH_COLS_M(l0.S, (k_post_m<T, double, true, FCG, IDX, K, kUnroll, true><<<g0, kMB, 0, s>>>(
-                          l0.A.n, l0.S.sptr, cols, P::val(l0), P::xp(m0), b0, P::dinv(l0), W.z, W.r, W.q,
-                          W.partials, ctl)));
+    WITH_COLS_M(l0.S, (launch_k(pdl, k_post_m<T, double, true, FCG, IDX, K, kUnroll, true>,
+                                wave_grid(W, k_post_m<T, double, true, FCG, IDX, K, kUnroll, true>, items0), kMB, s,
+                                l0.A.n, l0.S.sptr, cols, P::val(l0), P::xp(m0), b0, P::dinv(l0), W.z, W.r, W.q,
+                                W.partials, ctl)));
     PCG_LAUNCH_CK();
     return AMG_OK;
+}
+
+// k_residual_m of `mode` (INIT: the pending columns' first residual).
+template <bool INIT, int K>
+void launch_residual_m(amg_hier *h, MultiWS &W, int mode, cudaStream_t s) {
+    Level &l0 = h->lev[0];
+    MultiLevel &m0 = W.lev[0];
+    const int n = l0.A.n;
+    const int64_t items = (int64_t)n * (K / 2);
+#define PCG_RESIDUAL_M(MODE)                                                                                         \
+    WITH_COLS_M(l0.S, (launch_k(h->pdl, k_residual_m<INIT, MODE, IDX, K>,                                           \
+                                wave_grid(W, k_residual_m<INIT, MODE, IDX, K>, items), kMB, s, n, l0.S.sptr, cols,  \
+                                l0.S.v64, W.b, W.x, W.r, W.r32, l0.dinv32, m0.xpre32, l0.dinv, m0.xpre64,           \
+                                W.partials, W.ctl, W.hist, W.hist_cap)))
+    if (mode == AMG_MODE_FCG32) PCG_RESIDUAL_M(AMG_MODE_FCG32);
+    else PCG_RESIDUAL_M(AMG_MODE_PCG64);
+#undef PCG_RESIDUAL_M
 }
 
 template <int K>
 int launch_iteration_m(amg_hier *h, MultiWS &W, int mode, cudaStream_t s) {
     Level &l0 = h->lev[0];
     MultiLevel &m0 = W.lev[0];
-    int n = l0.A.n;
+    const int n = l0.A.n;
+    const int64_t items = (int64_t)n * (K / 2);
     if (mode == AMG_MODE_FCG32) PCG_TRY((launch_vcycle_m<float, true, K>(h, W, s)));
     else if (h->coarse_iter) PCG_TRY((launch_vcycle_m<double, true, K>(h, W, s)));  // flexible: FCG(1) beta
     else PCG_TRY((launch_vcycle_m<double, false, K>(h, W, s)));
-    k_axpy_m<K><<<W.grid, kMB, 0, s>>>(n, W.z, W.p, W.ctl);
-    WITH_COLS_M(l0.S, (k_spmm_m<IDX, K><<<W.grid, kMB, 0, s>>>(n, l0.S.sptr, cols, l0.S.v64, W.p, W.q, W.partials,
-                                                               W.ctl)));
-    int hs = W.hist_cap;
-    if (mode == AMG_MODE_FCG32) {
-        k_update_m<AMG_MODE_FCG32, K><<<W.grid, kMB, 0, s>>>(n, W.p, W.q, W.x, W.r, W.r32, l0.dinv32, m0.xpre32,
-                                                             l0.dinv, m0.xpre64, W.partials, W.ctl, W.hist, hs);
-        WITH_COLS_M(l0.S, (k_residual_m<false, AMG_MODE_FCG32, IDX, K><<<W.grid, kMB, 0, s>>>(
-                              n, l0.S.sptr, cols, l0.S.v64, W.b, W.x, W.r, W.r32, l0.dinv32, m0.xpre32, l0.dinv,
-                              m0.xpre64, W.partials, W.ctl, W.hist, hs)));
-    } else {
-        k_update_m<AMG_MODE_PCG64, K><<<W.grid, kMB, 0, s>>>(n, W.p, W.q, W.x, W.r, W.r32, l0.dinv32, m0.xpre32,
-                                                             l0.dinv, m0.xpre64, W.partials, W.ctl, W.hist, hs);
-        WITH_COLS_M(l0.S, (k_residual_m<false, AMG_MODE_PCG64, IDX, K><<<W.grid, kMB, 0, s>>>(
-                              n, l0.S.sptr, cols, l0.S.v64, W.b, W.x, W.r, W.r32, l0.dinv32, m0.xpre32, l0.dinv,
-                              m0.xpre64, W.partials, W.ctl, W.hist, hs)));
-    }
+    launch_k(h->pdl, k_axpy_m<K>, wave_grid(W, k_axpy_m<K>, items), kMB, s, n, W.z, W.p, W.ctl);
+    WITH_COLS_M(l0.S, (launch_k(h->pdl, k_spmm_m<IDX, K>, wave_grid(W, k_spmm_m<IDX, K>, items), kMB, s, n, l0.S.sptr,
+                                cols, l0.S.v64, W.p, W.q, W.partials, W.ctl)));
+    // half a wave of the update: its partials are what its last block reads
+    if (mode == AMG_MODE_FCG32)
+        launch_k(h->pdl, k_update_m<AMG_MODE_FCG32, K>, (wave_grid(W, k_update_m<AMG_MODE_FCG32, K>, items) + 1) / 2,
+                 kMB, s, n, W.p, W.q, W.x, W.r, W.r32, l0.dinv32, m0.xpre32, l0.dinv, m0.xpre64, W.partials, W.ctl,
+                 W.hist, W.hist_cap);
+    else
+        launch_k(h->pdl, k_update_m<AMG_MODE_PCG64, K>, (wave_grid(W, k_update_m<AMG_MODE_PCG64, K>, items) + 1) / 2,
+                 kMB, s, n, W.p, W.q, W.x, W.r, W.r32, l0.dinv32, m0.xpre32, l0.dinv, m0.xpre64, W.partials, W.ctl,
+                 W.hist, W.hist_cap);
+    launch_residual_m<false, K>(h, W, mode, s);
     PCG_LAUNCH_CK();
     return AMG_OK;
 }
@@ -997,18 +1184,7 @@ int launch_iteration_m(amg_hier *h, MultiWS &W, int mode, cudaStream_t s) {
 // First residual, ||b|| and state of the pending columns only.
 template <int K>
 int launch_init_residual_m(amg_hier *h, MultiWS &W, int mode, cudaStream_t s) {
-    Level &l0 = h->lev[0];
-    MultiLevel &m0 = W.lev[0];
-    int n = l0.A.n;
-    int hs = W.hist_cap;
-    if (mode == AMG_MODE_FCG32)
-        WITH_COLS_M(l0.S, (k_residual_m<true, AMG_MODE_FCG32, IDX, K><<<W.grid, kMB, 0, s>>>(
-                              n, l0.S.sptr, cols, l0.S.v64, W.b, W.x, W.r, W.r32, l0.dinv32, m0.xpre32, l0.dinv,
-                              m0.xpre64, W.partials, W.ctl, W.hist, hs)));
-    else
-        WITH_COLS_M(l0.S, (k_residual_m<true, AMG_MODE_PCG64, IDX, K><<<W.grid, kMB, 0, s>>>(
-                              n, l0.S.sptr, cols, l0.S.v64, W.b, W.x, W.r, W.r32, l0.dinv32, m0.xpre32, l0.dinv,
-                              m0.xpre64, W.partials, W.ctl, W.hist, hs)));
+    launch_residual_m<true, K>(h, W, mode, s);
     PCG_LAUNCH_CK();
     return AMG_OK;
 }
@@ -1234,11 +1410,12 @@ int mws_alloc(amg_hier *h, Mem &M, MultiWS &W, int K, int hist_cap, int which) {
             PCG_TRY(alloc(M, &v.xp64, m));
         }
     }
-    PCG_TRY(alloc(M, &W.bL, (int64_t)h->nL * K));
+    PCG_TRY(alloc(M, &W.bL, (int64_t)h->lev[direct_level_m(h, K)].A.n * K));
     W.flex = h->coarse_iter;
     if (h->coarse_iter) PCG_TRY(cws_alloc(h, M, W.cws, K));
     int sms = 0;
     PCG_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
+    W.sms = sms;
     int64_t want = (nk + kMB - 1) / kMB;
     int64_t cap = (int64_t)sms * 8;
     W.grid = (int)(want < cap ? want : cap);

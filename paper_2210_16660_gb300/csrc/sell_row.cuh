@@ -181,6 +181,33 @@ struct SellRow {
         }
         return acc;
     }
+
+    // The same product for V columns at once: xvec(j, x) reads x_j's V values.
+    template <int V, typename F>
+    __device__ __forceinline__ void dot_vec(int row, F xvec, T (&acc)[V]) {
+#pragma unroll
+        for (int q = 0; q < V; q++) acc[q] = 0;
+        for (int k = 0; k < w; k += U) {
+            T x[U][V];
+#pragma unroll
+            for (int u = 0; u < U; u++)
+                if (k + u < w) xvec(j[u], x[u]);
+            int jn[U];
+            T vn[U];
+            chunk(k + U, row, jn, vn);
+#pragma unroll
+            for (int u = 0; u < U; u++)
+                if (k + u < w) {
+#pragma unroll
+                    for (int q = 0; q < V; q++) acc[q] += v[u] * x[u][q];
+                }
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                j[u] = jn[u];
+                v[u] = vn[u];
+            }
+        }
+    }
 };
 
 // Rows of level-0 slices stored with a shared offset pattern and at most

@@ -82,3 +82,23 @@ def test_small_levels_as_one_matrix(N, kw, nu, rows, mode):
         assert (x1 - x2).norm().item() <= 1e-6 * x2.norm().item()
     for a in amgs:
         a.close()
+
+
+@pytest.mark.parametrize("mode", ["pcg64", "fcg32"])
+@pytest.mark.parametrize("N,k,env", [(13, 3, ()), (28, 9, (("PCGAMG_UNIFORM", "0"),)), (28, 20, (("PCGAMG_COL16", "0"),)),
+                                     (33, 32, ()), (41, 5, ())])
+def test_columns_agree_with_single_solves(N, k, env, mode):
+    """The coarse levels' multi-column kernels and the explicit operator (whose
+    level depends on the column count) against each column solved alone."""
+    prob = W.make_problem(N, 1.04, seed=5)
+    Bm, _ = W.make_rhs(prob, k, seed=77)
+    Bd = torch.from_numpy(np.ascontiguousarray(Bm)).cuda()
+    amg = _amg(prob.A, env, mode=mode)
+    X = torch.zeros_like(Bd)
+    st, it, _, sts, tr = amg.solve_multi(Bd, X, rtol=1e-8)
+    assert st == 0 and not sts.any() and (tr <= 1e-8).all()
+    for c in (0, k // 2, k - 1):
+        r, x = _solve(amg, Bd[:, c].contiguous())
+        assert abs(r.iters - int(it[c])) <= 1
+        assert (x - X[:, c]).norm().item() <= 1e-6 * x.norm().item()
+    amg.close()
