@@ -3,6 +3,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <iterator>
 #include <new>
 
 #include "internal.cuh"
@@ -28,9 +29,42 @@ static amg_alloc_fn g_alloc = nullptr;
 static amg_free_fn g_free = nullptr;
 static void *g_alloc_ctx = nullptr;
 
+// No arena under a byte budget (its one request could fail where the
+// temporaries one after another fit) or when the allocation fails.
+void Mem::arena_begin(size_t n) {
+    if (budget || dry || arena) return;
+    void *q = nullptr;
+    n = (n + 255) & ~(size_t)255;
+    if (alloc_bytes(&q, n)) {
+        set_error("");
+        return;
+    }
+    arena = static_cast<char *>(q);
+    arena_free[0] = n;
+}
+
+void Mem::arena_end() {
+    char *q = arena;
+    arena = nullptr;
+    arena_free.clear();
+    arena_live.clear();
+    if (q) release(q);
+}
+
 int Mem::alloc_bytes(void **p, size_t n) {
     *p = nullptr;
     n = (n + 255) & ~(size_t)255;
+    if (arena) {
+        for (auto it = arena_free.begin(); it != arena_free.end(); ++it) {
+            if (it->second < n) continue;
+            const size_t at = it->first, left = it->second - n;
+            arena_free.erase(it);
+            if (left) arena_free[at + n] = left;
+            *p = arena + at;
+            arena_live[*p] = n;
+            return AMG_OK;
+        }
+    }
     if (budget && bytes + n > budget) {
         set_error("device memory budget exceeded (%zu + %zu > %zu bytes)", bytes, n, budget);
         return AMG_ERR_OOM;
@@ -65,6 +99,25 @@ int Mem::alloc_bytes(void **p, size_t n) {
 }
 
 void Mem::release(void *p) {
+    auto al = arena_live.find(p);
+    if (al != arena_live.end()) {
+        size_t at = (size_t)(static_cast<char *>(p) - arena), n = al->second;
+        arena_live.erase(al);
+        auto next = arena_free.lower_bound(at);
+        if (next != arena_free.end() && next->first == at + n) {
+            n += next->second;
+            next = arena_free.erase(next);
+        }
+        if (next != arena_free.begin()) {
+            auto prev = std::prev(next);
+            if (prev->first + prev->second == at) {
+                prev->second += n;
+                return;
+            }
+        }
+        arena_free[at] = n;
+        return;
+    }
     auto it = live.find(p);
     if (it == live.end()) return;
     bytes -= it->second;
@@ -79,6 +132,9 @@ void Mem::release_all() {
         else cudaFree(kv.first);
     }
     live.clear();
+    arena = nullptr;
+    arena_free.clear();
+    arena_live.clear();
     bytes = 0;
 }
 

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <map>
 #include <string>
 #include <unordered_map>
 #include <vector>
@@ -85,6 +86,15 @@ struct Mem {
     size_t bytes = 0, peak = 0, budget = 0;
     bool dry = false;  // count requests (rounded as real ones) without allocating
     std::unordered_map<void *, size_t> live;
+    // Arena of one call's temporaries (amg_refresh: all on one stream, so a
+    // released range may be handed out again at once): requests are served
+    // from one allocation, first fit, until arena_end gives it back. A request
+    // that does not fit goes to the allocator.
+    char *arena = nullptr;
+    std::map<size_t, size_t> arena_free;              // offset -> bytes, disjoint and not adjacent
+    std::unordered_map<void *, size_t> arena_live;
+    void arena_begin(size_t bytes);
+    void arena_end();
     int alloc_bytes(void **p, size_t bytes);
     void release(void *p);
     void release_all();

@@ -332,17 +332,20 @@ __global__ void k_rap_count(int nc, const int32_t *__restrict__ mem0, const int3
 // Coarse row I of P^T A P for a pairwise aggregation: every stored a_ij with
 // i in G_I and agg(j) >= 0 contributes t = a_ij * (p_i * p_j) to entry
 // (I, agg(j)); contributions to one entry are added in increasing order of
-// (min(i,j), max(i,j)). Terms are kept sorted by (J, min, max) in the row's
-// scratch segment (insertion sort, stable), then runs are summed in place.
-__global__ void k_rap_terms(int nc, const int32_t *__restrict__ mem0, const int32_t *__restrict__ mem1,
-                            const int32_t *__restrict__ rp, const int32_t *__restrict__ ci,
-                            const double *__restrict__ v, const int32_t *__restrict__ agg,
-                            const double *__restrict__ p, const int32_t *__restrict__ off,
-                            int32_t *__restrict__ tJ, unsigned long long *__restrict__ tK,
-                            double *__restrict__ tT, int32_t *__restrict__ ucnt) {
-    int I = blockIdx.x * blockDim.x + threadIdx.x;
-    if (I >= nc) return;
-    int32_t base = off[I];
+// (min(i,j), max(i,j)). tJ/tT receive the row's distinct columns and sums in
+// the row's segment, ucnt their count.
+//
+// One warp per coarse row: its terms (two fine rows, at most kRapCap) sit in
+// shared memory, a lane counts each of its terms' rank among them, and the
+// head of each run of equal columns adds its run in order. (One thread per row
+// sorting in global memory was 3.9 of the 7.0 ms of device time that a refresh of the
+// 56^3 system took.) Longer rows are sorted by one lane in the scratch segment.
+constexpr int kRapWarps = 4, kRapCap = 128;
+
+// The row's terms by stable insertion sort in global scratch.
+__device__ int rap_insertion(int I, const int32_t *mem0, const int32_t *mem1, const int32_t *rp, const int32_t *ci,
+                             const double *v, const int32_t *agg, const double *p, int32_t base, int32_t *tJ,
+                             unsigned long long *tK, double *tT) {
     int m = 0;
     int mem[2] = {mem0[I], mem1[I]};
     for (int q = 0; q < 2; q++) {
@@ -379,16 +382,94 @@ __global__ void k_rap_terms(int nc, const int32_t *__restrict__ mem0, const int3
             tT[base + u - 1] = __dadd_rn(tT[base + u - 1], t);
         }
     }
-    ucnt[I] = u;
+    return u;
+}
+
+__global__ void __launch_bounds__(32 * kRapWarps) k_rap_terms(
+    int nc, const int32_t *__restrict__ mem0, const int32_t *__restrict__ mem1, const int32_t *__restrict__ rp,
+    const int32_t *__restrict__ ci, const double *__restrict__ v, const int32_t *__restrict__ agg,
+    const double *__restrict__ p, const int32_t *__restrict__ off, int32_t *__restrict__ tJ,
+    unsigned long long *__restrict__ tK, double *__restrict__ tT, int32_t *__restrict__ ucnt) {
+    __shared__ int sJ[kRapWarps][kRapCap];
+    __shared__ unsigned long long sK[kRapWarps][kRapCap];
+    __shared__ double sT[kRapWarps][kRapCap];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int I = blockIdx.x * kRapWarps + w;
+    if (I >= nc) return;
+    const int i0 = mem0[I], i1 = mem1[I];
+    const int32_t b0 = rp[i0], b1 = i1 >= 0 ? rp[i1] : 0;
+    const int n0 = rp[i0 + 1] - b0, m = n0 + (i1 >= 0 ? rp[i1 + 1] - b1 : 0);
+    const int32_t base = off[I];
+    if (m > kRapCap) {  // the whole warp
+        if (lane == 0) ucnt[I] = rap_insertion(I, mem0, mem1, rp, ci, v, agg, p, base, tJ, tK, tT);
+        return;
+    }
+    constexpr int kMine = kRapCap / 32;
+    int J[kMine];
+    unsigned long long K[kMine];
+    double T[kMine];
+    const double p0 = p[i0], p1 = i1 >= 0 ? p[i1] : 0.0;
+    int valid = 0;
+#pragma unroll
+    for (int t = 0; t < kMine; t++) {
+        const int e = lane + 32 * t;
+        J[t] = INT32_MAX;  // a column left out of the coarse space sorts last
+        K[t] = 0;
+        T[t] = 0.0;
+        if (e < m) {
+            const int i = e < n0 ? i0 : i1;
+            const int32_t k = e < n0 ? b0 + e : b1 + (e - n0);
+            const int j = ci[k], a = agg[j];
+            if (a >= 0) J[t] = a;
+            K[t] = ((unsigned long long)(unsigned)min(i, j) << 32) | (unsigned long long)(unsigned)max(i, j);
+            T[t] = __dmul_rn(v[k], __dmul_rn(e < n0 ? p0 : p1, p[j]));
+            sJ[w][e] = J[t];
+            sK[w][e] = K[t];
+        }
+        valid += __popc(__ballot_sync(0xffffffffu, e < m && J[t] != INT32_MAX));
+    }
+    __syncwarp();
+    int r[kMine] = {};
+    for (int f = 0; f < m; f++) {
+        const int Jf = sJ[w][f];
+        const unsigned long long Kf = sK[w][f];
+#pragma unroll
+        for (int t = 0; t < kMine; t++)
+            r[t] += Jf < J[t] || (Jf == J[t] && (Kf < K[t] || (Kf == K[t] && f < lane + 32 * t))) ? 1 : 0;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int t = 0; t < kMine; t++)
+        if (lane + 32 * t < m) {
+            sJ[w][r[t]] = J[t];
+            sT[w][r[t]] = T[t];
+        }
+    __syncwarp();
+    int u = 0;
+#pragma unroll
+    for (int t = 0; t < kMine; t++) {
+        const int e = lane + 32 * t;
+        const bool head = e < valid && (e == 0 || sJ[w][e] != sJ[w][e - 1]);
+        const unsigned heads = __ballot_sync(0xffffffffu, head);
+        if (head) {
+            double s = sT[w][e];
+            for (int f = e + 1; f < valid && sJ[w][f] == sJ[w][e]; f++) s = __dadd_rn(s, sT[w][f]);
+            const int at = base + u + __popc(heads & ((1u << lane) - 1u));
+            tJ[at] = sJ[w][e];
+            tT[at] = s;
+        }
+        u += __popc(heads);
+    }
+    if (lane == 0) ucnt[I] = u;
 }
 
 __global__ void k_rap_copy(int nc, const int32_t *__restrict__ off, const int32_t *__restrict__ rpc,
                            const int32_t *__restrict__ tJ, const double *__restrict__ tT,
                            int32_t *__restrict__ cic, double *__restrict__ vc) {
-    int I = blockIdx.x * blockDim.x + threadIdx.x;
+    const int I = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (I >= nc) return;
     int32_t o = off[I], s = rpc[I], e = rpc[I + 1];
-    for (int32_t q = 0; q < e - s; q++) {
+    for (int32_t q = lane; q < e - s; q += 32) {
         cic[s + q] = tJ[o + q];
         vc[s + q] = tT[o + q];
     }
@@ -609,57 +690,85 @@ __global__ void k_dense(int n, const int32_t *__restrict__ rp, const int32_t *__
     for (int32_t k = rp[i]; k < rp[i + 1]; k++) ad[(int64_t)i * n + ci[k]] = v[k];
 }
 
-// In-place Cholesky (lower triangle, row-major) by one block; flag = 1 when
-// a pivot is not positive.
-__global__ void k_chol(int n, double *a, int *flag) {
-    __shared__ double red[1024];
-    __shared__ double piv;
-    for (int j = 0; j < n; j++) {
-        double s = 0.0;
-        for (int k = threadIdx.x; k < j; k += blockDim.x) s += a[(int64_t)j * n + k] * a[(int64_t)j * n + k];
-        red[threadIdx.x] = s;
+// Inverse of the dense SPD matrix A (n x n, row-major) in place by block
+// Gauss-Jordan elimination over diagonal blocks of kGj rows, float64, no
+// pivoting. For each block column k: D = A_kk^-1 (k_gj_diag), R_j = D A_kj and
+// a copy C_i of A_ik (k_gj_panel), then A_ij -= C_i R_j, A_ik = -C_i D,
+// A_kj = R_j, A_kk = D (k_gj_update). The pivots are those of the Cholesky
+// factorization, squared; flag is set when one is not positive. Three launches
+// per block column instead of one block's column-by-column factorization and a
+// triangular solve per unit vector (127 rows: 2.15 ms; 3,483 rows: 3.3 s).
+constexpr int kGj = 32;
+__global__ void __launch_bounds__(kGj * kGj) k_gj_diag(int n, int k0, const double *__restrict__ A,
+                                                       double *__restrict__ D, int *flag) {
+    __shared__ double a[kGj][kGj + 1];
+    const int i = threadIdx.y, j = threadIdx.x;
+    // rows past the end: identity
+    double x = k0 + i < n && k0 + j < n ? A[(int64_t)(k0 + i) * n + k0 + j] : (i == j ? 1.0 : 0.0);
+    for (int k = 0; k < kGj; k++) {
+        a[i][j] = x;
         __syncthreads();
-        for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-            if (threadIdx.x < (unsigned)o) red[threadIdx.x] += red[threadIdx.x + o];
-            __syncthreads();
+        double piv = a[k][k];
+        if (!(piv > 0.0)) {
+            if (i == 0 && j == 0) atomicOr(flag, 1);
+            piv = 1.0;
         }
-        if (threadIdx.x == 0) {
-            double d = a[(int64_t)j * n + j] - red[0];
-            if (!(d > 0.0)) { *flag = 1; d = 1.0; }
-            piv = sqrt(d);
-            a[(int64_t)j * n + j] = piv;
-        }
-        __syncthreads();
-        for (int i = j + 1 + threadIdx.x; i < n; i += blockDim.x) {
-            double t = a[(int64_t)i * n + j];
-            for (int k = 0; k < j; k++) t -= a[(int64_t)i * n + k] * a[(int64_t)j * n + k];
-            a[(int64_t)i * n + j] = t / piv;
-        }
+        const double q = 1.0 / piv, r = a[k][j] * q, c = a[i][k];
+        if (i == k) x = j == k ? q : r;
+        else x = j == k ? -c * q : fma(-c, r, x);
         __syncthreads();
     }
+    D[i * kGj + j] = x;
 }
 
-// Column c of A^{-1} = L^{-T} L^{-1} e_c by one block per column.
-__global__ void k_chol_inverse(int n, const double *__restrict__ L, double *__restrict__ ainv) {
-    extern __shared__ double y[];
-    int c = blockIdx.x;
-    for (int k = threadIdx.x; k < n; k += blockDim.x) y[k] = k == c ? 1.0 : 0.0;
+// R (kGj x n): rows k0.. of D A; C (n x kGj): columns k0.. of A. One thread per
+// (panel row, column j); the panel's rows past n are zero.
+__global__ void __launch_bounds__(256) k_gj_panel(int n, int k0, const double *__restrict__ A,
+                                                  const double *__restrict__ D, double *__restrict__ R,
+                                                  double *__restrict__ C) {
+    __shared__ double d[kGj][kGj];
+    for (int t = threadIdx.x; t < kGj * kGj; t += blockDim.x) d[t / kGj][t % kGj] = D[t];
     __syncthreads();
-    for (int i = 0; i < n; i++) {           // L y = e_c
-        double yi = y[i] / L[(int64_t)i * n + i];
-        __syncthreads();
-        if (threadIdx.x == 0) y[i] = yi;
-        for (int k = i + 1 + threadIdx.x; k < n; k += blockDim.x) y[k] -= L[(int64_t)k * n + i] * yi;
-        __syncthreads();
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    double col[kGj];
+#pragma unroll
+    for (int t = 0; t < kGj; t++) col[t] = k0 + t < n ? A[(int64_t)(k0 + t) * n + j] : 0.0;
+#pragma unroll 4
+    for (int i = 0; i < kGj; i++) {
+        double s = 0.0;
+#pragma unroll
+        for (int t = 0; t < kGj; t++) s = fma(d[i][t], col[t], s);
+        R[(int64_t)i * n + j] = s;
     }
-    for (int i = n - 1; i >= 0; i--) {      // L^T x = y
-        double xi = y[i] / L[(int64_t)i * n + i];
-        __syncthreads();
-        if (threadIdx.x == 0) y[i] = xi;
-        for (int k = threadIdx.x; k < i; k += blockDim.x) y[k] -= L[(int64_t)i * n + k] * xi;
-        __syncthreads();
+    for (int t = 0; t < kGj; t++) C[(int64_t)j * kGj + t] = k0 + t < n ? A[(int64_t)j * n + k0 + t] : 0.0;
+}
+
+// One 32 x 32 tile of A per block of 32 x 8 threads.
+__global__ void __launch_bounds__(256) k_gj_update(int n, int k0, const double *__restrict__ R,
+                                                   const double *__restrict__ C, const double *__restrict__ D,
+                                                   double *__restrict__ A) {
+    __shared__ double c[kGj][kGj + 1], r[kGj][kGj + 1];
+    const int ti = blockIdx.y * kGj, tj = blockIdx.x * kGj, x = threadIdx.x, y0 = threadIdx.y;
+    const bool krow = ti == k0, kcol = tj == k0;
+    for (int y = y0; y < kGj; y += 8) {
+        c[y][x] = ti + y < n ? C[(int64_t)(ti + y) * kGj + x] : 0.0;
+        r[y][x] = kcol ? D[y * kGj + x] : (tj + x < n ? R[(int64_t)y * n + tj + x] : 0.0);
     }
-    for (int k = threadIdx.x; k < n; k += blockDim.x) ainv[(int64_t)k * n + c] = y[k];
+    __syncthreads();
+    for (int y = y0; y < kGj; y += 8) {
+        const int i = ti + y, j = tj + x;
+        if (i >= n || j >= n) continue;
+        double v;
+        if (krow) {
+            v = r[y][x];  // D or R
+        } else {
+            v = kcol ? 0.0 : A[(int64_t)i * n + j];
+#pragma unroll
+            for (int t = 0; t < kGj; t++) v = fma(-c[y][t], r[t][x], v);
+        }
+        A[(int64_t)i * n + j] = v;
+    }
 }
 
 // ------------------------------------------------------------ partial reuse
@@ -824,6 +933,35 @@ void free_csr(Mem &M, DevCSR &a) {
     release(M, a.v);
 }
 
+// The coarsest matrix's dense inverse into h->Ainv; *bad: a pivot was not
+// positive (not SPD).
+int dense_inverse(amg_hier *h, const DevCSR &a, int *bad, cudaStream_t s) {
+    Mem &M = h->mem;
+    const int n = a.n;
+    double *D = nullptr, *R = nullptr, *C = nullptr;
+    int *dflag = nullptr;
+    PCG_TRY(alloc(M, &dflag, 1));
+    PCG_TRY(alloc(M, &D, kGj * kGj));
+    PCG_TRY(alloc(M, &R, (size_t)kGj * n));
+    PCG_TRY(alloc(M, &C, (size_t)kGj * n));
+    PCG_CK(cudaMemsetAsync(h->Ainv, 0, sizeof(double) * (size_t)n * n, s));
+    PCG_CK(cudaMemsetAsync(dflag, 0, sizeof(int), s));
+    k_dense<<<grid_for(n), kBlock, 0, s>>>(n, a.rp, a.ci, a.v, h->Ainv);
+    const unsigned tiles = (unsigned)((n + kGj - 1) / kGj);
+    for (int k0 = 0; k0 < n; k0 += kGj) {
+        k_gj_diag<<<1, dim3(kGj, kGj), 0, s>>>(n, k0, h->Ainv, D, dflag);
+        k_gj_panel<<<(n + 255) / 256, 256, 0, s>>>(n, k0, h->Ainv, D, R, C);
+        k_gj_update<<<dim3(tiles, tiles), dim3(kGj, 8), 0, s>>>(n, k0, R, C, D, h->Ainv);
+    }
+    PCG_LAUNCH_CK();
+    PCG_TRY(read_flag(dflag, s, bad));
+    release(M, dflag);
+    release(M, D);
+    release(M, R);
+    release(M, C);
+    return AMG_OK;
+}
+
 // Galerkin product P^T cur P of one pairwise pass (aggregate members mem0 <
 // mem1, -1 = singleton; map agg; weights p) into a new CSR matrix c.
 int galerkin(amg_hier *h, const DevCSR &cur, const int32_t *agg, const double *p, const int32_t *mem0,
@@ -843,8 +981,8 @@ int galerkin(amg_hier *h, const DevCSR &cur, const int32_t *agg, const double *p
     PCG_TRY(alloc(M, &tK, nterm));
     PCG_TRY(alloc(M, &tT, nterm));
     PCG_TRY(alloc(M, &ucnt, nc));
-    k_rap_terms<<<grid_for(nc, 128), 128, 0, s>>>(nc, mem0, mem1, cur.rp, cur.ci, cur.v, agg, p, off, tJ,
-                                                   tK, tT, ucnt);
+    k_rap_terms<<<(unsigned)std::max(1, (nc + kRapWarps - 1) / kRapWarps), 32 * kRapWarps, 0, s>>>(
+        nc, mem0, mem1, cur.rp, cur.ci, cur.v, agg, p, off, tJ, tK, tT, ucnt);
     PCG_LAUNCH_CK();
     DevCSR c;
     c.n = nc;
@@ -854,7 +992,7 @@ int galerkin(amg_hier *h, const DevCSR &cur, const int32_t *agg, const double *p
     c.nnz = nzc;
     PCG_TRY(alloc(M, &c.ci, nzc));
     PCG_TRY(alloc(M, &c.v, nzc));
-    k_rap_copy<<<grid_for(nc), kBlock, 0, s>>>(nc, off, c.rp, tJ, tT, c.ci, c.v);
+    k_rap_copy<<<grid_for((int64_t)nc * 32), kBlock, 0, s>>>(nc, off, c.rp, tJ, tT, c.ci, c.v);
     PCG_LAUNCH_CK();
     PCG_CK(cudaStreamSynchronize(s));
     release(M, tJ);
@@ -1305,26 +1443,12 @@ int setup_impl(amg_hier *h, const amg_csr *A, const amg_params *prm, cudaStream_
         h->setup_ms[3] = h->setup_ms[0] - t_match - t_rap;
         return AMG_OK;
     }
-    double *ad = nullptr;
-    PCG_TRY(alloc(M, &ad, (size_t)nL * nL));
     PCG_TRY(alloc(M, &h->Ainv, (size_t)nL * nL));
-    PCG_TRY(alloc(M, &dflag, 1));
-    PCG_CK(cudaMemsetAsync(ad, 0, sizeof(double) * (size_t)nL * nL, s));
-    PCG_CK(cudaMemsetAsync(dflag, 0, sizeof(int), s));
-    k_dense<<<grid_for(nL), kBlock, 0, s>>>(nL, lc.A.rp, lc.A.ci, lc.A.v, ad);
-    k_chol<<<1, 256, 0, s>>>(nL, ad, dflag);
-    PCG_LAUNCH_CK();
-    PCG_TRY(read_flag(dflag, s, &flag));
-    release(M, dflag);
+    PCG_TRY(dense_inverse(h, lc.A, &flag, s));
     if (flag) {
-        release(M, ad);
         set_error("amg_setup: coarsest matrix is not SPD (Cholesky pivot <= 0)");
         return AMG_ERR_BREAKDOWN;
     }
-    k_chol_inverse<<<nL, 256, sizeof(double) * nL, s>>>(nL, ad, h->Ainv);
-    PCG_LAUNCH_CK();
-    PCG_CK(cudaStreamSynchronize(s));
-    release(M, ad);
     PCG_TRY(alloc_solve_workspace(h));
     PCG_TRY(ops_build(h, 0, 0, s));
     PCG_CK(cudaStreamSynchronize(s));
@@ -1342,7 +1466,24 @@ int setup_impl(amg_hier *h, const amg_csr *A, const amg_params *prm, cudaStream_
 // and the coarsest inverse. Every array keeps its address, so captured solve
 // graphs, batch graphs and serving engines stay valid. Nothing is changed
 // when the input is rejected (AMG_ERR_ARG).
+// Its temporaries come from one allocation (Mem::arena): the new CSR, then a
+// pass's terms (20 bytes per fine entry) and coarse matrix.
+int refresh_in_arena(amg_hier *h, const amg_csr *A, cudaStream_t s);
 int refresh_impl(amg_hier *h, const amg_csr *A, cudaStream_t s) {
+    Mem &M = h->mem;
+    const Level &l0 = h->lev[0];
+    M.stream = s;
+    if (!h->smoothed && A && A->n == l0.A.n && A->nnz == l0.A.nnz)
+        M.arena_begin(36 * (size_t)l0.A.nnz + 96 * (size_t)l0.A.n + ((size_t)1 << 20));
+    int st = refresh_in_arena(h, A, s);
+    if (M.arena) {
+        cudaStreamSynchronize(s);  // no kernel may still read what goes back
+        M.arena_end();
+    }
+    return st;
+}
+
+int refresh_in_arena(amg_hier *h, const amg_csr *A, cudaStream_t s) {
     double t_begin = now_ms();
     Mem &M = h->mem;
     M.stream = s;
@@ -1501,25 +1642,13 @@ int refresh_impl(amg_hier *h, const amg_csr *A, cudaStream_t s) {
         h->refresh_ms = now_ms() - t_begin;
         return AMG_OK;
     }
-    double *ad = nullptr;
-    PCG_TRY(alloc(M, &ad, (size_t)nL * nL));
-    PCG_CK(cudaMemsetAsync(ad, 0, sizeof(double) * (size_t)nL * nL, s));
-    PCG_CK(cudaMemsetAsync(dflag, 0, sizeof(int), s));
-    k_dense<<<grid_for(nL), kBlock, 0, s>>>(nL, lc.A.rp, lc.A.ci, lc.A.v, ad);
-    k_chol<<<1, 256, 0, s>>>(nL, ad, dflag);
-    PCG_LAUNCH_CK();
-    PCG_TRY(read_flag(dflag, s, &flag));
     release(M, dflag);
+    PCG_TRY(dense_inverse(h, lc.A, &flag, s));
     if (flag) {
-        release(M, ad);
         set_error("amg_refresh: coarsest matrix is not SPD (Cholesky pivot <= 0); the handle refuses "
                   "solves until a refresh succeeds");
         return AMG_ERR_BREAKDOWN;
     }
-    k_chol_inverse<<<nL, 256, sizeof(double) * nL, s>>>(nL, ad, h->Ainv);
-    PCG_LAUNCH_CK();
-    PCG_CK(cudaStreamSynchronize(s));
-    release(M, ad);
     PCG_TRY(refresh_smem_tail(h));
     PCG_TRY(ops_build(h, h->gs_nu, h->gs_blocks, s));
     PCG_CK(cudaStreamSynchronize(s));
