@@ -25,11 +25,13 @@
 // has stopped in every column returns at once. Reductions are two-stage and
 // deterministic (block partials, summed in block order by the last block).
 // K columns (multi right-hand-side solves) run side by side, each with its
-// own scalars and stop; a thread owns KC = 1 or 2 adjacent columns of a row.
+// own scalars and stop; a thread owns KC = 2 adjacent columns of a row. A single
+// column has kernels of its own (k_cinit1, k_cq1, k_cx1).
 #include <cmath>
 #include <cstdio>
 
 #include "internal.cuh"
+#include "reduce.cuh"
 
 namespace pcgamg {
 
@@ -558,6 +560,309 @@ __global__ void __launch_bounds__(kCT) k_cx(int n, int nb, int K, const double *
     }
 }
 
+// ------------------------------------------------- one column (solves)
+// The same iteration for a single right-hand side, where each kernel is a few
+// microseconds of latency: a block's sums run on the integer pipe, the kernel
+// that needs a scalar adds the partials itself (no fence, ticket or last
+// block), all loads are requested before the first is used, and the float64
+// work is spread over the schedulers, which issue one float64 warp instruction
+// in 64 clocks (a 32 x 32 block apply is 32 of them in one warp, 8 in each of
+// four). 64^3 system stalled at 4,162 rows: 14.1 ms a solve with the kernels
+// above, 12.3 with these; a kernel that finds the solve stopped takes 1.2 us.
+// ctl->any: whether the solve goes on; ctl->bn[0]: (tol ||b||)^2. Block 0
+// records the state; what another block may be writing is used by one thread.
+constexpr int kC1 = 128;  // threads: four warps
+
+// Start: x = 0, r = b, z = M^{-1} b; partial sums of b.b and r.z.
+template <typename TO>
+__global__ void __launch_bounds__(kC1) k_cinit1(int n, int nb, const double *__restrict__ bL, TO *__restrict__ xo,
+                                                double *__restrict__ x, double *__restrict__ r,
+                                                double *__restrict__ z, const double *__restrict__ Minv,
+                                                double *__restrict__ partials, CCtl *ctl, const int *outer_done) {
+    __shared__ double zp[4][kB];
+    __shared__ int stop;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    pdl_enter();
+    if (threadIdx.x == 0) {
+        stop = __ldcg(outer_done);
+        if (blockIdx.x == 0) ctl->any = stop ? 0 : 1;
+    }
+    __syncthreads();
+    if (stop) return;
+    double acc[2] = {};
+    for (int b = blockIdx.x; b < nb; b += gridDim.x) {
+        const int i = b * kB + lane;
+        const double *Mb = Minv + (int64_t)b * kB * kB;
+        const double bv = i < n ? __ldg(bL + i) : 0.0;
+        double t = 0.0;
+#pragma unroll
+        for (int k = 0; k < 8; k++)
+            t = fma(__ldg(Mb + (8 * w + k) * kB + lane), __shfl_sync(0xffffffffu, bv, 8 * w + k), t);
+        zp[w][lane] = t;
+        __syncthreads();
+        if (w == 0) {
+            const double zv = (zp[0][lane] + zp[1][lane]) + (zp[2][lane] + zp[3][lane]);
+            x[i] = 0.0;
+            r[i] = bv;
+            z[i] = zv;
+            if (i < n) xo[i] = (TO)0;
+            acc[0] += bv * bv;
+            acc[1] += bv * zv;
+        }
+        __syncthreads();
+    }
+    block_sum<2>(acc, 1);
+    if (threadIdx.x == 0) {
+        partials[blockIdx.x] = acc[0];
+        partials[gridDim.x + blockIdx.x] = acc[1];
+    }
+}
+
+// Iteration `iter` (1, 2, ...): takes the outcome of the kernel before it
+// (k_cinit1, or k_cx1 of iteration iter - 1: g partials of r.r, r.z, z.q), then
+// p = z + beta p_old, q = A z + beta q_old and the partial sums of p.q.
+template <typename IDX>
+__global__ void __launch_bounds__(kC1) k_cq1(int n, int nb, const int32_t *__restrict__ sptr,
+                                             const IDX *__restrict__ col, const double *__restrict__ val,
+                                             const double *__restrict__ z, const double *__restrict__ pold,
+                                             double *__restrict__ pnew, double *__restrict__ q,
+                                             const double *__restrict__ px, int g, double *__restrict__ pq, CCtl *ctl,
+                                             int iter, double tol) {
+    __shared__ double sbeta;
+    __shared__ bool run;
+    const int lane = threadIdx.x & 31, s = lane & 3;
+    const int nw = (gridDim.x * blockDim.x) >> 5;
+    int wi = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    // the warp's first rows: their matrix chunk does not depend on earlier kernels
+    int j0[kQU];
+    double a0[kQU];
+    int wdt = 0, row = 0;
+    int32_t base = 0;
+    auto rows_of = [&](int w_) {
+        const int b = w_ >> 2, rl = 8 * (w_ & 3) + (lane >> 2);
+        row = b * kB + rl;
+        wdt = 0;
+        if (w_ < nb * 4 && row < n) {
+            base = __ldg(sptr + b);
+            wdt = (__ldg(sptr + b + 1) - base) >> 5;
+            base += rl;
+        }
+    };
+    auto chunk = [&](int k0) {
+#pragma unroll
+        for (int u = 0; u < kQU; u++) {
+            const int k = k0 + 4 * u;
+            const bool in = k < wdt;
+            if constexpr (sizeof(IDX) == 2) j0[u] = in ? row + (int)__ldg(col + base + k * kB) : 0;
+            else j0[u] = in ? __ldg(col + base + k * kB) : 0;
+            a0[u] = in ? __ldg(val + base + k * kB) : 0.0;
+        }
+    };
+    rows_of(wi);
+    chunk(s);
+    pdl_enter();
+    z = after_wait(z);
+    pold = after_wait(pold);
+    q = after_wait(q);
+    ctl = after_wait(ctl);
+    px = after_wait(px);
+    // everything the block needs is requested before anything is used: the
+    // state, the partials, and the first rows' product A z, which waits for no
+    // scalar
+    const int any = __ldcg(&ctl->any);
+    double stop2 = 0.0, pq_old = 0.0;
+    if (threadIdx.x == 0) {
+        stop2 = __ldcg(&ctl->bn[0]);
+        pq_old = __ldcg(&ctl->pq[0]);
+    }
+    double sums[3] = {};
+    if (iter == 1) {
+        double two[2];
+        first_partials<2>(px, g, two);
+        sums[0] = two[0];
+        sums[1] = two[1];
+    } else {
+        first_partials<3>(px, g, sums);
+    }
+    double zj[kQU];
+    auto gather = [&](int k0) {
+#pragma unroll
+        for (int u = 0; u < kQU; u++) zj[u] = k0 + 4 * u < wdt ? __ldg(z + j0[u]) : 0.0;
+    };
+    auto product = [&]() {  // the first chunk is gathered
+        double t = 0.0;
+        for (int k0 = s;;) {
+#pragma unroll
+            for (int u = 0; u < kQU; u++)
+                if (k0 - s + 4 * u < wdt) t = fma(a0[u], zj[u], t);  // the row's four lanes alike
+            k0 += 4 * kQU;
+            if (k0 - s >= wdt) break;
+            chunk(k0);
+            gather(k0);
+        }
+        t += __shfl_xor_sync(0xffffffffu, t, 1);
+        t += __shfl_xor_sync(0xffffffffu, t, 2);
+        return t;
+    };
+    double zi = 0.0, po = 0.0, qo = 0.0;
+    auto vectors = [&]() {
+        if (s == 0 && wi < nb * 4) {
+            zi = __ldg(z + row);
+            po = pold[row];
+            qo = q[row];
+        }
+    };
+    vectors();
+    gather(s);
+    // stopped before this kernel: every thread has read the same word then (a
+    // stop that block 0 records meanwhile is found below by the other blocks)
+    if (__syncthreads_and(any == 0)) return;
+    double qi = product();
+    if (iter == 1) {
+        double two[2] = {sums[0], sums[1]};
+        rest_partials<2>(px, g, two);
+        sums[0] = two[0];
+        sums[1] = two[1];
+    } else {
+        rest_partials<3>(px, g, sums);
+    }
+    if (threadIdx.x == 0) {
+        // sums: b.b and r.z, or r.r, r.z and z.q
+        bool go = any != 0 && sums[1] > 0.0 && isfinite(sums[1]) && isfinite(sums[0]);
+        if (iter == 1) go = go && sums[0] > 0.0;
+        else go = go && sums[0] > stop2;
+        run = go;
+        sbeta = iter == 1 ? 0.0 : -sums[2] / pq_old;
+        if (blockIdx.x == 0 && any) {
+            if (go) {
+                ctl->rho[0] = sums[1];
+                if (iter == 1) ctl->bn[0] = (tol * tol) * sums[0];
+            } else {
+                ctl->any = 0;
+            }
+            if (iter == 1) ctl->its[0] = 0;
+        }
+    }
+    __syncthreads();
+    if (!run) return;
+    const double beta = sbeta;
+    double acc[1] = {};
+    while (wi < nb * 4) {
+        if (s == 0) {
+            double pi = zi;
+            if (beta != 0.0) {
+                pi = fma(beta, po, pi);
+                qi = fma(beta, qo, qi);
+            }
+            pnew[row] = pi;
+            q[row] = qi;
+            acc[0] += pi * qi;
+        }
+        wi += nw;
+        if (wi < nb * 4) {
+            rows_of(wi);
+            chunk(s);
+            vectors();
+            gather(s);
+            qi = product();
+        }
+    }
+    write_partials<1>(acc, pq);
+}
+
+// alpha = rho / p.q from k_cq1's partials, x += alpha p, r -= alpha q,
+// z = M^{-1} r, partial sums of r.r, r.z, z.q. Four warps per 32-row block,
+// each applying 8 columns of the block inverse.
+template <typename TO>
+__global__ void __launch_bounds__(kC1) k_cx1(int n, int nb, const double *__restrict__ Minv,
+                                             const double *__restrict__ p, const double *__restrict__ q,
+                                             double *__restrict__ x, double *__restrict__ r, double *__restrict__ z,
+                                             TO *__restrict__ xo, const double *__restrict__ pq, int g,
+                                             double *__restrict__ partials, CCtl *ctl, int iter) {
+    __shared__ double zp[4][kB];
+    __shared__ double salpha;
+    __shared__ bool run;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int b = blockIdx.x;
+    double m[8];
+    auto inverse = [&](int b_) {
+#pragma unroll
+        for (int k = 0; k < 8; k++)
+            m[k] = b_ < nb ? __ldg(Minv + (int64_t)b_ * kB * kB + (8 * w + k) * kB + lane) : 0.0;
+    };
+    inverse(b);
+    pdl_enter();
+    p = after_wait(p);
+    q = after_wait(q);
+    x = after_wait(x);
+    r = after_wait(r);
+    z = after_wait(z);
+    ctl = after_wait(ctl);
+    pq = after_wait(pq);
+    const int any = __ldcg(&ctl->any);
+    double rho = 0.0, qi = 0.0, ri = 0.0;
+    if (threadIdx.x == 0) rho = __ldcg(&ctl->rho[0]);
+    if (b < nb) {
+        qi = q[b * kB + lane];
+        ri = r[b * kB + lane];
+    }
+    double sums[1];
+    first_partials<1>(pq, g, sums);
+    if (__syncthreads_and(any == 0)) return;  // as in k_cq1
+    rest_partials<1>(pq, g, sums);
+    if (threadIdx.x == 0) {
+        const bool ok = any != 0 && sums[0] > 0.0 && isfinite(sums[0]);
+        run = ok;
+        salpha = rho / sums[0];
+        if (blockIdx.x == 0 && any) {
+            if (ok) {
+                ctl->pq[0] = sums[0];
+                ctl->its[0] = iter;
+            } else {
+                ctl->any = 0;
+            }
+        }
+    }
+    __syncthreads();
+    if (!run) return;
+    const double alpha = salpha;
+    double acc[3] = {};
+    while (b < nb) {
+        const int i = b * kB + lane;
+        const double rn = fma(-alpha, qi, ri);
+        double t = 0.0;
+#pragma unroll
+        for (int k = 0; k < 8; k++) t = fma(m[k], __shfl_sync(0xffffffffu, rn, 8 * w + k), t);
+        zp[w][lane] = t;
+        if (w == 1) {
+            const double xi = fma(alpha, p[i], x[i]);
+            x[i] = xi;
+            if (i < n) xo[i] = (TO)xi;
+        }
+        __syncthreads();
+        if (w == 0) {
+            const double zv = (zp[0][lane] + zp[1][lane]) + (zp[2][lane] + zp[3][lane]);
+            z[i] = zv;
+            r[i] = rn;
+            acc[0] += rn * rn;
+            acc[1] += rn * zv;
+            acc[2] += zv * qi;
+        }
+        __syncthreads();
+        b += gridDim.x;
+        if (b < nb) {
+            inverse(b);
+            qi = q[b * kB + lane];
+            ri = r[b * kB + lane];
+        }
+    }
+    block_sum<3>(acc, 1);
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int v = 0; v < 3; v++) partials[v * gridDim.x + blockIdx.x] = acc[v];
+    }
+}
+
 int grid_for_items(amg_hier *h, int items, int G) {
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess || sms < 1) sms = 152;
@@ -582,6 +887,31 @@ int grid_for_items(amg_hier *h, int items, int G) {
             BODY;                         \
         }                                 \
     } while (0)
+
+// The single-column solve: k_cinit1, then k_cq1 and k_cx1 per iteration.
+template <typename TO>
+int launch_c1(amg_hier *h, CoarseWS &W, const double *bL, TO *xL, const int *outer_done, cudaStream_t s) {
+    Level &lc = h->lev.back();
+    const CoarseIter &C = h->cit;
+    const int n = lc.A.n, nb = C.nb, gx = W.grid, gq = W.grid_q;
+    const bool pdl = h->pdl;
+    double *px = W.partials, *pq = W.partials + 3 * (size_t)gx;
+    PCG_CK(launch_k(pdl, k_cinit1<TO>, gx, kC1, s, n, nb, bL, xL, W.x, W.r, W.z, (const double *)C.Minv, px, W.ctl,
+                    outer_done));
+    for (int it = 1; it <= h->prm.coarse_maxit; it++) {
+        double *pold = (it & 1) ? W.p1 : W.p0;
+        double *pnew = (it & 1) ? W.p0 : W.p1;
+        cudaError_t e = cudaSuccess;
+        WITH_COARSE_COLS(lc.S, (e = launch_k(pdl, k_cq1<IDX>, gq, kC1, s, n, nb, (const int32_t *)lc.S.sptr, cols,
+                                             (const double *)lc.S.v64, (const double *)W.z, (const double *)pold,
+                                             pnew, W.q, (const double *)px, gx, pq, W.ctl, it,
+                                             h->prm.coarse_tol)));
+        PCG_CK(e);
+        PCG_CK(launch_k(pdl, k_cx1<TO>, gx, kC1, s, n, nb, (const double *)C.Minv, (const double *)pnew,
+                        (const double *)W.q, W.x, W.r, W.z, xL, (const double *)pq, gq, px, W.ctl, it));
+    }
+    return AMG_OK;
+}
 
 template <int KC, typename TO>
 int launch_ci(amg_hier *h, CoarseWS &W, const double *bL, TO *xL, const int *outer_done, const int *outer_live,
@@ -650,13 +980,21 @@ int cws_alloc(amg_hier *h, Mem &M, CoarseWS &W, int K) {
     int KC = K == 1 ? 1 : 2;
     W.grid = grid_for_items(h, nb * (K / KC), K / KC);
     W.grid_q = grid_for_items(h, nb * 4 * (K / KC), K / KC);
+    if (K == 1) {
+        // one block of four warps per 32-row block, and so many at most that a
+        // block sums their partials in three or four loads a thread
+        int sms = 0;
+        PCG_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
+        W.grid = nb < 2 * sms ? nb : 2 * sms;
+        W.grid_q = nb < 3 * sms ? nb : 3 * sms;
+    }
     PCG_TRY(alloc(M, &W.x, m));
     PCG_TRY(alloc(M, &W.r, m));
     PCG_TRY(alloc(M, &W.z, m));
     PCG_TRY(alloc(M, &W.p0, m));
     PCG_TRY(alloc(M, &W.p1, m));
     PCG_TRY(alloc(M, &W.q, m));
-    PCG_TRY(alloc(M, &W.partials, (size_t)3 * K * (W.grid > W.grid_q ? W.grid : W.grid_q)));
+    PCG_TRY(alloc(M, &W.partials, (size_t)(K == 1 ? 4 : 3 * K) * (W.grid > W.grid_q ? W.grid : W.grid_q)));
     PCG_TRY(alloc(M, &W.ctl, 1));
     if (M.dry) return AMG_OK;
     PCG_CK(cudaMemsetAsync(W.ctl, 0, sizeof(CCtl), M.stream));
@@ -691,7 +1029,7 @@ int coarse_iter_launches(const amg_hier *h) { return 1 + 2 * h->prm.coarse_maxit
 template <typename TO>
 int launch_coarse_iter(amg_hier *h, CoarseWS &W, const double *bL, TO *xL, const int *outer_done,
                        const int *outer_live, cudaStream_t s) {
-    if (W.K == 1) return launch_ci<1, TO>(h, W, bL, xL, outer_done, outer_live, s);
+    if (W.K == 1) return launch_c1<TO>(h, W, bL, xL, outer_done, s);
     return launch_ci<2, TO>(h, W, bL, xL, outer_done, outer_live, s);
 }
 

@@ -75,15 +75,26 @@ __device__ __forceinline__ void write_partials(double (&a)[NV], double *partials
 
 // Sums of the g partials of each slot, in the block's first warp. Every
 // thread of the block takes part; a thread's own partials (blockDim apart) are
-// added in order.
+// added in order. In two steps, so that a caller can place other loads between
+// them: the thread's first partials, then the sums.
 template <int NV>
-__device__ __forceinline__ void sum_partials(const double *partials, int g, double (&a)[NV]) {
+__device__ __forceinline__ void first_partials(const double *partials, int g, double (&a)[NV]) {
 #pragma unroll
     for (int v = 0; v < NV; v++) a[v] = (int)threadIdx.x < g ? __ldcg(partials + (int64_t)v * g + threadIdx.x) : 0.0;
+}
+
+template <int NV>
+__device__ __forceinline__ void rest_partials(const double *partials, int g, double (&a)[NV]) {
     for (int k = threadIdx.x + blockDim.x; k < g; k += blockDim.x)
 #pragma unroll
         for (int v = 0; v < NV; v++) a[v] += __ldcg(partials + (int64_t)v * g + k);
     block_sum<NV>(a, min((int)(blockDim.x >> 5), (g + 31) >> 5));
+}
+
+template <int NV>
+__device__ __forceinline__ void sum_partials(const double *partials, int g, double (&a)[NV]) {
+    first_partials<NV>(partials, g, a);
+    rest_partials<NV>(partials, g, a);
 }
 
 }  // namespace pcgamg

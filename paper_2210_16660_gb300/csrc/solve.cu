@@ -1700,14 +1700,15 @@ void launch_post0(amg_hier *h, const T *b0, cudaStream_t s) {
     }
     if constexpr (sizeof(T) == 4) {
         if (pat_rows(h)) {
-            WITH_COLS(l0.S, (launch_k(h->pdl, k_post<T, double, true, FCG, IDX, kPatRow, true, false>, grid0<T>(h), h->block0,
-                                      s, l0.A.n, l0.S.sptr, cols, P::val(l0), pats, P::xp(l0), b0, P::dinv(l0), h->z,
+            WITH_COLS(l0.S, (launch_k(h->pdl, k_post<T, double, true, FCG, IDX, kPatRow, true, false>, grid0<T>(h),
+                                      h->block0, s, l0.A.n, l0.S.sptr, cols, P::val(l0), pats, P::xp(l0), b0, P::dinv(l0), h->z,
                                       h->r, h->q, parts(h, kPartsRz), h->ctl,
                                       Up<T>{})));
             return;
         }
     }
-    WITH_COLS(l0.S, (launch_k(h->pdl, k_post<T, double, true, FCG, IDX, kUnroll, true, false>, grid0<T>(h), h->block0, s,
+    WITH_COLS(l0.S, (launch_k(h->pdl, k_post<T, double, true, FCG, IDX, kUnroll, true, false>, grid0<T>(h),
+                                  h->block0, s,
                                   l0.A.n, l0.S.sptr, cols, P::val(l0), pats, P::xp(l0), b0, P::dinv(l0), h->z, h->r,
                                   h->q, parts(h, kPartsRz), h->ctl, Up<T>{})));
 }
