@@ -24,8 +24,9 @@ constexpr int kOpThreads = 256;
 // smaller matrix by latency (about 2 us each). Alone, 400 rows instead cost
 // 812 us per 24^3 solve (834-row level, 727 with it), 1,536 and 2,600 rows the
 // same there, but 128^3 22.9 ms with 2,600 (22.0); twelve systems at once,
-// which share the pipe, ran 12.7 ms with 900 and 13.2 with 1,536.
-constexpr int kOpRows = 1100;
+// which share the pipe, ran 12.7 ms with 900 and 13.2 with 1,536; 41^3 float64
+// (a level between 1,100 and 1,280 rows) 2,412 us without it, 2,140 with it.
+constexpr int kOpRows = 1280;
 
 // One level's step, for column j (blockIdx.x) of B: x = S e_j + correction,
 // the smoothing and transfer steps of the V-cycle in plain float64.
