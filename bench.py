@@ -432,9 +432,9 @@ def level_table(amg, lev_prof, mode: str, peak: float) -> list:
         if down is None:
             row["note"] = "iterative coarsest solve (FCG + block-Jacobi ILU(1), at most the configured inner iterations)"
         if tail < L and lvl == tail:
-            row["note"] = f"time of the shared-memory cluster tail, levels {tail}..{L}"
+            row["note"] = f"time of the levels solved in one launch, {tail}..{L}"
         elif lvl > tail:
-            row["note"] = f"inside the cluster tail of level {tail}"
+            row["note"] = f"inside the one launch of level {tail}"
         out.append(row)
     return out
 

@@ -165,8 +165,8 @@ int amg_refresh(amg_handle h, const amg_csr *A, void *stream);
  * j outside i's block (the l1 form, no damping). One row per block and one
  * sweep give the values of the default. Re-forms every level's smoother
  * diagonal (and a float32 CSR copy of the level matrices for the sweeps);
- * the next solve recaptures its graph; the shared-memory cluster tail is not
- * used while nu > 0. In the float32 V-cycle, where a level's blocks divide
+ * the next solve recaptures its graph; the levels above the smallest (which
+ * are applied as one matrix where memory allows) are swept one by one. In the float32 V-cycle, where a level's blocks divide
  * its 32-row slices (and no row has more than 8 already-updated in-block
  * entries), a sweep is one launch, one warp per slice; otherwise two. Single and batched solves take nu > 0;
  * multi-column and served solves run the l1-Jacobi kernels only and return
@@ -346,8 +346,8 @@ void amg_server_destroy(amg_server s);
  * are launched on this device, not what they compute). For every level
  * l >= 1 with sweeps, each V-cycle precision and each of the down phase
  * (down sweep + restriction) and the up phase (prolongation + post sweep),
- * it times nine launch shapes -- rows loading 4 or 16 entries per chunk,
- * times a one-wave grid-stride grid or one thread per row, times two
+ * it times nine launch shapes -- rows loading 4 or 16 entries per chunk
+ * (whole rows in place of 16 on levels of up to 32768 rows), times a one-wave grid-stride grid or one thread per row, times two
  * launches or one fused launch (down sweep and restriction by aggregate;
  * prolongation formed per gathered entry inside the post sweep); and rows
  * read by 4 lanes each, every entry of a row gathered at once and the sum
@@ -436,7 +436,7 @@ int amg_profile_read(amg_handle h, double *ms, int64_t *counts, int nkinds);
  * 3l+2: the down phase (level l's down sweep, l >= 1, and the restriction
  * to level l+1), the up phase (prolongation to level l and its post sweep,
  * l >= 1) and the coarsest solve (on the coarsest level's entry, or on the
- * first level of the cluster tail when that is on). ms, counts: host arrays
+ * first of the levels solved in one launch). ms, counts: host arrays
  * of 3 nlev values (nlev <= 32), or NULL. */
 int amg_profile_levels(amg_handle h, int nlev, double *ms, int64_t *counts);
 
