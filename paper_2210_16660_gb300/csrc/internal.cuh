@@ -51,7 +51,8 @@ __device__ __forceinline__ void pdl_enter() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// A kernel that reads static data before pdl_enter() passes every pointer to
+// A kernel that reads static data before pdl_enter(), or loads anything after
+// it ahead of its first branch on the solve's state, passes the pointers to
 // data the preceding kernel wrote through after_wait() once pdl_enter() has
 // returned: the empty volatile asm stays after the wait (volatile asms keep
 // their order) and the pointer it yields is unknown to the compiler before

@@ -953,6 +953,10 @@ template <bool FCG>
 __global__ void __launch_bounds__(kVecBlock) k_axpy_p(int n, const double *__restrict__ z, double *__restrict__ p,
                                                       const double *pa, int ga, Ctl *ctl) {
     pdl_enter();
+    // no use of the state stands between the wait and these loads
+    z = after_wait(z);
+    p = after_wait(p);
+    ctl = after_wait(ctl);
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int stride = gridDim.x * blockDim.x;
     int halt = kRun, restart = 0;
@@ -1059,6 +1063,11 @@ __global__ void __launch_bounds__(kVecBlock) k_update(int n, const double *__res
                                                       double *__restrict__ r, REmit em, const double *pb, int gb,
                                                       double *partials, Ctl *ctl) {
     pdl_enter();
+    p = after_wait(p);  // as in k_axpy_p
+    q = after_wait(q);
+    x = after_wait(x);
+    r = after_wait(r);
+    ctl = after_wait(ctl);
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int stride = gridDim.x * blockDim.x;
     int halt = kRun, iter = 0;
@@ -1150,6 +1159,9 @@ __global__ void __launch_bounds__(kBlock, 4) k_residual(int n, const int32_t *__
                                                         REmit em, const double *pc, int gc, double *partials,
                                                         Ctl *ctl, double *hist, Cond cond) {
     pdl_enter();
+    b = after_wait(b);
+    x = after_wait(x);
+    ctl = after_wait(ctl);
     if (!INIT) {
         if (step_outcome(pc, gc, ctl, hist) != kCheck) {
             if (blockIdx.x == 0 && threadIdx.x == 0) set_cond(cond, ctl, true);
