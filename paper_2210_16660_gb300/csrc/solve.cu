@@ -2453,17 +2453,20 @@ int solve_impl(amg_hier *h, const double *b, double *x, double rtol, int maxit, 
         h->launches += h->graph_prefix_kernels + (int64_t)h->ctl_host->bodies * h->graph_body_kernels[h->mode];
     } else {
         PCG_TRY(launch_prefix(h, Cond{}, s));
-        // Iterate in chunks; once done, every later kernel returns at once.
+        // Iterate in chunks. A chunk's iterations past one whose recursive
+        // residual met rtol do nothing (the true residual is the chunk's last
+        // kernel), so what is left is counted by the iterations that ran; each
+        // chunk runs at least one, and once done every later kernel returns at
+        // once.
         const int chunk = 4;
-        int launched = 0;
-        for (;;) {
+        for (int chunks = 0;; chunks++) {
             PCG_CK(cudaMemcpyAsync(h->ctl_host, h->ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
             PCG_CK(cudaStreamSynchronize(s));
             if (h->profile) prof_collect(h);
-            if (h->ctl_host->done || launched >= maxit) break;
-            const int todo = std::min(chunk, maxit - launched);
-            for (int k = 0; k < todo; k++, launched++)
-                PCG_TRY(launch_iteration(h, k == 0, k + 1 == todo, Cond{}, s));
+            const int left = maxit - h->ctl_host->iter;
+            if (h->ctl_host->done || left <= 0 || chunks > maxit) break;
+            const int todo = std::min(chunk, left);
+            for (int k = 0; k < todo; k++) PCG_TRY(launch_iteration(h, k == 0, k + 1 == todo, Cond{}, s));
         }
     }
     Ctl &c = *h->ctl_host;

@@ -225,6 +225,27 @@ def test_int16_and_int32_columns_agree(mode):
 
 
 @pytest.mark.parametrize("mode", ["pcg64", "fcg32"])
+@pytest.mark.parametrize("maxit", [45, 50, 61])
+def test_restarts_run_to_maxit_on_both_launch_paths(mode, maxit):
+    """At an rtol below what the true residual can reach, the recursive one
+    meets it again and again and each true residual restarts the recurrence:
+    stream launches run maxit iterations as the graph does, with its values."""
+    prob = W.make_problem(20, 1.04, seed=6)
+    b = torch.from_numpy(prob.b).cuda()
+    out = []
+    for g in ("1", "0"):
+        amg = _with_env("PCGAMG_GRAPH", g, lambda: B.AMG.from_csr(prob.A, mode=mode))
+        x = torch.zeros_like(b)
+        out.append((amg.solve(b, x, rtol=1e-17, maxit=maxit), x))
+    (r1, x1), (r2, x2) = out
+    assert r1.status == B.ERR_NOCONV and r1.iters == maxit
+    # the last true residual is not the recursive one: there was a restart
+    assert r1.hist.min() < 1e-14 and r1.true_rel > 1e-17
+    assert r2.status == r1.status and r2.iters == r1.iters
+    assert np.array_equal(r1.hist, r2.hist) and torch.equal(x1, x2)
+
+
+@pytest.mark.parametrize("mode", ["pcg64", "fcg32"])
 @pytest.mark.parametrize("N", [32, 64])
 def test_cluster_tail_matches_separate_launches(mode, N):
     """Small levels in one thread-block cluster with their data in shared
