@@ -117,42 +117,45 @@ __device__ __forceinline__ void sell_row_vec(const IDX *__restrict__ c, const T 
     int c0 = (int)(g_ % (K / (V))) * (V);                                                     \
     int64_t e0 = (int64_t)i * K + c0;
 
-// Whether the solve goes on and any of the V columns from c0 still iterates, for
-// the small levels' kernels: all loads are issued together, and the answer is
-// used only before the store.
-template <int V>
-__device__ __forceinline__ int group_runs(const CtlM *ctl, int c0) {
-    int a = 0;
-    const int done = __ldcg(&ctl->done);
-#pragma unroll
-    for (int v = 0; v < V; v++) a |= __ldcg(&ctl->active[c0 + v]);
-    return a && !done;
+// The columns still iterating (run[c]) and whether the solve has ended (run[K]),
+// read once per block: thread c loads run_flag() and share_run() hands it on.
+// The state lies in a few sectors of L2, which serve one request after
+// another: read by every thread, those requests were what the kernels with
+// one row per thread waited for (k_prolong_m of 218,800 rows x 32 in float32
+// 51.5 us, 14.3 so; k_restrict_m to it 55.0 and 27.8).
+// Small levels' kernels load the flag before their gathers and share it only
+// before the store.
+template <int K>
+__device__ __forceinline__ int run_flag(const CtlM *ctl) {
+    const int c = threadIdx.x;
+    return c < K ? __ldcg(&ctl->active[c]) : c == K ? __ldcg(&ctl->done) : 0;
+}
+
+template <int K>
+__device__ __forceinline__ const int *share_run(int flag) {
+    __shared__ int run[K + 1];
+    if (threadIdx.x <= K) run[threadIdx.x] = flag;
+    __syncthreads();
+    return run;
 }
 
 // Whether any of the V columns from c0 is still iterating.
 template <int V>
-__device__ __forceinline__ bool group_live(const CtlM *ctl, int c0) {
+__device__ __forceinline__ bool group_live(const int *run, int c0) {
     int a = 0;
 #pragma unroll
-    for (int v = 0; v < V; v++) a |= __ldcg(&ctl->active[c0 + v]);
+    for (int v = 0; v < V; v++) a |= run[c0 + v];
     return a != 0;
 }
+
+// First column of a thread's fixed column group.
+#define MK_C0(V) ((int)((((int64_t)blockIdx.x * blockDim.x + threadIdx.x) % (K / (V))) * (V)))
 
 // A thread's column group is fixed over its grid-stride loop (the stride is a
 // multiple of K / V); a group whose columns have all stopped skips its rows,
 // so a block with few live columns moves only their vectors. The arithmetic
 // of a live column does not depend on which other columns are live.
-#define MK_LIVE(V)                                                                            \
-    const bool live_ = group_live<V>(                                                         \
-        ctl, (int)((((int64_t)blockIdx.x * blockDim.x + threadIdx.x) % (K / (V))) * (V)));
-
-// Per-column scalars of a thread's fixed column group, read once (c: its first
-// column).
-#define MK_COLS(V, BODY)                                                                      \
-    {                                                                                         \
-        const int c = (int)((((int64_t)blockIdx.x * blockDim.x + threadIdx.x) % (K / (V))) * (V)); \
-        _Pragma("unroll") for (int v = 0; v < (V); v++) { BODY; }                             \
-    }
+#define MK_LIVE(V) const bool live_ = group_live<V>(run, MK_C0(V));
 
 // Per-column sums of NV quantities: a thread holds a[s][v], the s-th quantity
 // of column c0 + v (c0 fixed per thread). The block's values meet in shared
@@ -236,7 +239,8 @@ __global__ void __launch_bounds__(kMB, 5) k_down_m(int n, const int32_t *__restr
                                                const CtlM *__restrict__ ctl) {
     constexpr int V = VW<T>::V;
     pdl_enter();
-    if (__ldcg(&ctl->done)) return;
+    const int *run = share_run<K>(run_flag<K>(ctl));
+    if (run[K]) return;
     MK_LIVE(V)
     MK_FOR(live_ ? n : 0, V) {
         MK_IDX(V)
@@ -278,15 +282,17 @@ __global__ void __launch_bounds__(kMB) k_down_c(int n, const int32_t *__restrict
     xpre = after_wait(xpre);
     b = after_wait(b);
     ctl = after_wait(ctl);
-    if (!in) return;
-    const int runs = group_runs<V>(ctl, c0);
+    const int flag = run_flag<K>(ctl);
     const int64_t e0 = (int64_t)i * K + c0;
-    T bv[V], acc[V], o[V];
-    ld_vec<T, V>(b + e0, bv);
-    R.template dot_vec<V>(i, [&](int j, T (&x)[V]) { ld_vec<T, V>(xpre + (int64_t)j * K + c0, x); }, acc);
+    T bv[V], acc[V], o[V] = {};
+    if (in) {
+        ld_vec<T, V>(b + e0, bv);
+        R.template dot_vec<V>(i, [&](int j, T (&x)[V]) { ld_vec<T, V>(xpre + (int64_t)j * K + c0, x); }, acc);
 #pragma unroll
-    for (int v = 0; v < V; v++) o[v] = pi * (bv[v] - acc[v]);
-    if (runs) st_vec<T, V>(t + e0, o);
+        for (int v = 0; v < V; v++) o[v] = pi * (bv[v] - acc[v]);
+    }
+    const int *run = share_run<K>(flag);
+    if (in && !run[K] && group_live<V>(run, c0)) st_vec<T, V>(t + e0, o);
 }
 
 template <typename T, typename IDX, int K, int U>
@@ -309,16 +315,18 @@ __global__ void __launch_bounds__(kMB) k_post_c(int n, const int32_t *__restrict
     xp = after_wait(xp);
     b = after_wait(b);
     ctl = after_wait(ctl);
-    if (!in) return;
-    const int runs = group_runs<V>(ctl, c0);
+    const int flag = run_flag<K>(ctl);
     const int64_t e0 = (int64_t)i * K + c0;
-    T xv[V], bv[V], acc[V], o[V];
-    ld_vec<T, V>(xp + e0, xv);
-    ld_vec<T, V>(b + e0, bv);
-    R.template dot_vec<V>(i, [&](int j, T (&x)[V]) { ld_vec<T, V>(xp + (int64_t)j * K + c0, x); }, acc);
+    T xv[V], bv[V], acc[V], o[V] = {};
+    if (in) {
+        ld_vec<T, V>(xp + e0, xv);
+        ld_vec<T, V>(b + e0, bv);
+        R.template dot_vec<V>(i, [&](int j, T (&x)[V]) { ld_vec<T, V>(xp + (int64_t)j * K + c0, x); }, acc);
 #pragma unroll
-    for (int v = 0; v < V; v++) o[v] = xv[v] + d * (bv[v] - acc[v]);
-    if (runs) st_vec<T, V>(z + e0, o);
+        for (int v = 0; v < V; v++) o[v] = xv[v] + d * (bv[v] - acc[v]);
+    }
+    const int *run = share_run<K>(flag);
+    if (in && !run[K] && group_live<V>(run, c0)) st_vec<T, V>(z + e0, o);
 }
 
 // b_c[I] = sum of t over the members of aggregate I in index order (and
@@ -346,8 +354,7 @@ __global__ void __launch_bounds__(kMB) k_restrict_m(int nc, const int32_t *__res
     pdl_enter();
     t = after_wait(t);
     ctl = after_wait(ctl);
-    if (!in) return;
-    const int runs = group_runs<V>(ctl, c0);
+    const int flag = run_flag<K>(ctl);
     const int64_t e0 = (int64_t)i * K + c0;
     T s[V], x[M][V];
 #pragma unroll
@@ -367,7 +374,8 @@ __global__ void __launch_bounds__(kMB) k_restrict_m(int nc, const int32_t *__res
 #pragma unroll
         for (int v = 0; v < V; v++) s[v] += y[v];
     }
-    if (!runs) return;
+    const int *run = share_run<K>(flag);
+    if (!in || run[K] || !group_live<V>(run, c0)) return;
 #pragma unroll
     for (int v = 0; v < V; v++) bc[e0 + v] = (TO)s[v];
     if (PRE) {
@@ -388,11 +396,12 @@ __global__ void __launch_bounds__(kMB) k_coarse_m(int nL, const double *__restri
                                                  const CtlM *__restrict__ ctl) {
     constexpr int V = 2;
     pdl_enter();
-    if (__ldcg(&ctl->done)) return;
+    const int *run = share_run<K>(run_flag<K>(ctl));
+    if (run[K]) return;
     int warp = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (warp >= nL * (K / V)) return;  // whole warps
     int row = warp / (K / V), c0 = (warp % (K / V)) * V;
-    if (!group_live<V>(ctl, c0)) return;
+    if (!group_live<V>(run, c0)) return;
     const double *a = ainv + (int64_t)row * nL;
     double s0 = 0.0, s1 = 0.0;
 #pragma unroll 4
@@ -416,7 +425,8 @@ __global__ void __launch_bounds__(kMB) k_prolong_m(int n, const T *__restrict__ 
                                                   T *__restrict__ xp, const CtlM *__restrict__ ctl) {
     constexpr int V = VW<T>::V;
     pdl_enter();
-    if (__ldcg(&ctl->done)) return;
+    const int *run = share_run<K>(run_flag<K>(ctl));
+    if (run[K]) return;
     MK_LIVE(V)
     MK_FOR(live_ ? n : 0, V) {
         MK_IDX(V)
@@ -471,7 +481,8 @@ __global__ void __launch_bounds__(kMB, K >= 16 ? 0 : 4) k_post_m(int n, const in
                                                double *partials, CtlM *ctl) {
     constexpr int V = VW<T>::V;
     pdl_enter();
-    if (__ldcg(&ctl->done)) return;
+    const int *run = share_run<K>(run_flag<K>(ctl));
+    if (run[K]) return;
     constexpr int NV = FCG ? 2 : 1;
     double sums[NV][V] = {};
     MK_LIVE(V)
@@ -521,13 +532,14 @@ __global__ void __launch_bounds__(kMB) k_gs_warp_m(int n, int nb, int w, const i
     constexpr int V = VW<T>::V;
     constexpr int G = K / V;
     pdl_enter();
-    if (__ldcg(&ctl->done)) return;
+    const int *run = share_run<K>(run_flag<K>(ctl));
+    if (run[K]) return;
     const int lane = threadIdx.x & 31;
     const int nsl = (n + 31) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t wi = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; wi < (int64_t)nsl * G; wi += nw) {
         const int sl = (int)(wi / G), c0 = (int)(wi % G) * V;
-        if (!group_live<V>(ctl, c0)) continue;  // uniform over the warp
+        if (!group_live<V>(run, c0)) continue;  // uniform over the warp
         const int i = (sl << 5) + lane;
         const bool valid = i < n;
         const int64_t e0 = (int64_t)i * K + c0;
@@ -618,7 +630,8 @@ __global__ void __launch_bounds__(kMB) k_gs_finish0_m(int n, const T *__restrict
                                                      double *partials, CtlM *ctl) {
     constexpr int V = VW<T>::V;
     pdl_enter();
-    if (__ldcg(&ctl->done)) return;
+    const int *run = share_run<K>(run_flag<K>(ctl));
+    if (run[K]) return;
     constexpr int NV = FCG ? 2 : 1;
     double sums[NV][V] = {};
     MK_LIVE(V)
@@ -643,11 +656,18 @@ __global__ void __launch_bounds__(kMB) k_axpy_m(int n, const double *__restrict_
                                                const CtlM *__restrict__ ctl) {
     constexpr int V = 2;
     pdl_enter();
-    if (__ldcg(&ctl->done)) return;
+    __shared__ double sbeta[K];
+    if (threadIdx.x < K) sbeta[threadIdx.x] = __ldcg(&ctl->beta[threadIdx.x]);
+    const int *run = share_run<K>(run_flag<K>(ctl));
+    if (run[K]) return;
     MK_LIVE(V)
     int act[V];
     double beta[V];
-    MK_COLS(V, act[v] = __ldcg(&ctl->active[c + v]); beta[v] = __ldcg(&ctl->beta[c + v]))
+#pragma unroll
+    for (int v = 0; v < V; v++) {
+        act[v] = run[MK_C0(V) + v];
+        beta[v] = sbeta[MK_C0(V) + v];
+    }
     MK_FOR(live_ ? n : 0, V) {
         MK_IDX(V)
         double zv[V], pv[V], o[V];
@@ -669,7 +689,8 @@ __global__ void __launch_bounds__(kMB, K >= 16 ? 8 : 4) k_spmm_m(int n, const in
                                                double *partials, CtlM *ctl) {
     constexpr int V = 2;
     pdl_enter();
-    if (__ldcg(&ctl->done)) return;
+    const int *run = share_run<K>(run_flag<K>(ctl));
+    if (run[K]) return;
     double pq[1][V] = {};
     MK_LIVE(V)
     MK_FOR(live_ ? n : 0, V) {
@@ -732,12 +753,19 @@ __global__ void __launch_bounds__(kMB) k_update_m(int n, const double *__restric
                                                  double *partials, CtlM *ctl, double *hist, int hstride) {
     constexpr int V = 2;
     pdl_enter();
-    if (__ldcg(&ctl->done)) return;
+    __shared__ double salpha[K];
+    if (threadIdx.x < K) salpha[threadIdx.x] = __ldcg(&ctl->alpha[threadIdx.x]);
+    const int *run = share_run<K>(run_flag<K>(ctl));
+    if (run[K]) return;
     double rr[1][V] = {};
     MK_LIVE(V)
     int act[V];
     double al[V];
-    MK_COLS(V, act[v] = __ldcg(&ctl->active[c + v]); al[v] = __ldcg(&ctl->alpha[c + v]))
+#pragma unroll
+    for (int v = 0; v < V; v++) {
+        act[v] = run[MK_C0(V) + v];
+        al[v] = salpha[MK_C0(V) + v];
+    }
     MK_FOR(live_ ? n : 0, V) {
         MK_IDX(V)
         double rv[V], xv[V], pv[V], qv[V];
@@ -807,13 +835,16 @@ __global__ void __launch_bounds__(kMB) k_residual_m(int n, const int32_t *__rest
                                                    double *partials, CtlM *ctl, double *hist, int hstride) {
     constexpr int V = 2;
     pdl_enter();
-    if (__ldcg(&ctl->done)) return;
-    if (!INIT && !__ldcg(&ctl->any_check)) return;
+    // as run_flag: the columns to form the residual of, and whether any is left to do
+    __shared__ int uses[K + 1];
+    if (threadIdx.x < K)
+        uses[threadIdx.x] = INIT ? __ldcg(&ctl->pending[threadIdx.x]) : __ldcg(&ctl->check[threadIdx.x]);
+    if (threadIdx.x == K) uses[K] = !__ldcg(&ctl->done) && (INIT || __ldcg(&ctl->any_check));
+    __syncthreads();
+    if (!uses[K]) return;
     constexpr int NV = INIT ? 2 : 1;
     double sums[NV][V] = {};
-    int use[V];
-    MK_COLS(V, use[v] = INIT ? __ldcg(&ctl->pending[c + v]) : __ldcg(&ctl->check[c + v]))
-    const bool use0 = use[0] != 0, use1 = use[1] != 0;
+    const bool use0 = uses[MK_C0(V)] != 0, use1 = uses[MK_C0(V) + 1] != 0;
     MK_FOR(use0 || use1 ? n : 0, V) {
         MK_IDX(V)
         int s = i >> 5, lane = i & 31;
