@@ -468,10 +468,10 @@ __device__ __forceinline__ void finish_rho_m(double (&sums)[NV][V], double *part
     }
 }
 
-// Below 16 columns four blocks per SM (registers for the row's gathers): served
-// burst 43.9 -> 42.4 ms, 40^3 x 5 6.78 -> 6.68 ms.
 // z = xp + D^-1 (b - A xp); DOT on level 0: per-column r.z and z.q_old, and
-// the last block forms rho_c and beta_c.
+// the last block forms rho_c and beta_c. Below 16 columns four blocks per SM
+// (registers for the row's gathers): served burst 43.9 -> 42.4 ms, 40^3 x 5
+// 6.78 -> 6.68 ms.
 template <typename T, typename TZ, bool DOT, bool FCG, typename IDX, int K, int U, bool STREAM>
 __global__ void __launch_bounds__(kMB, K >= 16 ? 0 : 4) k_post_m(int n, const int32_t *__restrict__ sptr,
                                                const IDX *__restrict__ col, const T *__restrict__ val,
@@ -680,8 +680,11 @@ __global__ void __launch_bounds__(kMB) k_axpy_m(int n, const double *__restrict_
 }
 
 // Bound by the float64 pipe (two FMAs per entry and thread); from 16 columns on
-// a full SM of warps at 32 registers keeps it busier than fewer with more
-// (96^3 x 32: whole solves 172 -> 164 ms; 40^3 x 8 7.0 -> 7.3 ms, so not there).
+// a full SM of warps at 32 registers, of which 84 bytes a thread are spilled,
+// keeps it busier than fewer with more (96^3 x 32 mixed: whole solves 164 ms,
+// 172 at the compiler's registers; 96^3 x 32 and 160^3 x 32 float64 308.4 and
+// 1,644 ms, 315.5 and 1,683; 40^3 x 8 lost, 7.0 -> 7.3 ms, and 96^3 x 8 mixed
+// with six blocks per SM too, 41.3 -> 43.2, so four below 16 columns).
 template <typename IDX, int K>
 __global__ void __launch_bounds__(kMB, K >= 16 ? 8 : 4) k_spmm_m(int n, const int32_t *__restrict__ sptr,
                                                const IDX *__restrict__ col, const double *__restrict__ val,
@@ -1066,8 +1069,8 @@ int direct_level_m(const amg_hier *h, int K) {
 }
 
 // Blocks of a grid-stride kernel: one thread per item up to two waves, else
-// one wave of what stays resident (a grid that is no multiple of it leaves SMs with blocks to spare
-// at the end: 96^3 x 32, q = A p 1549 us with 8 blocks per SM where 6 fit).
+// one wave of what stays resident (a grid that is no multiple of it leaves SMs
+// with blocks to spare at the end).
 template <typename F>
 int wave_grid(const MultiWS &W, F *kernel, int64_t items) {
     int per = 0;
@@ -1081,8 +1084,21 @@ inline int block_of(const MultiWS &W, int64_t items) {
     return items <= (int64_t)W.sms * 64 ? 64 : items <= (int64_t)W.sms * 128 ? 128 : kMB;
 }
 
-// Rows up to which a coarse level's rows load 16 entries per chunk, else 4.
-constexpr int kChunkRowsM = 16384;
+// Threads up to which a coarse level waits for latency and its rows load 16
+// entries per chunk (k_down_c, k_post_c), else 4 at a higher residency: 55,000
+// threads (13,800 rows x 8 in float64) 19.4 us with 16 and 22.3 with 4, 110,000
+// (x 32 in float32) 26.1 and 11.5, 220,000 (x 32 in float64) 52.9 and 32.4.
+constexpr int kChunkThreadsM = 65536;
+
+// Blocks of the level-0 sweeps and of q = A p. In float32 one wave of what
+// stays resident; in float64, which its pipe bounds, eight blocks per SM
+// whatever stays: 96^3 x 32 down sweep 1,541 us in one wave and 1,435 so, x 8
+// 391 and 360, post sweep 391 and 374, q = A p 364 and 345. In float32 eight
+// per SM cost 152.2 ms a solve (x 32) for 148.3.
+template <typename T, typename F>
+int sweep_grid(const MultiWS &W, F *kernel, int64_t items) {
+    return sizeof(T) == 8 ? W.grid : wave_grid(W, kernel, items);
+}
 
 template <typename T, bool FCG, int K>
 int launch_vcycle_m(amg_hier *h, MultiWS &W, cudaStream_t s) {
@@ -1106,7 +1122,7 @@ int launch_vcycle_m(amg_hier *h, MultiWS &W, cudaStream_t s) {
     const bool gs = h->gs_nu > 0;
     if (gs) launch_gs_m<T, K>(h, W, 0, true, b0, P::xpre(m0), s);
     WITH_COLS_M(l0.S, (launch_k(pdl, k_down_m<T, IDX, K, kUnroll, true>,
-                                wave_grid(W, k_down_m<T, IDX, K, kUnroll, true>, items0), kMB, s, l0.A.n, l0.S.sptr,
+                                sweep_grid<T>(W, k_down_m<T, IDX, K, kUnroll, true>, items0), kMB, s, l0.A.n, l0.S.sptr,
                                 cols, P::val(l0), P::xpre(m0), b0, P::p(l0), P::t(m0), ctl)));
     for (int l = 0; l < L; l++) {
         Level &lv = lev[l];
@@ -1116,7 +1132,7 @@ int launch_vcycle_m(amg_hier *h, MultiWS &W, cudaStream_t s) {
         if (l > 0) {
             if (gs) launch_gs_m<T, K>(h, W, l, true, P::b(mv), P::xpre(mv), s);
             const int blk = block_of(W, items), g = (int)((items + blk - 1) / blk);
-            if (n <= kChunkRowsM)
+            if (items <= kChunkThreadsM)
                 WITH_COLS_M(lv.S, (launch_k(pdl, k_down_c<T, IDX, K, kUnrollSmall>, g, blk, s, n, lv.S.sptr, cols,
                                             P::val(lv), pats, P::xpre(mv), P::b(mv), P::p(lv), P::t(mv), ctl)));
             else
@@ -1147,7 +1163,7 @@ int launch_vcycle_m(amg_hier *h, MultiWS &W, cudaStream_t s) {
                  ctl);
         if (gs)
             launch_gs_m<T, K>(h, W, l, false, P::b(mv), P::x(mv), s);
-        else if (n <= kChunkRowsM)
+        else if (items <= kChunkThreadsM)
             WITH_COLS_M(lv.S, (launch_k(pdl, k_post_c<T, IDX, K, kUnrollSmall>, g, blk, s, n, lv.S.sptr, cols,
                                         P::val(lv), pats, P::xp(mv), P::b(mv), P::dinv(lv), P::x(mv), ctl)));
         else
@@ -1166,7 +1182,7 @@ int launch_vcycle_m(amg_hier *h, MultiWS &W, cudaStream_t s) {
         return AMG_OK;
     }
     WITH_COLS_M(l0.S, (launch_k(pdl, k_post_m<T, double, true, FCG, IDX, K, kUnroll, true>,
-                                wave_grid(W, k_post_m<T, double, true, FCG, IDX, K, kUnroll, true>, items0), kMB, s,
+                                sweep_grid<T>(W, k_post_m<T, double, true, FCG, IDX, K, kUnroll, true>, items0), kMB, s,
                                 l0.A.n, l0.S.sptr, cols, P::val(l0), P::xp(m0), b0, P::dinv(l0), W.z, W.r, W.q,
                                 W.partials, ctl)));
     PCG_LAUNCH_CK();
@@ -1200,7 +1216,7 @@ int launch_iteration_m(amg_hier *h, MultiWS &W, int mode, cudaStream_t s) {
     else if (h->coarse_iter) PCG_TRY((launch_vcycle_m<double, true, K>(h, W, s)));  // flexible: FCG(1) beta
     else PCG_TRY((launch_vcycle_m<double, false, K>(h, W, s)));
     launch_k(h->pdl, k_axpy_m<K>, wave_grid(W, k_axpy_m<K>, items), kMB, s, n, W.z, W.p, W.ctl);
-    WITH_COLS_M(l0.S, (launch_k(h->pdl, k_spmm_m<IDX, K>, wave_grid(W, k_spmm_m<IDX, K>, items), kMB, s, n, l0.S.sptr,
+    WITH_COLS_M(l0.S, (launch_k(h->pdl, k_spmm_m<IDX, K>, sweep_grid<double>(W, k_spmm_m<IDX, K>, items), kMB, s, n, l0.S.sptr,
                                 cols, l0.S.v64, W.p, W.q, W.partials, W.ctl)));
     // half a wave of the update: its partials are what its last block reads
     if (mode == AMG_MODE_FCG32)
