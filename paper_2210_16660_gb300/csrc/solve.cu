@@ -45,7 +45,7 @@ namespace pcgamg {
 
 namespace {
 
-constexpr int kVecBlock = 1024;  // largest block of the vector kernels (k_axpy_p, k_update)
+constexpr int kVecBlock = 512;  // largest block of the vector kernels (k_axpy_p, k_update)
 
 template <typename T>
 __device__ __forceinline__ T ldg(const T *p) { return __ldg(p); }
@@ -1355,9 +1355,11 @@ constexpr int kWholeRows = 32768;
 // A solve that shares the device (batches, serving lanes: no_tail) is short of
 // registers and float64 cycles rather than waiting for latency: twelve systems
 // of 24^3 to 72^3 at once ran 14.2 ms with the limits of a lone solve, 13.1
-// with these (the bits are the same).
+// with 1,024 and 16,384 rows (the bits are the same); 48 of 24^3 to 112^3 199.5
+// ms (268.8 in float64) with 16,384 rows fused, 198.7 (266.5) with 4,096,
+// where the twelve take 12.6 ms either way.
 constexpr int kWholeRowsShared = 1024;
-constexpr int kFuseRowsShared = 16384;
+constexpr int kFuseRowsShared = 4096;
 int whole_rows(const amg_hier *h) { return h->no_tail ? kWholeRowsShared : kWholeRows; }
 
 // Blocks and threads of a coarse-level sweep over n rows (or positions).
@@ -2223,9 +2225,13 @@ int alloc_solve_workspace(amg_hier *h) {
     }
     PCG_TRY(wave((const void *)k_spmv<int32_t, kUnroll>, &h->grid64));
     PCG_TRY(wave((const void *)k_prolong<float>, &h->gridp));
-    // the vector kernels: at most two blocks per SM (their consumers read one
-    // partial per block), the block as large as the rows fill
-    const int vec_blocks = 2 * sms;
+    // the vector kernels: few blocks (their consumers read one partial per
+    // block), the block as large as the rows fill. Two per SM while they hold
+    // the rows (41^3 float64 2,242 us with three, 2,183 with two), three above
+    // (64^3 warm 2,155 and 2,136). Blocks of 1,024 threads, two per SM, waited
+    // for half an SM to fall free where systems share the device: 48 of 24^3 to
+    // 112^3 at once 203.8 ms (196.1 with three blocks of 512).
+    const int vec_blocks = (n <= 2 * sms * kVecBlock ? 2 : 3) * sms;
     h->blockv = (int)std::min<int64_t>(kVecBlock, std::max<int64_t>(128, ((int64_t)n + vec_blocks - 1) / vec_blocks));
     h->blockv = (h->blockv + 31) / 32 * 32;
     h->gridv = std::min(vec_blocks, (n + h->blockv - 1) / h->blockv);
