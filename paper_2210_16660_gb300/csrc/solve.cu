@@ -1646,7 +1646,15 @@ int launch_direct(amg_hier *h, cudaStream_t s, int *kernels, bool *prolonged) {
         return AMG_OK;
     }
     const bool up = down_fused(h, D - 1, prec_index<T>());
-    if (h->op_first) {
+    // k_op holds a row in registers ahead of the wait. In float64, where the
+    // kernel before it needs the registers and the pipe, a coarsest inverse
+    // above kOpMax64 rows runs faster one warp per row: per iteration 1,896 rows
+    // 57.7 us with k_op and 56.3 with k_coarse, 2,285 76.2 and 66.3, 2,845 100.3
+    // and 86.2, 3,906 115.7 and 109.6; in float32 45.6 and 51.8 at 1,896 rows,
+    // 90.5 and 110.8 at 3,906 (62.8 and 61.7 at 2,285).
+    constexpr int kOpMax64 = 1280;
+    const bool whole = sizeof(T) == 4 || D + 1 < (int)h->lev.size() || h->nL <= kOpMax64;
+    if (h->op_first && whole) {
         if (up) launch_op<T, true>(h, D, up_of<T>(h, D - 1), s);
         else launch_op<T, false>(h, D, Up<T>{}, s);
     } else {
