@@ -1092,7 +1092,9 @@ int pairwise_pass(amg_hier *h, const DevCSR &cur, const double *w, int32_t **agg
 // the sweep's scattered rows. On larger levels they cost more than they save:
 // in member order the down sweep of 2,097,152 rows took 86 us (57 in row order
 // and 7 for the restriction), and 520,192 rows 31.6 us (26.1 and 4.4). The
-// largest aggregate has to fit a warp.
+// largest aggregate has to fit a warp. The array may take what dropping int32
+// columns has given back, or any free memory of a handle without a budget;
+// where it does not fit, the level transfers in launches of its own.
 int member_order(amg_hier *h, Level &lv, int members, cudaStream_t s) {
     Mem &M = h->mem;
     const int n = lv.A.n, nc = lv.nc;
@@ -1108,12 +1110,18 @@ int member_order(amg_hier *h, Level &lv, int members, cudaStream_t s) {
     int slot = 1;
     while (slot < most) slot <<= 1;
     const int64_t want = (int64_t)slot * nc;
-    if (slot <= 32) {
+    const int64_t main = (want + 31) / 32 * 32, all = main + (n - members + 31) / 32 * 32;
+    const size_t need = sizeof(int32_t) * (size_t)all + 256;  // allocations are rounded up to 256 bytes
+    bool fits = slot <= 32 && (!M.budget || need <= h->col_bytes);
+    if (fits && alloc(M, &lv.mrow, (size_t)all)) {
+        set_error("");
+        fits = false;
+    }
+    if (fits) {
         lv.mslot = slot;
-        lv.mmain = (int)((want + 31) / 32 * 32);
-        lv.mpos = lv.mmain + (n - members + 31) / 32 * 32;
-        PCG_TRY(alloc(M, &lv.mrow, lv.mpos));
-        h->col_bytes -= std::min(h->col_bytes, sizeof(int32_t) * (size_t)lv.mpos);
+        lv.mmain = (int)main;
+        lv.mpos = (int)all;
+        h->col_bytes -= std::min(h->col_bytes, need);
         k_member_rows<<<grid_for(lv.mpos), kBlock, 0, s>>>(nc, slot, lv.mpos, lv.rptr, lv.ridx, lv.mrow);
         k_left_out<<<grid_for(n), kBlock, 0, s>>>(n, lv.agg, lv.mrow + lv.mmain, dmax + 1);
         PCG_LAUNCH_CK();

@@ -7,6 +7,7 @@ past a warp the separate launches), ragged sizes and both column widths. The
 explicit matrix of the small levels (left out under a byte budget that has no
 room for it) is the same operator as the levels one by one, up to rounding.
 """
+import ctypes as C
 import os
 
 import numpy as np
@@ -50,6 +51,65 @@ def test_fused_transfers_give_the_bits_of_separate_launches(N, npass, cmax, env,
     r2, x2 = _solve(_amg(prob.A, tuple(env) + (("PCGAMG_TAIL", "0"),), **kw), b)
     assert r1.status == r2.status == 0 and r1.iters == r2.iters
     assert np.array_equal(r1.hist, r2.hist) and torch.equal(x1, x2)
+
+
+class _Bytes:
+    """An allocator that counts the library's bytes (rounded by it already)."""
+
+    def __enter__(self):
+        self.live, self.now, self.peak, self.limit = {}, 0, 0, None
+
+        def alloc(n, stream, ctx):
+            if self.limit is not None and self.now + n > self.limit:
+                return None
+            p = torch.cuda.caching_allocator_alloc(int(n), torch.cuda.current_device(), stream or 0)
+            self.live[p] = n
+            self.now += n
+            self.peak = max(self.peak, self.now)
+            return p
+
+        def free(p, stream, ctx):
+            self.now -= self.live.pop(p)
+            torch.cuda.caching_allocator_delete(p)
+
+        self.refs = (B.ALLOC_FN(alloc), B.FREE_FN(free))
+        assert B.load().amg_set_allocator(C.cast(self.refs[0], C.c_void_p), C.cast(self.refs[1], C.c_void_p), None) == 0
+        return self
+
+    def __exit__(self, *a):
+        B.load().amg_set_allocator(None, None, None)
+
+
+def _up(n, to):
+    return -(-n // to) * to
+
+
+@pytest.mark.parametrize("N,npass", [(24, 2), (14, 3)])
+def test_member_order_is_left_out_of_a_budget_without_room(N, npass):
+    """With int32 columns kept nothing is given back for the member order or the
+    explicit matrix: a budget of the rest is enough for the hierarchy."""
+    prob = W.make_problem(N, 1.04, seed=3)
+    b = torch.from_numpy(prob.b).cuda()
+    env = (("PCGAMG_COL16", "0"), ("PCGAMG_TAIL", "0"))
+    with _Bytes() as mem:
+        a1 = _amg(prob.A, env, n_pass=npass)
+        rows = [n for n, _ in a1.info()]
+        extra = 0
+        for l, n in enumerate(rows[:-1]):
+            agg = a1.level_agg(l, -1)[0]
+            cnt = np.bincount(agg[agg >= 0], minlength=rows[l + 1])
+            slot = 1 << int(cnt.max() - 1).bit_length()
+            extra += _up(4 * (_up(slot * rows[l + 1], 32) + _up(int((agg < 0).sum()), 32)), 256)
+            if l > 0 and n <= 1280:
+                extra += _up(8 * n * n, 256)
+        r1, x1 = _solve(a1, b)
+        need = mem.peak - extra
+        a1.close()
+        a2 = _amg(prob.A, env, n_pass=npass, hbm_budget=need)
+        r2, x2 = _solve(a2, b)
+        a2.close()
+    assert r1.status == r2.status == 0 and abs(r1.iters - r2.iters) <= 1
+    assert (x1 - x2).norm().item() <= 1e-6 * x2.norm().item()
 
 
 @pytest.mark.parametrize("mode", ["pcg64", "fcg32"])
