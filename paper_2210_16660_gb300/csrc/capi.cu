@@ -5,6 +5,7 @@
 #include <cstring>
 #include <iterator>
 #include <new>
+#include <utility>
 
 #include "internal.cuh"
 
@@ -31,23 +32,30 @@ static void *g_alloc_ctx = nullptr;
 
 // No arena under a byte budget (its one request could fail where the
 // temporaries one after another fit) or when the allocation fails.
-void Mem::arena_begin(size_t n) {
-    if (budget || dry || arena) return;
+void Mem::temps_begin(size_t arena_bytes) {
+    if (dry || temps) return;
     void *q = nullptr;
-    n = (n + 255) & ~(size_t)255;
-    if (alloc_bytes(&q, n)) {
-        set_error("");
-        return;
+    arena_bytes = (arena_bytes + 255) & ~(size_t)255;
+    if (!budget && arena_bytes) {
+        if (alloc_bytes(&q, arena_bytes)) {
+            set_error("");
+        } else {
+            arena = static_cast<char *>(q);
+            arena_free[0] = arena_bytes;
+        }
     }
-    arena = static_cast<char *>(q);
-    arena_free[0] = n;
+    temps = true;
 }
 
-void Mem::arena_end() {
+void Mem::temps_end() {
     char *q = arena;
     arena = nullptr;
     arena_free.clear();
     arena_live.clear();
+    temps = false;
+    const std::unordered_set<void *> left = std::move(temps_outside);
+    temps_outside.clear();
+    for (void *p : left) release(p);
     if (q) release(q);
 }
 
@@ -92,6 +100,7 @@ int Mem::alloc_bytes(void **p, size_t n) {
         }
     }
     live[q] = n;
+    if (temps) temps_outside.insert(q);
     bytes += n;
     if (bytes > peak) peak = bytes;
     *p = q;
@@ -122,6 +131,7 @@ void Mem::release(void *p) {
     if (it == live.end()) return;
     bytes -= it->second;
     live.erase(it);
+    temps_outside.erase(p);
     if (g_free) g_free(p, (void *)stream, g_alloc_ctx);
     else cudaFree(p);
 }
@@ -135,6 +145,8 @@ void Mem::release_all() {
     arena = nullptr;
     arena_free.clear();
     arena_live.clear();
+    temps_outside.clear();
+    temps = false;
     bytes = 0;
 }
 

@@ -7,6 +7,7 @@
 #include <map>
 #include <string>
 #include <unordered_map>
+#include <unordered_set>
 #include <vector>
 
 #include "pcgamg.h"
@@ -87,15 +88,18 @@ struct Mem {
     size_t bytes = 0, peak = 0, budget = 0;
     bool dry = false;  // count requests (rounded as real ones) without allocating
     std::unordered_map<void *, size_t> live;
-    // Arena of one call's temporaries (amg_refresh: all on one stream, so a
-    // released range may be handed out again at once): requests are served
-    // from one allocation, first fit, until arena_end gives it back. A request
-    // that does not fit goes to the allocator.
+    // One call's temporaries (amg_refresh: all on one stream, so a released
+    // range may be handed out again at once), from temps_begin to temps_end:
+    // requests are served from one allocation of `arena_bytes`, first fit, and
+    // what does not fit goes to the allocator. temps_end gives everything back
+    // that a failed call has left, and the arena.
+    bool temps = false;
     char *arena = nullptr;
     std::map<size_t, size_t> arena_free;              // offset -> bytes, disjoint and not adjacent
     std::unordered_map<void *, size_t> arena_live;
-    void arena_begin(size_t bytes);
-    void arena_end();
+    std::unordered_set<void *> temps_outside;         // live temporaries outside the arena
+    void temps_begin(size_t arena_bytes);
+    void temps_end();
     int alloc_bytes(void **p, size_t bytes);
     void release(void *p);
     void release_all();

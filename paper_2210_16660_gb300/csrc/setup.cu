@@ -1474,24 +1474,32 @@ int setup_impl(amg_hier *h, const amg_csr *A, const amg_params *prm, cudaStream_
 // and the coarsest inverse. Every array keeps its address, so captured solve
 // graphs, batch graphs and serving engines stay valid. Nothing is changed
 // when the input is rejected (AMG_ERR_ARG).
-// Its temporaries come from one allocation (Mem::arena): the new CSR, then a
-// pass's terms (20 bytes per fine entry) and coarse matrix.
-int refresh_in_arena(amg_hier *h, const amg_csr *A, cudaStream_t s);
+// Its temporaries come from one allocation (Mem::temps_begin): the new CSR, then a
+// pass's terms (20 bytes per fine entry) and coarse matrix. Where coarse rows
+// share few columns a later pass needs more, and if that is not to be had
+// beside the arena, the refresh is done again with single allocations (the
+// input is still the caller's, and a refresh starts from it alone).
+int refresh_values(amg_hier *h, const amg_csr *A, cudaStream_t s);
 int refresh_impl(amg_hier *h, const amg_csr *A, cudaStream_t s) {
     Mem &M = h->mem;
     const Level &l0 = h->lev[0];
     M.stream = s;
-    if (!h->smoothed && A && A->n == l0.A.n && A->nnz == l0.A.nnz)
-        M.arena_begin(36 * (size_t)l0.A.nnz + 96 * (size_t)l0.A.n + ((size_t)1 << 20));
-    int st = refresh_in_arena(h, A, s);
-    if (M.arena) {
-        cudaStreamSynchronize(s);  // no kernel may still read what goes back
-        M.arena_end();
+    // a smoothed hierarchy's refresh replaces arrays of its own
+    if (h->smoothed || !A || A->n != l0.A.n || A->nnz != l0.A.nnz) return refresh_values(h, A, s);
+    size_t arena = 36 * (size_t)l0.A.nnz + 96 * (size_t)l0.A.n + ((size_t)1 << 20);
+    for (;;) {
+        M.temps_begin(arena);
+        const bool one = M.arena != nullptr;
+        const int st = refresh_values(h, A, s);
+        if (one || st) cudaStreamSynchronize(s);  // no kernel may still read what goes back
+        M.temps_end();
+        if (st != AMG_ERR_OOM || !one) return st;
+        set_error("");
+        arena = 0;
     }
-    return st;
 }
 
-int refresh_in_arena(amg_hier *h, const amg_csr *A, cudaStream_t s) {
+int refresh_values(amg_hier *h, const amg_csr *A, cudaStream_t s) {
     double t_begin = now_ms();
     Mem &M = h->mem;
     M.stream = s;

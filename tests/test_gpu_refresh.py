@@ -7,6 +7,8 @@ matrices; kept aggregates), and solves meet the oracle's bar (iterations
 are updated in place, so graphs captured before the refresh (whole-solve,
 batch) must give the same bits as a handle refreshed before its first solve.
 """
+import ctypes as C
+
 import numpy as np
 import pytest
 
@@ -165,6 +167,85 @@ def test_refresh_rejections_leave_the_handle_unchanged():
     x1 = torch.zeros_like(b)
     amg.solve(b, x1)
     assert torch.equal(x0, x1)
+
+
+class _Bytes:
+    """An allocator that counts the library's bytes and refuses past `limit`."""
+
+    def __enter__(self):
+        self.live, self.now, self.peak, self.limit = {}, 0, 0, None
+
+        def alloc(n, stream, ctx):
+            if self.limit is not None and self.now + n > self.limit:
+                return None
+            p = torch.cuda.caching_allocator_alloc(int(n), torch.cuda.current_device(), stream or 0)
+            self.live[p] = n
+            self.now += n
+            self.peak = max(self.peak, self.now)
+            return p
+
+        def free(p, stream, ctx):
+            self.now -= self.live.pop(p)
+            torch.cuda.caching_allocator_delete(p)
+
+        self.refs = (B.ALLOC_FN(alloc), B.FREE_FN(free))
+        assert B.load().amg_set_allocator(C.cast(self.refs[0], C.c_void_p), C.cast(self.refs[1], C.c_void_p), None) == 0
+        return self
+
+    def __exit__(self, *a):
+        B.load().amg_set_allocator(None, None, None)
+
+
+def _scattered(n, deg, seed):
+    """A graph Laplacian plus the identity with `deg` far-flung neighbours a row:
+    two rows share hardly a column, so a coarse matrix keeps most entries."""
+    rng = np.random.default_rng(seed)
+    i = np.repeat(np.arange(n), deg // 2)
+    j = rng.integers(0, n, i.size)
+    key = np.unique(np.minimum(i, j)[i != j] * n + np.maximum(i, j)[i != j])
+    i, j = key // n, key % n
+    r = np.concatenate([i, j, np.arange(n)])
+    c = np.concatenate([j, i, np.arange(n)])
+    off = rng.uniform(-1.0, -0.1, i.size)
+    diag = 1.0 - np.bincount(np.concatenate([i, j]), np.concatenate([off, off]), minlength=n)
+    v = np.concatenate([off, off, diag])
+    order = np.lexsort((c, r))
+    rp = np.zeros(n + 1, np.int64)
+    np.cumsum(np.bincount(r, minlength=n), out=rp[1:])
+    return W.CSR(n, rp.astype(np.int32), c[order].astype(np.int32), v[order])
+
+
+def test_refresh_where_only_single_temporaries_fit():
+    """Temporaries that outgrow the refresh's one allocation: memory for them one
+    after another is enough, and the temporaries go back."""
+    A = _scattered(12000, 60, seed=1)
+    A2 = W.rescaled(A, seed=2)
+    b = torch.from_numpy(W.spmv(A2, W.normals(3, A.n))).cuda()
+    kw = dict(max_levels=2, coarse_max=10)
+    with _Bytes() as mem:
+        a1 = B.AMG.from_csr(A, hbm_budget=1 << 40, **kw)      # a budget: single allocations
+        start = mem.peak = mem.now
+        a1.refresh(A2)
+        single, after = mem.peak - start, mem.now
+        assert after == start
+        a2 = B.AMG.from_csr(A, **kw)
+        start = mem.peak = mem.now
+        a2.refresh(A2)
+        assert mem.peak - start > single and mem.now == start   # the arena does not hold them all
+        a3 = B.AMG.from_csr(A, **kw)
+        start = mem.now
+        mem.limit = start + single
+        a3.refresh(A2)
+        assert mem.now == start
+        mem.limit = start + single // 2
+        assert a3.refresh(A, check=False) == B.ERR_OOM and mem.now == start
+        mem.limit = None
+        a3.refresh(A2)
+        x2, x3 = torch.zeros_like(b), torch.zeros_like(b)
+        r2, r3 = a2.solve(b, x2, rtol=RTOL), a3.solve(b, x3, rtol=RTOL)
+        assert r2.status == r3.status == 0 and torch.equal(x2, x3)
+        for a in (a1, a2, a3):
+            a.close()
 
 
 def test_full_size_128_refresh():
