@@ -142,7 +142,7 @@ int ops_alloc(amg_hier *h) {
     const int L = (int)h->lev.size() - 1;
     h->op_first = 0;
     h->op.assign(L + 1, nullptr);
-    if (h->coarse_iter || L == 0) return AMG_OK;
+    if (h->coarse_iter || L == 0 || h->no_op) return AMG_OK;
     int D = 1;
     while (D < L && h->lev[D].A.n > kOpRows) D++;
     size_t need = 0;

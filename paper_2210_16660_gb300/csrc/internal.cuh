@@ -332,7 +332,8 @@ struct amg_hier {
     // The V-cycle from level op_first down as one explicit matrix (a fixed
     // linear operator with the dense coarsest solve), row-major float64:
     // op[l] for l = op_first..L-1, and the coarsest inverse itself at L.
-    // op_first = 0: none (iterative coarsest solve, or no room under the budget).
+    // op_first = 0: none (iterative coarsest solve, PCGAMG_OP=0, or no room under
+    // the budget).
     int op_first = 0;
     std::vector<double *> op;
     size_t col_bytes = 0;     // device bytes given back by dropping int32 columns beside int16 ones
@@ -385,6 +386,7 @@ struct amg_hier {
     int use_graph = 1;
     int fuse = 1;  // transfers inside the sweeps (PCGAMG_TAIL=0: every sweep and transfer its own launch)
     int no_col16 = 0;
+    int no_op = 0;    // PCGAMG_OP=0: no explicit operator
     int no_uniform = 0;  // PCGAMG_UNIFORM=0: no shared offset patterns on level 0
     int pdl = 1;  // programmatic dependent launch between solve kernels
     int graph_gen = 0;       // bumped whenever captured graphs go stale

@@ -1300,6 +1300,10 @@ int setup_impl(amg_hier *h, const amg_csr *A, const amg_params *prm, cudaStream_
     if (un && un[0] == '0') h->no_uniform = 1;
     const char *pd = getenv("PCGAMG_PDL");
     if (pd && pd[0] == '0') h->pdl = 0;
+    // PCGAMG_OP=0 sweeps the small levels one by one (or in the cluster tail)
+    // instead of applying their explicit matrix.
+    const char *op = getenv("PCGAMG_OP");
+    if (op && op[0] == '0') h->no_op = 1;
     // PCGAMG_GS_FUSED=0 keeps the two-launch Gauss-Seidel sweeps everywhere.
     const char *gf = getenv("PCGAMG_GS_FUSED");
     if (gf && gf[0] == '0') h->gs_fused = 0;

@@ -2174,8 +2174,9 @@ bool is_device_ptr(const void *p) {
 
 }  // namespace
 
-// Shared-memory cluster tail (tail.cu); PCGAMG_TAIL=0 launches every level
-// separately instead.
+// Shared-memory cluster tail (tail.cu) of a handle without the explicit
+// operator. PCGAMG_TAIL=0: no tail and no transfers inside the sweeps, every
+// sweep and transfer of the levels above the directly solved one its own launch.
 int setup_tail(amg_hier *h) {
     h->tail_first[0] = h->tail_first[1] = 0;
     const char *e = getenv("PCGAMG_TAIL");

@@ -4,8 +4,8 @@ The down sweep that restricts in the same launch (member order) and the
 kernels that prolong the x they form give the bits of the separate launches
 (PCGAMG_TAIL=0): checked for aggregates of 2 to 64 rows (slots of 2 to 32, and
 past a warp the separate launches), ragged sizes and both column widths. The
-explicit matrix of the small levels (left out under a byte budget that has no
-room for it) is the same operator as the levels one by one, up to rounding.
+explicit matrix of the small levels (left out by PCGAMG_OP=0) is the same
+operator as the levels one by one, up to rounding.
 """
 import ctypes as C
 import os
@@ -19,6 +19,7 @@ torch = pytest.importorskip("torch")
 
 from paper_2210_16660_gb300 import binding as B  # noqa: E402
 from paper_2210_16660_gb300 import workloads as W  # noqa: E402
+from test_gpu_parity import direct_level  # noqa: E402
 
 
 def _amg(A, env=(), **kw):
@@ -120,7 +121,10 @@ def test_small_levels_as_one_matrix(N, kw, nu, rows, mode):
     prob = W.make_problem(N, 1.04, seed=4)
     b = torch.from_numpy(prob.b).cuda()
     A2 = W.rescaled(prob.A, seed=9)
-    amgs = [B.AMG.from_csr(prob.A, mode=mode, **kw), B.AMG.from_csr(prob.A, mode=mode, hbm_budget=1 << 34, **kw)]
+    amgs = [_amg(prob.A, mode=mode, **kw),
+            _amg(prob.A, (("PCGAMG_OP", "0"), ("PCGAMG_TAIL", "0")), mode=mode, **kw)]
+    L = len(amgs[0].info()) - 1
+    assert direct_level(amgs[0], b) < L and direct_level(amgs[1], b) == L
     for step in ("setup", "refresh"):
         out = []
         for a in amgs:
@@ -128,11 +132,10 @@ def test_small_levels_as_one_matrix(N, kw, nu, rows, mode):
                 a.refresh(A2)
             elif nu:
                 a.set_smoother(nu, -(-prob.A.n // rows))
-            n0 = a.launch_count()
             r, x = _solve(a, b)
             assert r.status == 0, r.message
-            out.append((r, x, a.launch_count() - n0))
-        (r1, x1, n1), (r2, x2, n2) = out
+            out.append((r, x))
+        (r1, x1), (r2, x2) = out
         assert abs(r1.iters - r2.iters) <= 1
         # the two V-cycles differ by rounding alone: u = 2^-53 per operation in
         # float64 (2^-24 in float32), a few hundred operations deep, so the

@@ -196,6 +196,16 @@ def test_graph_and_stream_launch_paths_agree():
         assert prof["spmv"][1] >= r1.iters and prof["spmv"][0] > 0
 
 
+def direct_level(amg, b):
+    """The first level solved in one launch, from a profiled solve: the explicit
+    operator's, the cluster tail's, or the coarsest one."""
+    amg.profile(True)
+    amg.solve(b, torch.zeros_like(b))
+    _, counts = amg.profile_levels()
+    amg.profile(False)
+    return int(np.flatnonzero(counts[:, 2])[0])
+
+
 def _with_env(key, val, fn):
     import os
     old = os.environ.get(key)
@@ -249,12 +259,15 @@ def test_restarts_run_to_maxit_on_both_launch_paths(mode, maxit):
 @pytest.mark.parametrize("N", [32, 64])
 def test_cluster_tail_matches_separate_launches(mode, N):
     """Small levels in one thread-block cluster with their data in shared
-    memory (the default) give the same solve, bit for bit, as one launch per
-    sweep (PCGAMG_TAIL=0)."""
+    memory (handles without the explicit operator) give the same solve, bit for
+    bit, as one launch per sweep (PCGAMG_TAIL=0)."""
     prob = W.make_problem(N, 1.04, seed=10)
     b = torch.from_numpy(prob.b).cuda()
-    a1 = B.AMG.from_csr(prob.A, mode=mode)
-    a2 = _with_env("PCGAMG_TAIL", "0", lambda: B.AMG.from_csr(prob.A, mode=mode))
+    a1 = _with_env("PCGAMG_OP", "0", lambda: B.AMG.from_csr(prob.A, mode=mode))
+    a2 = _with_env("PCGAMG_OP", "0", lambda: _with_env("PCGAMG_TAIL", "0",
+                                                       lambda: B.AMG.from_csr(prob.A, mode=mode)))
+    L = len(a1.info()) - 1
+    assert 1 <= direct_level(a1, b) < L and direct_level(a2, b) == L    # with the tail, without
     x1, x2 = torch.zeros_like(b), torch.zeros_like(b)
     n1, n2 = a1.launch_count(), a2.launch_count()
     r1, r2 = a1.solve(b, x1), a2.solve(b, x2)

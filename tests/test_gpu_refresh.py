@@ -19,6 +19,7 @@ torch = pytest.importorskip("torch")
 import oracle as O  # noqa: E402
 from paper_2210_16660_gb300 import binding as B  # noqa: E402
 from paper_2210_16660_gb300 import workloads as W  # noqa: E402
+from test_gpu_parity import direct_level  # noqa: E402
 
 RTOL = 1e-8
 X_TOL = 1e-6
@@ -130,12 +131,14 @@ def test_cluster_tail_is_refreshed():
     prob = W.make_problem(48, 1.04, seed=15)
     A2 = W.rescaled(prob.A, seed=16)
     b = torch.from_numpy(_rhs(A2, 17)).cuda()
-    a1 = B.AMG.from_csr(prob.A, mode="fcg32")
-    os.environ["PCGAMG_TAIL"] = "0"
+    os.environ["PCGAMG_OP"] = "0"                # the levels of the tail are not one matrix
     try:
+        a1 = B.AMG.from_csr(prob.A, mode="fcg32")
+        os.environ["PCGAMG_TAIL"] = "0"
         a2 = B.AMG.from_csr(prob.A, mode="fcg32")
     finally:
-        del os.environ["PCGAMG_TAIL"]
+        del os.environ["PCGAMG_OP"], os.environ["PCGAMG_TAIL"]
+    assert direct_level(a1, b) < direct_level(a2, b) == len(a2.info()) - 1
     a1.refresh(A2)
     a2.refresh(A2)
     x1, x2 = torch.zeros_like(b), torch.zeros_like(b)
