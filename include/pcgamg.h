@@ -440,8 +440,9 @@ int amg_profile_read(amg_handle h, double *ms, int64_t *counts, int nkinds);
  * of 3 nlev values (nlev <= 32), or NULL. */
 int amg_profile_levels(amg_handle h, int nlev, double *ms, int64_t *counts);
 
-/* Kernels launched by solves on h since setup (every launch, including the
- * ones that find the solve finished and return at once). */
+/* Kernels launched by solves on h and by amg_autotune since setup (every
+ * launch, including the ones that find the solve finished and return at
+ * once). */
 int64_t amg_launch_count(amg_handle h);
 
 /* r = b - A x on the finest level of h, with norms[0] = ||r||_2 and

@@ -1382,12 +1382,15 @@ Geo shape_geo(const amg_hier *h, int n, int pi, int sweep, unsigned char shape) 
     return {w > 0 && w < g ? w : g, blk};
 }
 
-// Whether level l's down sweep restricts in the same launch (member order);
-// l >= 1 only with a down shape that is not one of the older forms.
-bool down_fused(const amg_hier *h, int l, int pi) {
+// Whether level l's down sweep can restrict in the same launch (member order),
+// and whether it does: on l >= 1 only with a down shape that is not one of the
+// older forms.
+bool fusable(const amg_hier *h, int l) {
     const Level &lv = h->lev[l];
-    return h->fuse && lv.mslot > 0 && !h->smoothed && !h->gs_nu && !(h->no_tail && lv.A.n > kFuseRowsShared) &&
-           (l == 0 || !(lv.shape[pi][0] & 12));
+    return h->fuse && lv.mslot > 0 && !h->smoothed && !h->gs_nu && !(h->no_tail && lv.A.n > kFuseRowsShared);
+}
+bool down_fused(const amg_hier *h, int l, int pi) {
+    return fusable(h, l) && (l == 0 || !(h->lev[l].shape[pi][0] & 12));
 }
 
 // Weight of the down sweep's output t = w (b - A xpre): the tentative
@@ -2293,42 +2296,82 @@ int alloc_solve_workspace(amg_hier *h) {
     return AMG_OK;
 }
 
-// Launch-shape tuner: for every level l in 1..L-1 (the levels with down and
-// post sweeps), each V-cycle precision and each phase (down: down sweep +
-// restriction; up: prolongation + post sweep), times the eight shapes
-// (4- or 16-entry chunks x one-wave or one-thread-per-row grid x separate or
-// fused launches) on this device, `reps` runs each after one warm-up run,
-// and moves to the fastest only if it beats the current shape by more than
-// 3% (so timing noise does not flip shapes). Work vectors are zeroed first;
-// the inputs only set the timing. Captured solve graphs are dropped.
+// Launch-shape tuner: for every swept level l >= 1, from the coarsest up, each
+// V-cycle precision and each phase (down: down sweep + restriction; up:
+// prolongation + post sweep), times the nine shapes (4- or 16-entry chunks x
+// one-wave or one-thread-per-row grid x separate sweeps and transfers or those
+// fused by aggregate; rows by four lanes) on this device, `reps` runs each
+// after one warm-up run, and moves to the fastest only if it beats the current
+// shape by more than 3% (so timing noise does not flip shapes). A candidate is
+// timed as it would run: it is the level's shape meanwhile, as that decides
+// which transfers are fused, and a prolongation that it leaves to a launch of
+// its own where another candidate would not is timed with it. Work vectors are
+// zeroed first; the inputs only set the timing. Captured solve graphs are
+// dropped.
 constexpr int kShapes = 9;  // 0..7, and 8: multi-lane rows
+
+// Whether the kernel that forms x_{l+1} prolongs it to a level l that is fused.
+template <typename T>
+bool below_prolongs(const amg_hier *h, int l) {
+    const int pi = prec_index<T>();
+    const int tf = h->no_tail || h->op_first ? 0 : h->tail_first[pi];
+    if (l + 1 >= (tf > 0 ? tf : direct_level(h))) return tf == 0 && !h->coarse_iter;
+    return !(h->lev[l + 1].shape[pi][1] & 12);
+}
+
+// One run of a level's down (sweep = 0) or up phase with its current shapes
+// (an up shape with bit 2 takes no prolongation).
+template <typename T>
+void run_phase(amg_hier *h, int l, int sweep, cudaStream_t s) {
+    const int pi = prec_index<T>();
+    const unsigned char *sh = h->lev[l].shape[pi];
+    const bool ready = down_fused(h, l, pi) && below_prolongs<T>(h, l);
+    int kernels = 0;
+    if (sweep == 0) {
+        launch_down_phase<T>(h, l, sh[0], s, &kernels);
+        if (!ready && fusable(h, l) && below_prolongs<T>(h, l) && !(sh[1] & 4)) {
+            launch_prolong<T>(h, l, grid_rows(h->lev[l].A.n), s);
+            kernels += 1;
+        }
+    } else if (!launch_up_phase<T>(h, l, sh[1], ready, s, &kernels) && down_fused(h, l - 1, pi) &&
+               (l == 1 || !(h->lev[l - 1].shape[pi][1] & 4))) {
+        launch_prolong<T>(h, l - 1, l == 1 ? h->gridp : grid_rows(h->lev[l - 1].A.n), s);
+        kernels += 1;
+    }
+    h->launches += kernels;
+}
+
 template <typename T>
 int tune_level(amg_hier *h, int l, cudaStream_t s, int reps, cudaEvent_t e0, cudaEvent_t e1, int *changed) {
-    int pi = prec_index<T>();
-    Level &lv = h->lev[l];
+    const int pi = prec_index<T>();
     for (int sweep = 0; sweep < 2; sweep++) {
+        unsigned char &shape = h->lev[l].shape[pi][sweep];
+        const unsigned char had = shape;
         float best = 0.0f, cur = 0.0f;
-        int pick = -1, kernels = 0;
-        for (int shape = 0; shape < kShapes; shape++) {
-            for (int r = -1; r < reps; r++) {
-                if (r == 0) PCG_CK(cudaEventRecord(e0, s));
-                if (sweep == 0) launch_down_phase<T>(h, l, (unsigned char)shape, s, &kernels);
-                else launch_up_phase<T>(h, l, (unsigned char)shape, down_fused(h, l, pi), s, &kernels);
-            }
-            PCG_CK(cudaEventRecord(e1, s));
-            PCG_CK(cudaEventSynchronize(e1));
-            PCG_LAUNCH_CK();
+        int pick = -1;
+        cudaError_t e = cudaSuccess;
+        for (int c = 0; c < kShapes && e == cudaSuccess; c++) {
+            shape = (unsigned char)c;
+            run_phase<T>(h, l, sweep, s);
+            e = cudaEventRecord(e0, s);
+            for (int r = 0; r < reps; r++) run_phase<T>(h, l, sweep, s);
+            if (e == cudaSuccess) e = cudaEventRecord(e1, s);
+            if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+            if (e == cudaSuccess) e = cudaGetLastError();
             float ms = 0.0f;
-            PCG_CK(cudaEventElapsedTime(&ms, e0, e1));
-            if (shape == lv.shape[pi][sweep]) cur = ms;
+            if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+            if (c == had) cur = ms;
             if (pick < 0 || ms < best) {
                 best = ms;
-                pick = shape;
+                pick = c;
             }
         }
-        if (best > 0.97f * cur) pick = lv.shape[pi][sweep];
-        if (lv.shape[pi][sweep] != pick) (*changed)++;
-        lv.shape[pi][sweep] = (unsigned char)pick;
+        shape = had;
+        PCG_CK(e);
+        if (best <= 0.97f * cur && pick != had) {
+            shape = (unsigned char)pick;
+            (*changed)++;
+        }
     }
     return AMG_OK;
 }
@@ -2353,7 +2396,7 @@ int autotune_impl(amg_hier *h, cudaStream_t s, int reps, int *changed) {
     cudaError_t ce = cudaEventCreate(&e0);
     if (ce == cudaSuccess) ce = cudaEventCreate(&e1);
     if (ce != cudaSuccess) st = cuda_fail(ce, "autotune events", __FILE__, __LINE__);
-    for (int l = 1; l < direct_level(h) && !st; l++) {
+    for (int l = direct_level(h) - 1; l >= 1 && !st; l--) {
         st = tune_level<float>(h, l, s, reps, e0, e1, changed);
         if (!st) st = tune_level<double>(h, l, s, reps, e0, e1, changed);
     }

@@ -341,6 +341,26 @@ def test_full_size_128_graded(mode):
     assert np.linalg.norm(xs - ref["x"]) / np.linalg.norm(ref["x"]) <= X_TOL
 
 
+def test_autotune_times_what_a_shape_would_run():
+    """A fused down sweep is timed fused also where the level's present shape is
+    an older form, and the others with the prolongation that they leave over."""
+    prob = W.make_problem(24, 1.04, seed=6)
+    amg = B.AMG.from_csr(prob.A, mode="fcg32")
+    b = torch.from_numpy(prob.b).cuda()
+    assert direct_level(amg, b) == 2                    # one level is tuned
+    amg.set_level_shape(1, [4, 3, 4, 3])
+    n0, reps = amg.launch_count(), 2
+    amg.autotune(reps=reps)
+    n = amg.launch_count() - n0
+    # down: shapes 0..3 one launch each, 4..7 and a prolongation, 8 a sweep, a
+    # restriction and a prolongation
+    down = 4 * 1 + 4 * 2 + 3
+    # up, after a fused down shape: 0..3 prolong to level 0 as well, 4..8 leave that
+    # to a launch; after another: 0..3 and 8 one prolongation more
+    fused, other = down + 4 * 1 + 4 * 2 + 2, down + 4 * 2 + 4 * 2 + 3
+    assert n in [(reps + 1) * (p + q) for p in (fused, other) for q in (fused, other)]
+
+
 @pytest.mark.parametrize("mode", ["pcg64", "fcg32"])
 def test_every_launch_shape_gives_the_same_bits(mode):
     """Sweep launch shapes (chunk depth x grid form x fused or separate
