@@ -358,7 +358,8 @@ void amg_server_destroy(amg_server s);
  * bits before and after tuning; only their speed changes. The level work
  * vectors are overwritten; captured solve graphs are rebuilt on the next
  * solve. *changed (may be NULL): shapes that differ from before. Call it
- * between solves, not while a batch or server holding h is in use. */
+ * between solves, not while a batch or server holding h is in use. Batches and
+ * servers, whose solves share the device, do not take the picked shapes. */
 int amg_autotune(amg_handle h, int reps, int *changed, void *stream);
 
 /* Launch shapes of a level (4 ints: float down, float up, float64 down,

@@ -291,7 +291,10 @@ int amg_set_level_shape(amg_handle h, int level, const int *shape) {
             return AMG_ERR_ARG;
         }
     for (int p = 0; p < 2; p++)
-        for (int k = 0; k < 2; k++) h->lev[level].shape[p][k] = (unsigned char)shape[2 * p + k];
+        for (int k = 0; k < 2; k++) {
+            h->lev[level].shape[p][k] = (unsigned char)shape[2 * p + k];
+            h->lev[level].tuned[p][k] = false;
+        }
     drop_graphs(h);
     return AMG_OK;
 }

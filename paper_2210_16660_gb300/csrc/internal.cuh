@@ -212,6 +212,8 @@ struct Level {
     // shape. The shape never changes a result: every shape forms the same
     // values and sums a row's entries in storage order.
     unsigned char shape[2][2] = {{0, 0}, {0, 0}};
+    unsigned char rule_shape = 0;                     // the fixed rule's
+    bool tuned[2][2] = {{false, false}, {false, false}};  // shape picked by amg_autotune
 };
 
 // Device-resident Krylov state; every scalar of the iteration lives here so

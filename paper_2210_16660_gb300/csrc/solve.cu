@@ -1382,6 +1382,14 @@ Geo shape_geo(const amg_hier *h, int n, int pi, int sweep, unsigned char shape) 
     return {w > 0 && w < g ? w : g, blk};
 }
 
+// Level l's shape of a phase (0 down, 1 up). The tuner times a shape alone;
+// solves that share the device keep the fixed rule's in place of its picks (48
+// systems of 24^3 to 112^3 at once 196.4 ms, 200.8 with them).
+unsigned char shape_of(const amg_hier *h, int l, int pi, int phase) {
+    const Level &lv = h->lev[l];
+    return h->no_tail && lv.tuned[pi][phase] ? lv.rule_shape : lv.shape[pi][phase];
+}
+
 // Whether level l's down sweep can restrict in the same launch (member order),
 // and whether it does: on l >= 1 only with a down shape that is not one of the
 // older forms.
@@ -1390,7 +1398,7 @@ bool fusable(const amg_hier *h, int l) {
     return h->fuse && lv.mslot > 0 && !h->smoothed && !h->gs_nu && !(h->no_tail && lv.A.n > kFuseRowsShared);
 }
 bool down_fused(const amg_hier *h, int l, int pi) {
-    return fusable(h, l) && (l == 0 || !(h->lev[l].shape[pi][0] & 12));
+    return fusable(h, l) && (l == 0 || !(shape_of(h, l, pi, 0) & 12));
 }
 
 // Weight of the down sweep's output t = w (b - A xpre): the tentative
@@ -1765,9 +1773,8 @@ int launch_vcycle(amg_hier *h, bool step, cudaStream_t s) {
     // sweep and the restriction that leaves it (level 0: the restriction)
     int kernels = 1;  // down sweep of level 0
     for (int l = 0; l < F; l++) {
-        Level &lv = lev[l];
         int spl = prof_begin(h, kLevelSpan + 3 * l, s);
-        unsigned char sh = lv.shape[prec_index<T>()][0];
+        unsigned char sh = shape_of(h, l, prec_index<T>(), 0);
         if (l == 0) {
             if (!down_fused(h, 0, prec_index<T>())) {
                 launch_restrict<T>(h, 0, s);
@@ -1788,9 +1795,8 @@ int launch_vcycle(amg_hier *h, bool step, cudaStream_t s) {
     }
     prof_end(h, spc, s);
     for (int l = F - 1; l >= 1; l--) {
-        Level &lv = lev[l];
         int spl = prof_begin(h, kLevelSpan + 3 * l + 1, s);
-        xp_ready = launch_up_phase<T>(h, l, lv.shape[prec_index<T>()][1], xp_ready, s, &kernels);
+        xp_ready = launch_up_phase<T>(h, l, shape_of(h, l, prec_index<T>(), 1), xp_ready, s, &kernels);
         prof_end(h, spl, s);
     }
     kernels += 1;  // post sweep of level 0
@@ -1942,7 +1948,7 @@ int launch_vcycle_gs(amg_hier *h, cudaStream_t s) {
     int sp2 = prof_begin(h, 5, s);
     for (int l = 0; l < L; l++) {
         int spl = prof_begin(h, kLevelSpan + 3 * l, s);
-        unsigned char sh = lev[l].shape[prec_index<T>()][0];
+        unsigned char sh = shape_of(h, l, prec_index<T>(), 0);
         if (l == 0) {
             launch_restrict<T>(h, 0, s);
             kernels += 1;
@@ -2275,6 +2281,7 @@ int alloc_solve_workspace(amg_hier *h) {
             }
     for (size_t l = 1; l < h->lev.size(); l++) {
         unsigned char d = (unsigned char)((h->lev[l].A.n <= kSmallRows ? 1 : 0) | 2);
+        h->lev[l].rule_shape = d;
         for (auto &pr : h->lev[l].shape) pr[0] = pr[1] = d;
     }
     PCG_TRY(alloc(M, &h->b, n));
@@ -2370,6 +2377,7 @@ int tune_level(amg_hier *h, int l, cudaStream_t s, int reps, cudaEvent_t e0, cud
         PCG_CK(e);
         if (best <= 0.97f * cur && pick != had) {
             shape = (unsigned char)pick;
+            h->lev[l].tuned[pi][sweep] = true;
             (*changed)++;
         }
     }

@@ -99,3 +99,29 @@ def test_full_size_48_systems():
             assert abs(ref["iters"] - int(it[k])) <= 1
             assert np.linalg.norm(xh - ref["x"]) <= 1e-6 * np.linalg.norm(ref["x"])
     batch.close()
+
+
+@pytest.mark.parametrize("mode", ["pcg64", "fcg32"])
+def test_batches_keep_the_fixed_shapes_of_tuned_handles(mode):
+    """Shapes picked by timing a solve alone are not taken into a batch; shapes set
+    by hand are."""
+    prob = W.make_problem(64, 1.04, seed=6)
+    b = torch.from_numpy(prob.b).cuda()
+
+    def launches(prepare):
+        amg = B.AMG.from_csr(prob.A, mode=mode)
+        prepare(amg)
+        batch, x = B.Batch([amg]), torch.zeros_like(b)
+        n0 = amg.launch_count()
+        st, it, _ = batch.solve([b], [x], rtol=1e-8)
+        assert st == 0
+        n = amg.launch_count() - n0
+        batch.close()
+        amg.close()
+        return n, int(it[0]), x
+
+    n0, it0, x0 = launches(lambda a: None)
+    n1, it1, x1 = launches(lambda a: a.autotune(reps=3))
+    n2, it2, x2 = launches(lambda a: [a.set_level_shape(l, [8, 8, 8, 8]) for l in range(1, len(a.info()))])
+    assert it0 == it1 == it2 and torch.equal(x0, x1) and torch.equal(x0, x2)
+    assert n0 == n1 < n2
