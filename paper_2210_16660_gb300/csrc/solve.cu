@@ -1354,7 +1354,7 @@ constexpr int kPartsRz = 0, kPartsPq = 1, kPartsRr = 2, kPartsTrue = 3, kPartSec
 
 // Threads per block of a sweep with one thread per row: small levels spread
 // over the SMs (4,096 rows are 64 blocks of 64 rows, not 16 of 256).
-int small_block(int n) { return n <= 152 * 64 ? 64 : n <= 152 * 128 ? 128 : kBlock; }
+int small_block(const amg_hier *h, int n) { return n <= h->sms * 64 ? 64 : n <= h->sms * 128 ? 128 : kBlock; }
 
 // Rows up to which a level's rows are read whole (WholeRow: one thread per
 // row, ~100 registers in float32); above, 16-entry chunks keep more warps
@@ -1370,17 +1370,20 @@ constexpr int kWholeRowsShared = 1024;
 constexpr int kFuseRowsShared = 4096;
 int whole_rows(const amg_hier *h) { return h->no_tail ? kWholeRowsShared : kWholeRows; }
 
-// Blocks and threads of a coarse-level sweep over n rows (or positions).
-struct Geo {
-    int grid, block;
-};
-Geo shape_geo(const amg_hier *h, int n, int pi, int sweep, unsigned char shape) {
-    const int blk = shape & 1 ? small_block(n) : kBlock;
-    const int g = (n + blk - 1) / blk;
-    if (shape & 2) return {g, blk};
-    const int w = h->wave[pi][sweep][shape & 1] * (kBlock / blk);
-    return {w > 0 && w < g ? w : g, blk};
+// A coarse-level sweep over n rows (or positions) in a launch shape: a thread
+// per row, or without bit 1 at most one wave of the kernel's resident blocks.
+template <typename... KArgs, typename... Args>
+void launch_shaped(const amg_hier *h, void (*kernel)(KArgs...), int n, unsigned char shape, int blk, cudaStream_t s,
+                   Args... args) {
+    int g = (n + blk - 1) / blk;
+    if (!(shape & 2)) {
+        int per = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, blk, 0) != cudaSuccess || per < 1) per = 1;
+        g = std::min(g, h->sms * per);
+    }
+    launch_k(h->pdl, kernel, g, blk, s, args...);
 }
+int shape_block(const amg_hier *h, int n, unsigned char shape) { return shape & 1 ? small_block(h, n) : kBlock; }
 
 // Level l's shape of a phase (0 down, 1 up). The tuner times a shape alone;
 // solves that share the device keep the fixed rule's in place of its picks (48
@@ -1437,17 +1440,17 @@ void launch_down(amg_hier *h, int l, unsigned char shape, cudaStream_t s) {
                                   P::t(lv), (const Ctl *)h->ctl)));
         return;
     }
-    const Geo g = shape_geo(h, n, prec_index<T>(), 0, shape);
+    const int blk = shape_block(h, n, shape);
     if ((shape & 1) && n <= whole_rows(h))
-        WITH_COLS(lv.S, (launch_k(h->pdl, k_down<T, IDX, kWholeRow, false, false>, g.grid, g.block, s, n, lv.S.sptr,
+        WITH_COLS(lv.S, (launch_shaped(h, k_down<T, IDX, kWholeRow, false, false>, n, shape, blk, s, n, lv.S.sptr,
                                   cols, P::val(lv), pats, P::xpre(lv), P::b(lv), pdown<T>(h, lv), P::t(lv),
                                   (const double *)nullptr, 0, h->ctl, (double *)nullptr)));
     else if (shape & 1)
-        WITH_COLS(lv.S, (launch_k(h->pdl, k_down<T, IDX, kUnrollSmall, false, false>, g.grid, g.block, s, n,
+        WITH_COLS(lv.S, (launch_shaped(h, k_down<T, IDX, kUnrollSmall, false, false>, n, shape, blk, s, n,
                                   lv.S.sptr, cols, P::val(lv), pats, P::xpre(lv), P::b(lv), pdown<T>(h, lv),
                                   P::t(lv), (const double *)nullptr, 0, h->ctl, (double *)nullptr)));
     else
-        WITH_COLS(lv.S, (launch_k(h->pdl, k_down<T, IDX, kUnroll, false, false>, g.grid, g.block, s, n, lv.S.sptr, cols,
+        WITH_COLS(lv.S, (launch_shaped(h, k_down<T, IDX, kUnroll, false, false>, n, shape, blk, s, n, lv.S.sptr, cols,
                                   P::val(lv), pats, P::xpre(lv), P::b(lv), pdown<T>(h, lv), P::t(lv),
                                   (const double *)nullptr, 0, h->ctl, (double *)nullptr)));
 }
@@ -1491,13 +1494,13 @@ Up<T> up_of(amg_hier *h, int to) {
 
 // Down sweep of level l with its restriction in one launch (down_fused).
 template <typename T, typename TO, int U, bool STREAM, bool STEP>
-void launch_down_r(amg_hier *h, int l, const T *b, TO *bc, bool pre, Geo g, cudaStream_t s) {
+void launch_down_r(amg_hier *h, int l, const T *b, TO *bc, bool pre, unsigned char shape, int blk, cudaStream_t s) {
     using P = LP<T>;
     Level &lv = h->lev[l];
     Level &nx = h->lev[l + 1];
     int lg = 0;
     while ((1 << lg) < lv.mslot) lg++;
-    WITH_COLS(lv.S, (launch_k(h->pdl, k_down_r<T, TO, IDX, U, STREAM, STEP>, g.grid, g.block, s,
+    WITH_COLS(lv.S, (launch_shaped(h, k_down_r<T, TO, IDX, U, STREAM, STEP>, lv.mpos, shape, blk, s,
                               DownR<T, TO, IDX>{lv.mrow, lv.mpos, lv.mmain, lg, lv.S.sptr, cols, P::val(lv), pats,
                                                 P::xpre(lv), b, P::p(lv), bc, pre ? P::dinv(nx) : nullptr,
                                                 pre ? P::xpre(nx) : nullptr, P::xp(lv),
@@ -1513,22 +1516,22 @@ void launch_down_phase(amg_hier *h, int l, unsigned char shape, cudaStream_t s, 
     using P = LP<T>;
     if (down_fused(h, l, prec_index<T>()) && !(shape & 12)) {
         Level &lv = h->lev[l];
-        const Geo g = shape_geo(h, lv.mpos, prec_index<T>(), 0, shape);
+        const int blk = shape_block(h, lv.mpos, shape);
         const T *b = P::b(lv);
         *kernels += 1;
         if (l + 1 == direct_level(h)) {
             if ((shape & 1) && lv.A.n <= whole_rows(h))
-                launch_down_r<T, double, kWholeRow, false, false>(h, l, b, h->bL, false, g, s);
+                launch_down_r<T, double, kWholeRow, false, false>(h, l, b, h->bL, false, shape, blk, s);
             else if (shape & 1)
-                launch_down_r<T, double, kUnrollSmall, false, false>(h, l, b, h->bL, false, g, s);
-            else launch_down_r<T, double, kUnroll, false, false>(h, l, b, h->bL, false, g, s);
+                launch_down_r<T, double, kUnrollSmall, false, false>(h, l, b, h->bL, false, shape, blk, s);
+            else launch_down_r<T, double, kUnroll, false, false>(h, l, b, h->bL, false, shape, blk, s);
         } else {
             T *bc = P::b(h->lev[l + 1]);
             if ((shape & 1) && lv.A.n <= whole_rows(h))
-                launch_down_r<T, T, kWholeRow, false, false>(h, l, b, bc, true, g, s);
+                launch_down_r<T, T, kWholeRow, false, false>(h, l, b, bc, true, shape, blk, s);
             else if (shape & 1)
-                launch_down_r<T, T, kUnrollSmall, false, false>(h, l, b, bc, true, g, s);
-            else launch_down_r<T, T, kUnroll, false, false>(h, l, b, bc, true, g, s);
+                launch_down_r<T, T, kUnrollSmall, false, false>(h, l, b, bc, true, shape, blk, s);
+            else launch_down_r<T, T, kUnroll, false, false>(h, l, b, bc, true, shape, blk, s);
         }
         return;
     }
@@ -1573,18 +1576,18 @@ void launch_post(amg_hier *h, int l, unsigned char shape, cudaStream_t s) {
         return;
     }
     const Up<T> up = UP ? up_of<T>(h, l - 1) : Up<T>{};
-    const Geo g = shape_geo(h, n, prec_index<T>(), 1, shape);
+    const int blk = shape_block(h, n, shape);
     if ((shape & 1) && n <= whole_rows(h))
-        WITH_COLS(lv.S, (launch_k(h->pdl, k_post<T, T, false, false, IDX, kWholeRow, false, UP>, g.grid, g.block, s,
+        WITH_COLS(lv.S, (launch_shaped(h, k_post<T, T, false, false, IDX, kWholeRow, false, UP>, n, shape, blk, s,
                                   n, lv.S.sptr, cols, P::val(lv), pats, P::xp(lv), P::b(lv), P::dinv(lv), P::x(lv),
                                   (const double *)nullptr, (const double *)nullptr, (double *)nullptr, h->ctl, up)));
     else if (shape & 1)
-        WITH_COLS(lv.S, (launch_k(h->pdl, k_post<T, T, false, false, IDX, kUnrollSmall, false, UP>, g.grid, g.block,
+        WITH_COLS(lv.S, (launch_shaped(h, k_post<T, T, false, false, IDX, kUnrollSmall, false, UP>, n, shape, blk,
                                   s, n, lv.S.sptr, cols, P::val(lv), pats, P::xp(lv), P::b(lv), P::dinv(lv),
                                   P::x(lv), (const double *)nullptr, (const double *)nullptr, (double *)nullptr,
                                   h->ctl, up)));
     else
-        WITH_COLS(lv.S, (launch_k(h->pdl, k_post<T, T, false, false, IDX, kUnroll, false, UP>, g.grid, g.block, s, n,
+        WITH_COLS(lv.S, (launch_shaped(h, k_post<T, T, false, false, IDX, kUnroll, false, UP>, n, shape, blk, s, n,
                                   lv.S.sptr, cols, P::val(lv), pats, P::xp(lv), P::b(lv), P::dinv(lv), P::x(lv),
                                   (const double *)nullptr, (const double *)nullptr, (double *)nullptr, h->ctl, up)));
 }
@@ -1613,13 +1616,12 @@ bool launch_up_phase(amg_hier *h, int l, unsigned char shape, bool xp_ready, cud
         launch_post<T, false>(h, l, shape, s);
         return false;
     }
-    const Geo g = shape_geo(h, n, prec_index<T>(), 1, (unsigned char)(shape & 2));
     if (shape & 1)
-        WITH_COLS(lv.S, (launch_k(h->pdl, k_prolong_post<T, IDX, kUnrollSmall>, g.grid, g.block, s, n, lv.S.sptr,
+        WITH_COLS(lv.S, (launch_shaped(h, k_prolong_post<T, IDX, kUnrollSmall>, n, shape, kBlock, s, n, lv.S.sptr,
                                   cols, P::val(lv), (const T *)P::xpre(lv), P::p(lv), lv.agg,
                                   (const T *)P::x(lev[l + 1]), (const T *)P::b(lv), P::dinv(lv), P::x(lv), ctl)));
     else
-        WITH_COLS(lv.S, (launch_k(h->pdl, k_prolong_post<T, IDX, kUnroll>, g.grid, g.block, s, n, lv.S.sptr, cols,
+        WITH_COLS(lv.S, (launch_shaped(h, k_prolong_post<T, IDX, kUnroll>, n, shape, kBlock, s, n, lv.S.sptr, cols,
                                   P::val(lv), (const T *)P::xpre(lv), P::p(lv), lv.agg, (const T *)P::x(lev[l + 1]),
                                   (const T *)P::b(lv), P::dinv(lv), P::x(lv), ctl)));
     return false;
@@ -1699,14 +1701,14 @@ void launch_down0_t(amg_hier *h, const T *b0, cudaStream_t s) {
     Level &l0 = h->lev[0];
     const double *pc = parts(h, kPartsRr);
     if (down_fused(h, 0, prec_index<T>())) {
-        const int blk = std::min(h->block0, small_block(l0.mpos));
-        const Geo g{(l0.mpos + blk - 1) / blk, blk};
+        const int blk = std::min(h->block0, small_block(h, l0.mpos));
+        constexpr unsigned char shape = 2;
         T *bc = P::b(h->lev[1]);
         const bool direct = direct_level(h) == 1, whole = l0.A.n <= whole_rows(h);
-        if (direct && whole) launch_down_r<T, double, kWholeRow, false, STEP>(h, 0, b0, h->bL, false, g, s);
-        else if (direct) launch_down_r<T, double, kUnrollSmall, false, STEP>(h, 0, b0, h->bL, false, g, s);
-        else if (whole) launch_down_r<T, T, kWholeRow, false, STEP>(h, 0, b0, bc, true, g, s);
-        else launch_down_r<T, T, kUnrollSmall, false, STEP>(h, 0, b0, bc, true, g, s);
+        if (direct && whole) launch_down_r<T, double, kWholeRow, false, STEP>(h, 0, b0, h->bL, false, shape, blk, s);
+        else if (direct) launch_down_r<T, double, kUnrollSmall, false, STEP>(h, 0, b0, h->bL, false, shape, blk, s);
+        else if (whole) launch_down_r<T, T, kWholeRow, false, STEP>(h, 0, b0, bc, true, shape, blk, s);
+        else launch_down_r<T, T, kUnrollSmall, false, STEP>(h, 0, b0, bc, true, shape, blk, s);
         return;
     }
     if constexpr (sizeof(T) == 4) {
@@ -2223,6 +2225,7 @@ int alloc_solve_workspace(amg_hier *h) {
     PCG_CK(cudaGetDevice(&dev));
     PCG_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     h->device = dev;
+    h->sms = sms;
     // One wave of resident blocks per level-0 kernel family (grid = SMs x
     // blocks resident per SM), capped by the rows available.
     // A mesh of less than a full block per SM takes smaller blocks, one per SM.
@@ -2262,23 +2265,7 @@ int alloc_solve_workspace(amg_hier *h) {
     h->blockv = (h->blockv + 31) / 32 * 32;
     h->gridv = std::min(vec_blocks, (n + h->blockv - 1) / h->blockv);
     h->nblk = std::max(h->grid32, std::max(h->grid64, h->gridv));
-    // One wave of each coarse-level sweep variant, and the fixed shape rule.
-    const void *fns[2][2][2] = {
-        {{(const void *)k_down_r<float, float, int16_t, kUnroll, false, false>,
-          (const void *)k_down_r<float, float, int16_t, kUnrollSmall, false, false>},
-         {(const void *)k_post<float, float, false, false, int16_t, kUnroll, false, true>,
-          (const void *)k_post<float, float, false, false, int16_t, kUnrollSmall, false, true>}},
-        {{(const void *)k_down_r<double, double, int16_t, kUnroll, false, false>,
-          (const void *)k_down_r<double, double, int16_t, kUnrollSmall, false, false>},
-         {(const void *)k_post<double, double, false, false, int16_t, kUnroll, false, true>,
-          (const void *)k_post<double, double, false, false, int16_t, kUnrollSmall, false, true>}}};
-    for (int a = 0; a < 2; a++)
-        for (int b = 0; b < 2; b++)
-            for (int c = 0; c < 2; c++) {
-                int per = 0;
-                PCG_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fns[a][b][c], kBlock, 0));
-                h->wave[a][b][c] = sms * (per > 0 ? per : 1);
-            }
+    // the coarse levels' fixed shape rule
     for (size_t l = 1; l < h->lev.size(); l++) {
         unsigned char d = (unsigned char)((h->lev[l].A.n <= kSmallRows ? 1 : 0) | 2);
         h->lev[l].rule_shape = d;
