@@ -834,6 +834,15 @@ __global__ void __launch_bounds__(kC1) k_cx1(int n, int nb, const double *__rest
 #pragma unroll
         for (int k = 0; k < 8; k++) t = fma(m[k], __shfl_sync(0xffffffffu, rn, 8 * w + k), t);
         zp[w][lane] = t;
+        // the next block's loads, in flight over the barriers (27,896 rows, three
+        // blocks of rows each: 160^3 float64 97.3 -> 95.6 ms a solve)
+        const double qb = qi;
+        b += gridDim.x;
+        inverse(b);
+        if (b < nb) {
+            qi = q[b * kB + lane];
+            ri = r[b * kB + lane];
+        }
         if (w == 1) {
             const double xi = fma(alpha, p[i], x[i]);
             x[i] = xi;
@@ -846,15 +855,9 @@ __global__ void __launch_bounds__(kC1) k_cx1(int n, int nb, const double *__rest
             r[i] = rn;
             acc[0] += rn * rn;
             acc[1] += rn * zv;
-            acc[2] += zv * qi;
+            acc[2] += zv * qb;
         }
         __syncthreads();
-        b += gridDim.x;
-        if (b < nb) {
-            inverse(b);
-            qi = q[b * kB + lane];
-            ri = r[b * kB + lane];
-        }
     }
     block_sum<3>(acc, 1);
     if (threadIdx.x == 0) {
@@ -982,7 +985,9 @@ int cws_alloc(amg_hier *h, Mem &M, CoarseWS &W, int K) {
     W.grid_q = grid_for_items(h, nb * 4 * (K / KC), K / KC);
     if (K == 1) {
         // one block of four warps per 32-row block, and so many at most that a
-        // block sums their partials in three or four loads a thread
+        // block sums their partials in three or four loads a thread (27,896
+        // rows: four and six per SM 103.9 ms a 160^3 float64 solve for 97.3, one
+        // and three 100.8, one of each 102.0)
         int sms = 0;
         PCG_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
         W.grid = nb < 2 * sms ? nb : 2 * sms;
