@@ -1363,11 +1363,14 @@ constexpr int kWholeRows = 32768;
 // A solve that shares the device (batches, serving lanes: no_tail) is short of
 // registers and float64 cycles rather than waiting for latency: twelve systems
 // of 24^3 to 72^3 at once ran 14.2 ms with the limits of a lone solve, 13.1
-// with 1,024 and 16,384 rows (the bits are the same); 48 of 24^3 to 112^3 199.5
-// ms (268.8 in float64) with 16,384 rows fused, 198.7 (266.5) with 4,096,
-// where the twelve take 12.6 ms either way.
+// with 1,024 and 16,384 rows (the bits are the same). In float64 the large
+// systems' coarse levels lose by fusing: 48 of 24^3 to 112^3 266.3 ms with
+// 16,384 rows, 263.7 with 4,096, where five small ones lose without it (24^3 to
+// 41^3 2.47 ms, 2.51), so the lower limit holds for systems above 131,072 rows
+// (264.6 and 2.48). In float32 twelve systems take 12.42 ms with 16,384 rows
+// and 12.52 with 4,096, the 48 196.9 and 196.1.
 constexpr int kWholeRowsShared = 1024;
-constexpr int kFuseRowsShared = 4096;
+constexpr int kFuseRowsShared = 16384, kFuseRowsLarge64 = 4096, kLargeRows64 = 131072;
 int whole_rows(const amg_hier *h) { return h->no_tail ? kWholeRowsShared : kWholeRows; }
 
 // A coarse-level sweep over n rows (or positions) in a launch shape: a thread
@@ -1396,12 +1399,13 @@ unsigned char shape_of(const amg_hier *h, int l, int pi, int phase) {
 // Whether level l's down sweep can restrict in the same launch (member order),
 // and whether it does: on l >= 1 only with a down shape that is not one of the
 // older forms.
-bool fusable(const amg_hier *h, int l) {
+bool fusable(const amg_hier *h, int l, int pi) {
     const Level &lv = h->lev[l];
-    return h->fuse && lv.mslot > 0 && !h->smoothed && !h->gs_nu && !(h->no_tail && lv.A.n > kFuseRowsShared);
+    const int shared = pi == 1 && h->lev[0].A.n > kLargeRows64 ? kFuseRowsLarge64 : kFuseRowsShared;
+    return h->fuse && lv.mslot > 0 && !h->smoothed && !h->gs_nu && !(h->no_tail && lv.A.n > shared);
 }
 bool down_fused(const amg_hier *h, int l, int pi) {
-    return fusable(h, l) && (l == 0 || !(shape_of(h, l, pi, 0) & 12));
+    return fusable(h, l, pi) && (l == 0 || !(shape_of(h, l, pi, 0) & 12));
 }
 
 // Weight of the down sweep's output t = w (b - A xpre): the tentative
@@ -2323,7 +2327,7 @@ void run_phase(amg_hier *h, int l, int sweep, cudaStream_t s) {
     int kernels = 0;
     if (sweep == 0) {
         launch_down_phase<T>(h, l, sh[0], s, &kernels);
-        if (!ready && fusable(h, l) && below_prolongs<T>(h, l) && !(sh[1] & 4)) {
+        if (!ready && fusable(h, l, pi) && below_prolongs<T>(h, l) && !(sh[1] & 4)) {
             launch_prolong<T>(h, l, grid_rows(h->lev[l].A.n), s);
             kernels += 1;
         }
