@@ -23,9 +23,11 @@ constexpr int kOpThreads = 256;
 // pipe (n^2 FMAs at 304 a clock: 1,036 rows 1.7 us), two more sweeps and a
 // smaller matrix by latency (about 2 us each). Alone, 400 rows instead cost
 // 812 us per 24^3 solve (834-row level, 727 with it), 1,536 and 2,600 rows the
-// same there, but 128^3 22.9 ms with 2,600 (22.0); twelve systems at once,
-// which share the pipe, ran 12.7 ms with 900 and 13.2 with 1,536; 41^3 float64
-// (a level between 1,100 and 1,280 rows) 2,412 us without it, 2,140 with it.
+// same there, but 128^3 22.9 ms with 2,600 (22.0); 41^3 float64 (a level between
+// 1,100 and 1,280 rows) 2,412 us without it, 2,230 with it. Systems that share
+// the pipe would rather have less: twelve at once 12.6 ms with 1,280, 12.5 with
+// 900 and 13.2 with 1,536, 48 of 24^3 to 112^3 198.7 and 196.6 with 900, where
+// the same 48 one by one take 272 either way (277 with 600, 282 with 300).
 constexpr int kOpRows = 1280;
 
 // One level's step, for column j (blockIdx.x) of B: x = S e_j + correction,

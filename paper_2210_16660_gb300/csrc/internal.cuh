@@ -350,7 +350,7 @@ struct amg_hier {
     int nblk = 0;                // largest level-0 grid (sizes the partial sums)
     int grid32 = 0, grid64 = 0, gridp = 0;  // one wave of the float32 sweeps, float64 sweeps, prolongation
     int block0 = 0;                         // threads per block of the level-0 matrix kernels
-    int gridv = 0, blockv = 0;              // vector kernels
+    int gridv = 0, blockv = 0, vec_per_sm = 2;  // vector kernels
     int sms = 0;                 // multiprocessors of the device
     double last_true_rel = 0.0;
     double setup_ms[4] = {0, 0, 0, 0};

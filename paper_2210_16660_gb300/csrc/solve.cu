@@ -1064,9 +1064,12 @@ __device__ __forceinline__ void emit_r(int i, double ri, const REmit &e) {
 // alpha = rho / p.q from the partial sums of k_spmv, then x += alpha p,
 // r -= alpha q and the partial sums of ||r||^2; one thread advances the
 // iteration. The first row's vectors and the scalars are requested before the
-// partials are summed.
-template <int MODE>
-__global__ void __launch_bounds__(kVecBlock) k_update(int n, const double *__restrict__ p,
+// partials are summed. BOUND: the compiler's block size. At 512 it takes 40
+// registers, so that three blocks of 512 fit an SM (at 44 two do: 48 systems at
+// once 198.7 ms, 196.4); at 1,024 it takes 44 and asks for the small meshes' rows
+// earlier (32^3 mixed 917 us, 901).
+template <int MODE, int BOUND>
+__global__ void __launch_bounds__(BOUND) k_update(int n, const double *__restrict__ p,
                                                       const double *__restrict__ q, double *__restrict__ x,
                                                       double *__restrict__ r, REmit em, const double *pb, int gb,
                                                       double *partials, Ctl *ctl) {
@@ -2034,8 +2037,12 @@ int launch_iteration_t(amg_hier *h, bool first, bool last, const Cond &cond, cud
                                   pats, h->p, h->q, parts(h, kPartsPq), h->ctl)));
     prof_end(h, sp5, s);
     int sp6 = prof_begin(h, 3, s);
-    launch_k(pdl, k_update<MODE>, h->gridv, h->blockv, s, n, h->p, h->q, h->x, h->r, remit(h), parts(h, kPartsPq),
-             h->grid64, parts(h, kPartsRr), h->ctl);
+    if (h->vec_per_sm == 2)
+        launch_k(pdl, k_update<MODE, 2 * kVecBlock>, h->gridv, h->blockv, s, n, h->p, h->q, h->x, h->r, remit(h),
+                 parts(h, kPartsPq), h->grid64, parts(h, kPartsRr), h->ctl);
+    else
+        launch_k(pdl, k_update<MODE, kVecBlock>, h->gridv, h->blockv, s, n, h->p, h->q, h->x, h->r, remit(h),
+                 parts(h, kPartsPq), h->grid64, parts(h, kPartsRr), h->ctl);
     prof_end(h, sp6, s);
     h->launches += 3;
     if (last || !takes) {
@@ -2264,7 +2271,8 @@ int alloc_solve_workspace(amg_hier *h) {
     // (64^3 warm 2,155 and 2,136). Blocks of 1,024 threads, two per SM, waited
     // for half an SM to fall free where systems share the device: 48 of 24^3 to
     // 112^3 at once 203.8 ms (196.1 with three blocks of 512).
-    const int vec_blocks = (n <= 2 * sms * kVecBlock ? 2 : 3) * sms;
+    h->vec_per_sm = n <= 2 * sms * kVecBlock ? 2 : 3;
+    const int vec_blocks = h->vec_per_sm * sms;
     h->blockv = (int)std::min<int64_t>(kVecBlock, std::max<int64_t>(128, ((int64_t)n + vec_blocks - 1) / vec_blocks));
     h->blockv = (h->blockv + 31) / 32 * 32;
     h->gridv = std::min(vec_blocks, (n + h->blockv - 1) / h->blockv);
