@@ -54,8 +54,8 @@ def test_fused_transfers_give_the_bits_of_separate_launches(N, npass, cmax, env,
     assert np.array_equal(r1.hist, r2.hist) and torch.equal(x1, x2)
 
 
-class _Bytes:
-    """An allocator that counts the library's bytes (rounded by it already)."""
+class Bytes:
+    """An allocator that counts the library's bytes and refuses past `limit`."""
 
     def __enter__(self):
         self.live, self.now, self.peak, self.limit = {}, 0, 0, None
@@ -92,7 +92,7 @@ def test_member_order_is_left_out_of_a_budget_without_room(N, npass):
     prob = W.make_problem(N, 1.04, seed=3)
     b = torch.from_numpy(prob.b).cuda()
     env = (("PCGAMG_COL16", "0"), ("PCGAMG_TAIL", "0"))
-    with _Bytes() as mem:
+    with Bytes() as mem:
         a1 = _amg(prob.A, env, n_pass=npass)
         rows = [n for n, _ in a1.info()]
         extra = 0

@@ -7,8 +7,6 @@ matrices; kept aggregates), and solves meet the oracle's bar (iterations
 are updated in place, so graphs captured before the refresh (whole-solve,
 batch) must give the same bits as a handle refreshed before its first solve.
 """
-import ctypes as C
-
 import numpy as np
 import pytest
 
@@ -19,6 +17,7 @@ torch = pytest.importorskip("torch")
 import oracle as O  # noqa: E402
 from paper_2210_16660_gb300 import binding as B  # noqa: E402
 from paper_2210_16660_gb300 import workloads as W  # noqa: E402
+from test_gpu_fused import Bytes  # noqa: E402
 from test_gpu_parity import direct_level  # noqa: E402
 
 RTOL = 1e-8
@@ -172,33 +171,6 @@ def test_refresh_rejections_leave_the_handle_unchanged():
     assert torch.equal(x0, x1)
 
 
-class _Bytes:
-    """An allocator that counts the library's bytes and refuses past `limit`."""
-
-    def __enter__(self):
-        self.live, self.now, self.peak, self.limit = {}, 0, 0, None
-
-        def alloc(n, stream, ctx):
-            if self.limit is not None and self.now + n > self.limit:
-                return None
-            p = torch.cuda.caching_allocator_alloc(int(n), torch.cuda.current_device(), stream or 0)
-            self.live[p] = n
-            self.now += n
-            self.peak = max(self.peak, self.now)
-            return p
-
-        def free(p, stream, ctx):
-            self.now -= self.live.pop(p)
-            torch.cuda.caching_allocator_delete(p)
-
-        self.refs = (B.ALLOC_FN(alloc), B.FREE_FN(free))
-        assert B.load().amg_set_allocator(C.cast(self.refs[0], C.c_void_p), C.cast(self.refs[1], C.c_void_p), None) == 0
-        return self
-
-    def __exit__(self, *a):
-        B.load().amg_set_allocator(None, None, None)
-
-
 def _scattered(n, deg, seed):
     """A graph Laplacian plus the identity with `deg` far-flung neighbours a row:
     two rows share hardly a column, so a coarse matrix keeps most entries."""
@@ -225,7 +197,7 @@ def test_refresh_where_only_single_temporaries_fit():
     A2 = W.rescaled(A, seed=2)
     b = torch.from_numpy(W.spmv(A2, W.normals(3, A.n))).cuda()
     kw = dict(max_levels=2, coarse_max=10)
-    with _Bytes() as mem:
+    with Bytes() as mem:
         a1 = B.AMG.from_csr(A, hbm_budget=1 << 40, **kw)      # a budget: single allocations
         start = mem.peak = mem.now
         a1.refresh(A2)
